@@ -79,7 +79,10 @@ typedef enum {
 
 /* Propagation variants of rt_reconstruct; all give identical output. */
 enum {
-    RT_AUTO = 0,    /* library choice (RT_RASTER) */
+    RT_AUTO = 0,    /* library choice: with 8-connectivity the contraction of the image to the
+                       clusters that matter for widest paths (csrc/contract.cu), which makes no
+                       tile visits; RT_RASTER for 4-connectivity and where the call bounds the
+                       propagation's visits or time, or sets its visit budget or strip length */
     RT_RASTER = 1,  /* directional sweeps of 32 x 64 tiles, revisiting flagged tiles */
     RT_QUEUE = 2,   /* per-tile pixel FIFOs (irregular wavefront propagation) */
     RT_HYBRID = 3,  /* one sweep visit of every tile, then pixel FIFOs for what remains */
@@ -225,7 +228,7 @@ enum {
  * rt_kernel_launches returns how many kernels the context has launched.
  * rt_recon_stats waits for the device and reports how many tile visits,
  * dense sweep iterations and queue pops the last reconstruction made
- * (statistics; 0 if none); any pointer may be NULL.
+ * (statistics; 0 if none, as after a contraction); any pointer may be NULL.
  */
 RT_API rt_status rt_timing_enable(rt_ctx *ctx, int enable);
 RT_API rt_status rt_timing_read(rt_ctx *ctx, double *ms, int64_t *count, int reset);
@@ -336,7 +339,10 @@ RT_API rt_status rt_synth_tile(rt_ctx *ctx, uint8_t *out, int64_t ld, int H, int
  * iterations: short visits win on small tiles, longer ones on large tiles).
  * The budgets are learned on lone tiles; in a chunk of several tiles the
  * shared launch's throughput sets the time, and raster budgets below the
- * call's plain one are raised to it.
+ * call's plain one are raised to it. Where the call's plain schedule is the
+ * contraction (RT_AUTO), which is faster than every raster budget, tiles
+ * with a raster class run it too: the picks of a lone tile are then computed
+ * beside the chain and reported, and change no schedule.
  *
  * rt_tile_features: features of n tiles (host arrays of device pointers,
  * strides and sizes; n <= 32) into out, a device float array n x

@@ -8,6 +8,7 @@
 
 #include "ccl.cuh"
 #include "common.cuh"
+#include "contract.cuh"
 #include "edt.cuh"
 #include "features.cuh"
 #include "fill.cuh"
@@ -37,6 +38,8 @@ struct rt_ctx {
     int32_t *picks_mapped = nullptr;       // the same memory as the device sees it
     cudaEvent_t picks_ev = nullptr;        // recorded after their copy (not under stream capture)
     bool picks_ev_valid = false;
+    cudaStream_t side = nullptr;           // the picker's stream where its picks change no schedule
+    cudaEvent_t fork = nullptr, join = nullptr;   // order it behind the call's start and before its end
     int n_last_picks = 0;
     PickTable classes{{0, 0, 0, 0}, {4, 12, 24, 12}};   // picker classes (rt_set_picker_classes); entry 3 per call
     int max_iters = 0;                     // limits of the single-operation entry points (rt_set_limits)
@@ -144,6 +147,15 @@ bool overlaps(const void *a, size_t na, const void *b, size_t nb)
     return pa < pb + nb && pb < pa + na;
 }
 
+// Releases the context's events, side stream and pinned buffer.
+void free_host_side(rt_ctx *c)
+{
+    if (c->side) cudaStreamDestroy(c->side);
+    for (cudaEvent_t e : {c->picks_ev, c->fork, c->join})
+        if (e) cudaEventDestroy(e);
+    if (c->picks_host) cudaFreeHost(c->picks_host);
+}
+
 size_t span(int H, int64_t ld, size_t elem, int W) { return ((size_t)(H - 1) * ld + W) * elem; }
 
 rt_status cuda_status(cudaError_t e)
@@ -233,10 +245,27 @@ struct Limits {
 
 Limits ctx_limits(const rt_ctx *ctx) { return {ctx->max_iters, ctx->timeout_ns ? ctx->timeout_ns : kSweepTimeoutNs}; }
 
+Limits seg_limits(const rt_ctx *ctx, const rt_seg_params &P)
+{
+    Limits lim = ctx ? ctx_limits(ctx) : Limits{0, kSweepTimeoutNs};
+    if (P.max_iters > 0) lim.max_iters = P.max_iters;
+    if (P.timeout_ms > 0) lim.timeout_ns = (uint64_t)P.timeout_ms * 1000000ull;
+    lim.strip = P.strip_tiles;
+    return lim;
+}
+
 int default_max_local(int variant) { return variant == RT_HYBRID || variant == RT_FRONTIER ? 64 : 12; }
 
 // sweep budget of every raster tile in a launch shared by several tiles
 int shared_raster_budget(int max_local) { return max_local > 0 ? max_local : default_max_local(RT_RASTER); }
+
+// Whether every class of the picker propagates by RT_RASTER.
+bool raster_classes(const rt_ctx *ctx)
+{
+    for (int c = 0; ctx && c < kPickClasses; ++c)
+        if (ctx->classes.group[c] != 0) return false;
+    return true;
+}
 
 // In a launch shared by several tiles every raster class runs at the plain
 // budget, so when the plain schedule and every class of the picker are
@@ -245,9 +274,7 @@ bool picks_matter(const rt_ctx *ctx, const rt_seg_params &P, int n_tiles)
 {
     if (n_tiles == 1) return true;
     if (P.variant != RT_AUTO && P.variant != RT_RASTER) return true;
-    for (int c = 0; c < kPickClasses; ++c)
-        if (ctx->classes.group[c] != 0) return true;
-    return false;
+    return !raster_classes(ctx);
 }
 
 rt_status run_recon(rt_ctx *ctx, ReconBatch &b, ReconWs &w, int conn, int variant, int max_local, int32_t *err,
@@ -344,6 +371,43 @@ rt_status run_recon(rt_ctx *ctx, ReconBatch &b, ReconWs &w, int conn, int varian
     return RT_OK;
 }
 
+// ------------------------------------------------------------ contraction
+// RT_AUTO with 8-connectivity runs the reconstruction by contraction, unless
+// the call sets something that only the propagation has: a bound on its tile
+// visits or its device time, a visit budget, a strip length.
+bool use_contraction(int conn, int variant, int max_local, int strip, const Limits &lim)
+{
+    return conn == 8 && variant == RT_AUTO && max_local == 0 && strip == 0 && lim.max_iters == 0 &&
+           lim.timeout_ns == kSweepTimeoutNs;
+}
+
+void carve_contract(Carve &cv, CtBatch &b)
+{
+    const size_t nt = (size_t)b.ntiles;
+    b.ctl = cv.take<uint32_t>(kCtCtlWords);
+    b.plane = cv.take<uint16_t>(nt * kCtPx);
+    b.cnt = cv.take<uint32_t>(nt);
+    b.S = cv.take<uint32_t>(nt * kCtNodes);
+    b.link = cv.take<unsigned long long>(nt * kCtNodes);
+    b.best = cv.take<unsigned long long>(nt * kCtNodes);
+    b.act = cv.take<uint32_t>(nt * kCtNodes);
+    b.ea = cv.take<uint32_t>(nt * kCtEdges);
+    b.eb = cv.take<uint32_t>(nt * kCtEdges);
+    b.ew = cv.take<uint8_t>(nt * kCtEdges);
+}
+
+// Enqueue the contraction of a carved batch; launch_contract_out writes R.
+rt_status run_contract(rt_ctx *ctx, CtBatch &b, int32_t *err, cudaStream_t s, const Limits &lim)
+{
+    b.err = err;
+    ctx->visits_dev = nullptr;   // no tile visits
+    RT_CUDA_TRY(zero_words(b.ctl, kCtCtlWords, s));
+    Phase ph(ctx, RT_PHASE_RECON_SWEEP, s);
+    RT_CUDA_TRY(launch_contract(b, ctx->num_sms, lim.timeout_ns, s));
+    ctx->launches += 3;
+    return RT_OK;
+}
+
 void add_image(ReconBatch &b, const uint8_t *marker, int64_t ld_marker, const uint8_t *mask, int64_t ld_mask,
                int H, int W, int h_offset)
 {
@@ -407,8 +471,11 @@ bool bad_tile(const rt_tile &t)
 // union-find arrays, the kept-pixel bit plane and the distance transform's
 // column masks.
 struct Chunk {
+    bool contract = false;   // reconstruction by contraction (cb), else by propagation (b, w)
+    CtBatch cb;
     ReconBatch b;
     ReconWs w;
+    int32_t *err = nullptr;
     FeatBatch fb;
     float *feat = nullptr;
     int32_t *picks = nullptr;
@@ -421,16 +488,26 @@ struct Chunk {
 // Lays chunk [c0, c0 + cn) out in cv. With cv.base == nullptr only the size
 // is measured (cv.off); no pointer is formed.
 void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, const rt_seg_params &P, bool learned,
-                  const rt_ctx *ctx)
+                  const rt_ctx *ctx, const Limits &lim, bool may_contract = true)
 {
     const bool real = cv.base != nullptr;
-    std::memset(&c.b, 0, sizeof(c.b));
+    c.err = cv.take<int32_t>(1);
+    c.cb.n = c.cb.ntiles = 0;
     for (int i = 0; i < cn; ++i) {
         const rt_tile &t = tiles[c0 + i];
-        add_image(c.b, nullptr, 0, t.img, t.ld_img, t.H, t.W, P.h_offset);
+        ct_plan_image(c.cb, nullptr, 0, t.img, t.ld_img, t.H, t.W, P.h_offset);
     }
-    carve_recon(cv, c.b, c.w, learned,
-                uses_frontier(ctx, P.variant, learned) ? frontier_capacity(ctx, c.b) : 0u);
+    c.contract = may_contract && use_contraction(P.conn_recon, P.variant, P.max_local, P.strip_tiles, lim) &&
+                 c.cb.ntiles < kCtMaxTiles && (!learned || raster_classes(ctx));
+    if (!c.contract) {
+        std::memset(&c.b, 0, sizeof(c.b));
+        for (int i = 0; i < cn; ++i) {
+            const rt_tile &t = tiles[c0 + i];
+            add_image(c.b, nullptr, 0, t.img, t.ld_img, t.H, t.W, P.h_offset);
+        }
+        carve_recon(cv, c.b, c.w, learned,
+                    uses_frontier(ctx, P.variant, learned) ? frontier_capacity(ctx, c.b) : 0u);
+    }
     if (learned) {
         c.fb.n = cn;
         for (int i = 0; i < cn; ++i) {
@@ -456,18 +533,36 @@ void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, con
     for (int i = 0; i < cn; ++i) {
         const rt_tile &t = tiles[c0 + i];
         const int H = t.H, W = t.W;
-        ReconImage &d = c.b.img[i];
         // B = (R < threshold); F replaces it in place unless the caller wants F
         uint8_t *B = cv.take<uint8_t>((size_t)H * W);
-        d.out = t.recon;
-        d.ld_out = t.ld_recon;
-        d.bin = B;
-        d.ld_bin = W;
+        auto outputs = [&](auto &d) {
+            d.out = t.recon;
+            d.ld_out = t.ld_recon;
+            d.bin = B;
+            d.ld_bin = W;
+        };
+        if (c.contract) outputs(c.cb.img[i]);
+        else outputs(c.b.img[i]);
         uint8_t *F = t.filled ? t.filled : B;
         const int64_t ldF = t.filled ? t.ld_filled : W;
         char *fws = cv.take<char>(fill_image_bytes(H, W));
         if (real) fill_add(c.fill, B, W, F, ldF, H, W, fws);
         fill_tiles += (int)(ceil_div(H, kFillTH) * ceil_div(W, kFillTW));
+    }
+    c.fill_flags = cv.take<uint32_t>((size_t)fill_tiles);
+    c.fill_pending = cv.take<uint32_t>(1);
+    // The contraction's arrays are dead once R and B are written; the stages
+    // from the labeling on reuse their memory.
+    size_t contract_end = 0;
+    if (c.contract) {
+        const size_t off = cv.off;
+        carve_contract(cv, c.cb);
+        contract_end = cv.off;
+        cv.off = off;
+    }
+    for (int i = 0; i < cn; ++i) {
+        const rt_tile &t = tiles[c0 + i];
+        const int H = t.H, W = t.W;
         char *uws = cv.take<char>(uf_workspace_bytes(H, W));
         uint32_t *kept = cv.take<uint32_t>((size_t)H * ceil_div(W, 32));
         char *ews = cv.take<char>(edt_bits_workspace_bytes(H, W));
@@ -475,8 +570,8 @@ void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, con
             UfImage u;
             std::memset(&u, 0, sizeof(u));
             uf_carve(u, uws, H, W);
-            u.in = F;
-            u.ld_in = ldF;
+            u.in = c.fill.img[i].out;
+            u.ld_in = c.fill.img[i].ld_out;
             u.labels = t.labels;
             u.ld_lab = t.ld_labels;
             u.n_kept = t.n_kept;
@@ -485,22 +580,54 @@ void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, con
             edt_bits_add(c.eb, kept, H, W, t.d2, t.ld_d2, ews);
         }
     }
-    c.fill_flags = cv.take<uint32_t>((size_t)fill_tiles);
-    c.fill_pending = cv.take<uint32_t>(1);
+    if (cv.off < contract_end) cv.off = contract_end;
     c.uf.amin = P.min_area;
     c.uf.amax = P.max_area;
+}
+
+// The picker's features and network on a chunk, into its picks.
+rt_status run_picker(rt_ctx *ctx, const Chunk &c, const rt_seg_params &P, cudaStream_t s)
+{
+    Phase ph(ctx, RT_PHASE_PICK, s);
+    RT_CUDA_TRY(launch_features_pick(c.fb, c.feat, ctx->picker_wb, ctx->picker_norm, c.picks,
+                                     (float)P.pick_min_prob / 1000.0f, kPickClasses, s));
+    ctx->launches += 4;
+    return RT_OK;
+}
+
+// The chunk's picks for rt_last_picks (NULL: every tile ran the plain
+// schedule), written by a kernel into the mapped pinned buffer: a copy-engine
+// transfer would queue behind the caller's read-backs on the same engine and
+// hold up the rest of the chain.
+rt_status report_picks(rt_ctx *ctx, const int32_t *picks, int cn, cudaStream_t s)
+{
+    copy_picks_kernel<<<1, 32, 0, s>>>(picks, ctx->picks_mapped, cn);
+    RT_CUDA_TRY(cudaGetLastError());
+    ctx->launches += 1;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    ctx->picks_ev_valid = cap == cudaStreamCaptureStatusNone;
+    if (ctx->picks_ev_valid) RT_CUDA_TRY(cudaEventRecord(ctx->picks_ev, s));
+    ctx->n_last_picks = cn;
+    return RT_OK;
 }
 
 // Workspace bytes rt_segment_batch needs for these tiles (the largest chunk).
 size_t segment_ws_bytes(const rt_tile *tiles, int n, const rt_seg_params &P, bool learned, const rt_ctx *ctx)
 {
+    const Limits lim = seg_limits(ctx, P);
     size_t most = 0;
     for (int c0 = 0; c0 < n; c0 += kMaxImgs) {
         const int cn = n - c0 < kMaxImgs ? n - c0 : kMaxImgs;
-        Carve cv;
-        Chunk c;
-        layout_chunk(cv, c, tiles, c0, cn, P, learned, ctx);
-        most = cv.off > most ? cv.off : most;
+        // A call that contracts fits where the same call with a bound on its
+        // propagation fits: a reservation serves both.
+        for (bool may_contract : {true, false}) {
+            Carve cv;
+            Chunk c;
+            layout_chunk(cv, c, tiles, c0, cn, P, learned, ctx, lim, may_contract);
+            most = cv.off > most ? cv.off : most;
+            if (!c.contract) break;
+        }
     }
     return most;
 }
@@ -544,15 +671,17 @@ rt_status rt_create(rt_ctx **ctx, int device, size_t workspace_bytes)
     if (cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         cudaHostAlloc((void **)&c->picks_host, kMaxImgs * sizeof(int32_t), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer((void **)&c->picks_mapped, c->picks_host, 0) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->picks_ev, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&c->picks_ev, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
-        if (c->picks_host) cudaFreeHost(c->picks_host);
+        free_host_side(c);
         delete c;
         return RT_ECUDA;
     }
     if (workspace_bytes > 0 && ensure_ws(c, workspace_bytes) != RT_OK) {
-        cudaEventDestroy(c->picks_ev);
-        cudaFreeHost(c->picks_host);
+        free_host_side(c);
         delete c;
         return RT_ENOMEM;
     }
@@ -596,8 +725,7 @@ void rt_destroy(rt_ctx *ctx)
         cudaEventDestroy(r.b);
     }
     for (cudaEvent_t e : ctx->pool) cudaEventDestroy(e);
-    if (ctx->picks_ev) cudaEventDestroy(ctx->picks_ev);
-    if (ctx->picks_host) cudaFreeHost(ctx->picks_host);
+    free_host_side(ctx);
     delete ctx;
 }
 
@@ -687,6 +815,30 @@ rt_status rt_reconstruct(rt_ctx *ctx, const uint8_t *marker, int64_t ld_marker, 
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
 
+    const Limits lim = ctx_limits(ctx);
+    if (use_contraction(conn, variant, 0, 0, lim)) {
+        CtBatch cb;
+        cb.n = cb.ntiles = 0;
+        ct_plan_image(cb, marker, ld_marker, mask, ld_mask, H, W, h_offset);
+        cb.img[0].out = out;
+        cb.img[0].ld_out = ld_out;
+        int32_t *cerr = nullptr;
+        rt_status cst = RT_OK;
+        for (int pass = 0; pass < 2; ++pass) {   // size, then carve
+            Carve cc;
+            if (pass) cc.base = (char *)ctx->ws;
+            cerr = cc.take<int32_t>(1);
+            carve_contract(cc, cb);
+            if (!pass && (cst = ensure_ws(ctx, cc.off)) != RT_OK) return cst;
+        }
+        if (dev_status) cerr = dev_status;
+        RT_CUDA_TRY(cudaMemsetAsync(cerr, 0, sizeof(int32_t), s));
+        cst = run_contract(ctx, cb, cerr, s, lim);
+        if (cst != RT_OK) return cst;
+        Phase ph(ctx, RT_PHASE_RECON_OUT, s);
+        ctx->launches += 1;
+        return cuda_status(launch_contract_out(cb, 0, s));
+    }
     ReconBatch b;
     std::memset(&b, 0, sizeof(b));
     add_image(b, marker, ld_marker, mask, ld_mask, H, W, h_offset);
@@ -702,7 +854,7 @@ rt_status rt_reconstruct(rt_ctx *ctx, const uint8_t *marker, int64_t ld_marker, 
 
     int32_t *err = dev_status ? dev_status : w.err;
     RT_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int32_t), s));
-    st = run_recon(ctx, b, w, conn, variant, 0, err, s, ctx_limits(ctx));
+    st = run_recon(ctx, b, w, conn, variant, 0, err, s, lim);
     if (st != RT_OK) return st;
     b.img[0].out = out;
     b.img[0].ld_out = ld_out;
@@ -1072,10 +1224,7 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
     const bool learned = P.policy == RT_POLICY_LEARNED && ctx->picker_wb && ctx->picker_norm;
-    Limits lim = ctx_limits(ctx);
-    if (P.max_iters > 0) lim.max_iters = P.max_iters;
-    if (P.timeout_ms > 0) lim.timeout_ns = (uint64_t)P.timeout_ms * 1000000ull;
-    lim.strip = P.strip_tiles;
+    const Limits lim = seg_limits(ctx, P);
     // one allocation for the largest chunk, before anything is enqueued
     rt_status st = ensure_ws(ctx, segment_ws_bytes(tiles, n, P, learned, ctx));
     if (st != RT_OK) return st;
@@ -1085,47 +1234,50 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
         Chunk c;
         Carve cv;
         cv.base = (char *)ctx->ws;
-        layout_chunk(cv, c, tiles, c0, cn, P, learned, ctx);
-        RT_CUDA_TRY(zero_words(c.w.err, 1, s));
+        layout_chunk(cv, c, tiles, c0, cn, P, learned, ctx, lim);
+        RT_CUDA_TRY(zero_words(c.err, 1, s));
         ctx->launches += 1;
+        auto reconstruct = [&](const int32_t *pick) {
+            return c.contract ? run_contract(ctx, c.cb, c.err, s, lim)
+                              : run_recon(ctx, c.b, c.w, P.conn_recon, P.variant, P.max_local, c.err, s, lim, pick);
+        };
+        bool aside = false;
         if (!learned) {
-            st = run_recon(ctx, c.b, c.w, P.conn_recon, P.variant, P.max_local, c.w.err, s, lim);
+            st = reconstruct(nullptr);
             if (st != RT_OK) return st;
         } else {
             // the picker chooses a variant per tile on the device; the
-            // propagation reads its choices directly (no host round trip)
+            // propagation reads its choices directly (no host round trip).
+            // With raster classes and a contracted reconstruction the picks
+            // are reported but change no schedule: then the picker runs
+            // beside the chain on the context's own stream, forked at the
+            // call's start and joined at its end (by events, so a capture of
+            // the call captures both).
             const bool pick = picks_matter(ctx, P, cn);
-            if (pick) {
-                Phase ph(ctx, RT_PHASE_PICK, s);
-                RT_CUDA_TRY(launch_features_pick(c.fb, c.feat, ctx->picker_wb, ctx->picker_norm, c.picks,
-                                                 (float)P.pick_min_prob / 1000.0f, kPickClasses, s));
-                ctx->launches += 4;
+            aside = pick && c.contract;
+            if (aside) {
+                RT_CUDA_TRY(cudaEventRecord(ctx->fork, s));
+            } else if (pick) {
+                st = run_picker(ctx, c, P, s);
+                if (st != RT_OK) return st;
             }
-            st = run_recon(ctx, c.b, c.w, P.conn_recon, P.variant, P.max_local, c.w.err, s, lim,
-                           pick ? c.picks : nullptr);
+            st = reconstruct(pick ? c.picks : nullptr);
             if (st != RT_OK) return st;
-            // written by a kernel into the mapped pinned buffer: a copy-engine
-            // transfer here would queue behind the caller's read-backs on the
-            // same engine and hold up the rest of the chain
-            copy_picks_kernel<<<1, 32, 0, s>>>(pick ? c.picks : nullptr, ctx->picks_mapped, cn);
-            RT_CUDA_TRY(cudaGetLastError());
-            ctx->launches += 1;
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-            if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
-            ctx->picks_ev_valid = cap == cudaStreamCaptureStatusNone;
-            if (ctx->picks_ev_valid) RT_CUDA_TRY(cudaEventRecord(ctx->picks_ev, s));
-            ctx->n_last_picks = cn;
+            if (!aside) {
+                st = report_picks(ctx, pick ? c.picks : nullptr, cn, s);
+                if (st != RT_OK) return st;
+            }
         }
         {
             Phase ph(ctx, RT_PHASE_RECON_OUT, s);
             ctx->launches += 1;
-            RT_CUDA_TRY(launch_recon_out(c.b, P.threshold, s));
+            RT_CUDA_TRY(c.contract ? launch_contract_out(c.cb, P.threshold, s) : launch_recon_out(c.b, P.threshold, s));
         }
         {
             c.fill.conn = P.conn_fill;
             c.fill.flags = c.fill_flags;
             c.fill.pending = c.fill_pending;
-            c.fill.err = c.w.err;
+            c.fill.err = c.err;
             c.fill.timeout_ns = lim.timeout_ns;
             Phase ph(ctx, RT_PHASE_FILL, s);
             ctx->launches += 3;
@@ -1141,6 +1293,14 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
             ctx->launches += 3;
             RT_CUDA_TRY(launch_edt_bits_batch(c.eb, s));
         }
+        if (aside) {   // enqueued last: its launches delay none of the chain's
+            RT_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork, 0));
+            st = run_picker(ctx, c, P, ctx->side);
+            if (st == RT_OK) st = report_picks(ctx, c.picks, cn, ctx->side);
+            RT_CUDA_TRY(cudaEventRecord(ctx->join, ctx->side));
+            RT_CUDA_TRY(cudaStreamWaitEvent(s, ctx->join, 0));
+            if (st != RT_OK) return st;
+        }
         StatusOut so;
         bool any_status = false;
         for (int i = 0; i < cn; ++i) {
@@ -1148,7 +1308,7 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
             any_status |= so.dst[i] != nullptr;
         }
         if (any_status) {
-            copy_status_kernel<<<1, 32, 0, s>>>(c.w.err, so, cn);
+            copy_status_kernel<<<1, 32, 0, s>>>(c.err, so, cn);
             ctx->launches += 1;
             RT_CUDA_TRY(cudaGetLastError());
         }
