@@ -391,9 +391,7 @@ void carve_contract(Carve &cv, CtBatch &b)
     b.link = cv.take<unsigned long long>(nt * kCtNodes);
     b.best = cv.take<unsigned long long>(nt * kCtNodes);
     b.act = cv.take<uint32_t>(nt * kCtNodes);
-    b.ea = cv.take<uint32_t>(nt * kCtEdges);
-    b.eb = cv.take<uint32_t>(nt * kCtEdges);
-    b.ew = cv.take<uint8_t>(nt * kCtEdges);
+    b.edge = cv.take<unsigned long long>(nt * kCtUnits * kCtUnitEdges);
 }
 
 // Enqueue the contraction of a carved batch; launch_contract_out writes R.

@@ -17,16 +17,18 @@
 // values pixel by pixel across the image, each round at least halves the
 // open clusters, so the chain of dependent steps is logarithmic.
 //
-// Three facts make the first steps cheap:
+// Two facts make the first steps cheap:
 //   * a pixel with a neighbour q of I(q) >= I(p) satisfies R(p) =
 //     min(I(p), R(q)) for any such q, so the first contraction is one
 //     3 x 3 maximum: every pixel points at its largest neighbour (ties by
 //     raster order) and only the local maxima remain as clusters (one in
 //     nine pixels of a noisy image);
-//   * an edge that is the smallest of a triangle is in no maximum spanning
-//     forest. In a 2 x 2 window all four pixels are neighbours, so of its
-//     six edges only the three at its largest pixel can matter; and of two
-//     edges from one pixel into one cluster only the larger can.
+//   * an edge that is the smallest of a cycle is in no maximum spanning
+//     forest. A pixel p needs one edge of weight I(p) into each connected
+//     group of its larger neighbours (inside a group they reach each other by
+//     larger edges), and the group of its largest neighbour is the one p
+//     already points into. So only the pixels whose larger neighbours fall
+//     into several groups (one in four) have edges between clusters to give.
 //
 // Launches: ct_local_kernel contracts every 64 x 64 tile in shared memory
 // until each open cluster's best edge leaves the tile; what is left of a
@@ -37,9 +39,9 @@
 // ct_out_kernel writes R.
 //
 // Measured on one GB300 against the directional sweeps (rt_segment_batch or
-// rt_reconstruct, whole call): 512 x 512 reconstruction 155 us against 341;
-// one 4096 x 4096 tile 0.81 ms against 1.40; eight of them 4.84 ms against
-// 5.69; a 16384 x 16384 slide 9.4 ms against 10.3. So the contraction runs
+// rt_reconstruct, whole call): 512 x 512 reconstruction 85 us against 357;
+// one 4096 x 4096 tile 0.66 ms against 1.37; eight of them 3.55 ms against
+// 5.65; a 16384 x 16384 slide 6.9 ms against 10.4. So the contraction runs
 // wherever the call leaves the schedule to the library.
 #include "contract.cuh"
 
@@ -47,51 +49,83 @@ namespace rtk {
 
 namespace {
 
-constexpr int kT = 256;                    // threads of the local kernel
-constexpr int kWarps = kT / 32;
-constexpr int kStride = 68;                // words per row of the pixel array
-// Pixel (r, c) of the tile, -1 <= r, c <= 64 (one pixel of halo), is word
-// (r + 1) * kStride + c + 4; column 64 falls on the unused first word of the
-// next row. Indices grow in raster order.
-constexpr int kPixWords = (kCtSide + 2) * kStride + 4;
 // Roots of the first contraction: local maxima in the tile, no two adjacent.
 constexpr int kRoots = 1024;
-// Edges between clusters after the triangle rule: one diagonal in each of
-// the 65 x 65 windows that meet the tile, at most 32 straight pairs per row
-// or column of windows (2 x 32 x 65), less the tree edges of the first
-// contraction that are among them (at least 3072 - 252).
-constexpr int kList = 5632;
-constexpr size_t kLocalSmem = sizeof(uint32_t) * (kPixWords + kList + 2 * kRoots);
+// Edges that the pixels give: the groups of larger neighbours beyond the
+// first, summed over the tile, are roots + minima - 1 (Euler characteristic;
+// a minimum: all four edge neighbours larger, so no two of them adjacent and
+// none on the rim): at most 1024 + 62 * 62 / 2.
+constexpr int kList = 2976;
+// A neighbour's code: (row + 1) * 3 + column + 1 of its step; 4: the pixel itself.
+constexpr int kCodes = 9;
+// Shared memory: pixel words, edges, link words, the parents (whose memory
+// then holds the best edges and two lists of roots), the groups' table. It
+// is cut to let five CTAs share an SM.
+constexpr size_t kLocalSmem = sizeof(uint32_t) * (kCtPx + kList + kRoots) + sizeof(uint16_t) * (kCtPx + kCodes * 256);
+static_assert(sizeof(uint16_t) * kCtPx == sizeof(uint32_t) * kRoots + 2 * sizeof(uint16_t) * kRoots, "reused memory");
 
-// A pixel's word: I << 24 | index << 11 | low. Words order pixels by (I,
-// raster index). A pixel outside the image is 0, below every pixel. low of a
-// pixel of the tile: first the step to its parent + 128, then kIn | cluster;
-// low of a halo pixel: its row and column parity (no two of a 2 x 2 window
-// alike).
-constexpr uint32_t kLow = 0x7ffu, kIn = 0x400u, kIdx = 0x3ffu;
-
-// An edge's key: I << 24 | index << 11 of its smaller pixel, I of the larger
-// one << 3, direction from the smaller to the larger (0..7 in raster order:
-// NW N NE W E SW S SE). Keys order the edges totally, by (smaller, larger)
-// pixel, in the same way in every tile that sees them. 0: none.
-__device__ __forceinline__ int step_of(uint32_t key)
+// For every set of larger neighbours (bit j: kNear[j]) and code of the
+// largest: one neighbour of each group that does not hold the largest, as up
+// to three nibbles code + 1.
+struct alignas(16) GroupTable {
+    uint16_t v[kCodes * 256];
+};
+constexpr int kNear[8] = {0, 1, 2, 3, 5, 6, 7, 8};
+constexpr GroupTable group_table()
 {
-    // bytes -69 -68 -67 -1 | 1 67 68 69
-    return (int)(int8_t)__byte_perm(0xffbdbcbbu, 0x45444301u, key & 7u);
+    GroupTable g{};
+    for (int c = 0; c < kCodes; ++c)
+        for (int m = 0; m < 256; ++m) {
+            int left = m, out = 0, shift = 0;
+            bool valid = false;
+            for (int j = 0; j < 8; ++j) valid = valid || (kNear[j] == c && ((m >> j) & 1));
+            while (valid && left) {
+                int grp = left & -left, rep = 0;
+                while (!((left >> rep) & 1)) ++rep;
+                for (bool more = true; more;) {
+                    more = false;
+                    for (int a = 0; a < 8; ++a)
+                        for (int b = 0; b < 8; ++b) {
+                            const int dr = kNear[a] / 3 - kNear[b] / 3, dc = kNear[a] % 3 - kNear[b] % 3;
+                            const bool next = dr >= -1 && dr <= 1 && dc >= -1 && dc <= 1;
+                            if (((grp >> a) & 1) && ((m >> b) & 1) && !((grp >> b) & 1) && next) grp |= 1 << b, more = true;
+                        }
+                }
+                left &= ~grp;
+                bool own = false;
+                for (int j = 0; j < 8; ++j) own = own || (((grp >> j) & 1) && kNear[j] == c);
+                if (!own) out |= (kNear[rep] + 1) << shift, shift += 4;
+            }
+            g.v[c * 256 + m] = (uint16_t)out;
+        }
+    return g;
 }
-__device__ __forceinline__ uint32_t edge_key(uint32_t lo, uint32_t hi, uint32_t dir)
-{
-    return (lo & ~kLow) | ((hi >> 24) << 3) | dir;
-}
+__device__ constexpr GroupTable kGroupTable = group_table();
 
-// A cluster's link word: root: kRootBit | S; else weight << 16 | parent.
+// A pixel's word: I << 24 | index in the tile << 12 | kPix, later | kIn |
+// cluster. Words order the tile's pixels by (I, raster index); a pixel
+// outside the image is 0, below every pixel.
+constexpr uint32_t kPix = 0x800u, kIn = 0x400u, kIdx = 0x3ffu, kLabel = 0x7ffu;
+
+// A node's link word: root: kNodeRoot | kNodeDone (final) | S << 40 | itself;
+// else weight << 32 | parent. An edge of nodes: weight << 56 | node << 28 | node.
+constexpr unsigned long long kNodeRoot = 1ull << 63, kNodeDone = 1ull << 62;
+constexpr uint32_t kNodeId = (1u << 28) - 1u;
+__device__ __forceinline__ unsigned long long node_edge(uint32_t a, uint32_t b, uint32_t w)
+{
+    return (unsigned long long)w << 56 | (unsigned long long)a << 28 | b;
+}
+__device__ __forceinline__ uint32_t node_S(unsigned long long root) { return (uint32_t)(root >> 40) & 0xffu; }
+
+// A cluster's link word: root: kRootBit | X << 8 | S, X = 1 + the weight of its
+// best edge that leaves the tile (0: none); else weight << 16 | parent.
 constexpr uint32_t kRootBit = 0x80000000u;
 __device__ __forceinline__ uint32_t root_of(const volatile uint32_t *nlink, uint32_t k)
 {
-    const uint32_t v = nlink[k];   // links point at the root between rounds
+    const uint32_t v = nlink[k];   // k was a root in the last round, or links are compressed
     return (v & kRootBit) ? k : (v & 0xffffu);
 }
-
+// In the rounds an edge is weight << 24 | cluster << 12 | cluster.
 __device__ __forceinline__ const CtImage &ct_image(const CtBatch &b, int t)
 {
     int k = 0;
@@ -100,20 +134,31 @@ __device__ __forceinline__ const CtImage &ct_image(const CtBatch &b, int t)
 }
 
 __device__ __forceinline__ uint32_t max3(uint32_t a, uint32_t b, uint32_t c) { return max(a, max(b, c)); }
-
 }  // namespace
 
 // ------------------------------------------------------------------ local
-template <bool MARKER>
-__global__ void __launch_bounds__(kT, 4) ct_local_kernel(const __grid_constant__ CtBatch b)
+// NT threads; a warp takes 64 / warps rows, a lane two adjacent columns.
+// Bound by instruction issue (77 % active, 49 k warp instructions a tile,
+// 220 us per 4096 x 4096 image, DRAM idle). What it measured on that image:
+// edges from 2 x 2 windows with flags 377 us; cluster ids in the edges, lists
+// of open roots, parents apart from the pixel words 290; edges from groups of
+// larger neighbours by table 240; loops kept rolled (43 KB of code instead of
+// 88, which missed the instruction cache) and five CTAs an SM instead of four
+// 220. The first full version took 373 us.
+template <bool MARKER, int NT>
+__global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const __grid_constant__ CtBatch b)
 {
+    constexpr int kWarps = NT / 32, kRows = kCtSide / kWarps, kPer = kRoots / NT;
     extern __shared__ __align__(16) uint32_t ct_smem[];
     uint32_t *W = ct_smem;                      // pixel words
-    uint32_t *list = W + kPixWords;             // edge keys
-    volatile uint32_t *best = list + kList;     // per cluster: its best edge
-    volatile uint32_t *nlink = best + kRoots;   // per cluster: link word
+    uint32_t *list = W + kCtPx;                 // edges
+    volatile uint32_t *nlink = list + kList;    // per cluster: link word
+    volatile uint16_t *P = reinterpret_cast<volatile uint16_t *>(nlink + kRoots);   // per pixel: code << 12 | parent
+    volatile uint32_t *best = nlink + kRoots;   // then, per cluster: weight << 13 | position of its best edge, + 1
+    volatile uint16_t *live = P + 2 * kRoots;   // and two lists of open roots
+    uint16_t *table = const_cast<uint16_t *>(P) + kCtPx;                            // kGroupTable
     volatile uint32_t *VW = W;
-    __shared__ int s_roots, s_edges, s_nodes, s_forest;
+    __shared__ int s_roots, s_edges, s_nodes, s_forest, s_live[2];
 
     const int tile = blockIdx.x;
     const CtImage &d = ct_image(b, tile);
@@ -122,81 +167,84 @@ __global__ void __launch_bounds__(kT, 4) ct_local_kernel(const __grid_constant__
     const int r0 = ty * kCtSide, c0 = tx * kCtSide;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const uint32_t below = (1u << lane) - 1u;
+    const int rs = warp * kRows, cl = 2 * lane;
 
-    if (t == 0) s_roots = s_edges = s_nodes = s_forest = 0;
+    if (t == 0) s_roots = s_edges = s_nodes = s_forest = s_live[0] = s_live[1] = 0;
 
-    // ---- load the tile and its halo
+    // ---- load the tile; the rim threads (four sides of 64) also the largest
+    // halo pixel next to their pixel, + 1 (0: none)
+    uint32_t halo = 0;
+    const int side = t >> 6, si = t & 63;
+    const int rim = side == 0 ? si : side == 1 ? (kCtSide - 1) * kCtSide + si : side == 2 ? si * kCtSide : si * kCtSide + kCtSide - 1;
+    if (t < 256) {
+        const bool open = side == 0 ? ty > 0 : side == 1 ? ty + 1 < d.ny : side == 2 ? tx > 0 : tx + 1 < d.nx;
+        if (open) {
+#pragma unroll
+            for (int k = -1; k <= 1; ++k) {
+                const int r = side == 0 ? r0 - 1 : side == 1 ? r0 + kCtSide : r0 + si + k;
+                const int c = side == 2 ? c0 - 1 : side == 3 ? c0 + kCtSide : c0 + si + k;
+                if (r >= 0 && r < d.H && c >= 0 && c < d.W)
+                    halo = max(halo, (uint32_t)__ldg(d.mask + (int64_t)r * d.ld_mask + c) + 1u);
+            }
+        }
+    }
+#pragma unroll 1
+    for (int i = t; i < kCodes * 256 / 8; i += NT)
+        reinterpret_cast<uint4 *>(table)[i] = __ldg(reinterpret_cast<const uint4 *>(kGroupTable.v) + i);
     {
         const bool wide = (((uintptr_t)d.mask | (uintptr_t)d.ld_mask) & 3u) == 0;
-        const int q = t & 15;
-        const int c = c0 + 4 * q;
-        for (int rr = t >> 4; rr < kCtSide + 2; rr += kT / 16) {
-            const int r = r0 + rr - 1;
-            const int n = (r >= 0 && r < d.H) ? min(4, d.W - c) : 0;   // may be negative: none
+        const int c = c0 + 4 * (t & 15);
+#pragma unroll
+        for (int rr = t >> 4; rr < kCtSide; rr += NT / 16) {
+            const int r = r0 + rr, n = r < d.H ? min(4, d.W - c) : 0;   // may be negative: none
             uint32_t v = 0;
             const uint8_t *p = d.mask + (int64_t)r * d.ld_mask + c;
             if (n == 4 && wide) {
                 v = __ldg(reinterpret_cast<const uint32_t *>(p));
             } else {
+#pragma unroll 1
                 for (int k = 0; k < n; ++k) v |= (uint32_t)__ldg(p + k) << (8 * k);
             }
-            const int idx = rr * kStride + 4 * q + 4;
-            const bool halo = rr == 0 || rr == kCtSide + 1;
+            const uint32_t idx = (uint32_t)(rr * kCtSide + 4 * (t & 15));
             uint32_t o[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t low = halo ? (uint32_t)((rr & 1) << 1 | (k & 1)) : 0u;
-                o[k] = k < n ? ((v >> (8 * k)) & 0xffu) << 24 | (uint32_t)(idx + k) << 11 | low : 0u;
-            }
+            for (int k = 0; k < 4; ++k) o[k] = k < n ? __byte_perm(v, 0u, k << 12 | 0x0444u) | (idx + k) << 12 | kPix : 0u;
             *reinterpret_cast<uint4 *>(W + idx) = make_uint4(o[0], o[1], o[2], o[3]);
-        }
-        if (t < 2 * (kCtSide + 2)) {
-            const int rr = t >> 1, right = t & 1;
-            const int r = r0 + rr - 1, ch = right ? c0 + kCtSide : c0 - 1;
-            const int idx = rr * kStride + (right ? kCtSide + 4 : 3);
-            uint32_t w = 0;
-            if (r >= 0 && r < d.H && ch >= 0 && ch < d.W)
-                w = (uint32_t)__ldg(d.mask + (int64_t)r * d.ld_mask + ch) << 24 | (uint32_t)idx << 11 |
-                    (uint32_t)((rr & 1) << 1 | (right ? 0 : 1));
-            W[idx] = w;
         }
     }
     __syncthreads();
 
     // ---- first contraction: every pixel points at the largest pixel of its
-    // 3 x 3 neighbourhood in the tile. Thread = column, 16 rows of one strip.
-    // Only the low bits of words change here, which no comparison sees.
-    const int c = t & (kCtSide - 1), rs = (t >> 6) * 16;
-    uint32_t rootmask = 0;
+    // 3 x 3 neighbourhood in the tile. (At the row's ends the shuffles return
+    // the lane's own word, which is in the neighbourhood anyway.)
+    auto row_of = [&](int r) -> uint2 {
+        if (r < 0 || r >= kCtSide) return make_uint2(0u, 0u);   // whole warp
+        return *reinterpret_cast<const uint2 *>(W + r * kCtSide + cl);
+    };
+    uint32_t rootmask = 0;   // bit 2 j + k: pixel (rs + j, cl + k) is a root
     {
-        auto row3 = [&](int r, uint32_t &ctr) -> uint32_t {
-            if (r < 0 || r >= kCtSide) {
-                ctr = 0u;
-                return 0u;
-            }
-            const volatile uint32_t *x = VW + (r + 1) * kStride + c + 4;
-            ctr = x[0];
-            const uint32_t l = c > 0 ? x[-1] : 0u, rt = c < kCtSide - 1 ? x[1] : 0u;
-            return max3(l, ctr, rt);
+        auto across = [&](uint2 v) -> uint2 {
+            const uint32_t l = __shfl_up_sync(0xffffffffu, v.y, 1), r = __shfl_down_sync(0xffffffffu, v.x, 1);
+            const uint32_t m = max(v.x, v.y);
+            return make_uint2(max(lane ? l : 0u, m), max(lane < 31 ? r : 0u, m));
         };
-        uint32_t ca, cb, cc;
-        uint32_t ha = row3(rs - 1, ca), hb = row3(rs, cb);
-#pragma unroll 4
-        for (int j = 0; j < 16; ++j) {
-            const uint32_t hc = row3(rs + j + 1, cc);
-            const uint32_t m = max3(ha, hb, hc);
-            if (cb) {
-                if (m == cb) {
-                    rootmask |= 1u << j;
-                } else {
-                    const int idx = (rs + j + 1) * kStride + c + 4;
-                    const int st = (int)((m >> 11) & 0x1fffu) - idx;
-                    VW[idx] = (cb & ~kLow) | (uint32_t)(st + 128);
-                }
-            }
+        uint2 vb = row_of(rs), ha = across(row_of(rs - 1)), hb = across(vb);
+#pragma unroll 2
+        for (int j = 0; j < kRows; ++j) {
+            const uint2 vc = row_of(rs + j + 1), hc = across(vc);
+            const uint32_t m0 = max3(ha.x, hb.x, hc.x) >> 12, m1 = max3(ha.y, hb.y, hc.y) >> 12;
+            if (vb.x && m0 == vb.x >> 12) rootmask |= 1u << (2 * j);
+            if (vb.y && m1 == vb.y >> 12) rootmask |= 2u << (2 * j);
+            const uint32_t at = (uint32_t)((rs + j) * kCtSide + cl);
+            auto pack = [](uint32_t own, uint32_t to, uint32_t here) -> uint32_t {
+                if (!own) to = here;
+                const uint32_t step = to - here + 65u;   // 64 (row + 1) + column + 1
+                return to | ((step >> 6) * 3u + (step & 3u)) << 12;
+            };
+            reinterpret_cast<volatile uint32_t *>(P)[at / 2] = pack(vb.x, m0 & 0xfffu, at) | pack(vb.y, m1 & 0xfffu, at + 1) << 16;
             ha = hb;
             hb = hc;
-            cb = cc;
+            vb = vc;
         }
     }
     {
@@ -210,125 +258,148 @@ __global__ void __launch_bounds__(kT, 4) ct_local_kernel(const __grid_constant__
         int base = 0;
         if (lane == 31) base = atomicAdd(&s_roots, inc);
         uint32_t k = (uint32_t)(__shfl_sync(0xffffffffu, base, 31) + inc - n);
+#pragma unroll 1
         while (rootmask) {
             const int j = __ffs(rootmask) - 1;
             rootmask &= rootmask - 1;
-            const int idx = (rs + j + 1) * kStride + c + 4;
+            const int idx = (rs + (j >> 1)) * kCtSide + cl + (j & 1);
             const uint32_t w = VW[idx];
             // the derived marker's largest value in the cluster is at its maximum
             const uint32_t I = w >> 24;
             const uint32_t S = MARKER ? 0u : (I > (uint32_t)d.h_offset ? I - (uint32_t)d.h_offset : 0u);
-            VW[idx] = (w & ~kLow) | kIn | k;
+            VW[idx] = w | kIn | k;
             nlink[k] = kRootBit | S;
-            best[k] = 0u;
             ++k;
         }
     }
     __syncthreads();
     const int nr = s_roots;
 
-    // ---- every pixel's cluster: follow the steps uphill. A finished pixel's
-    // word ends the walk of those that come through it.
+    // ---- every pixel's cluster: four steps uphill without a test (nearly
+    // always enough), then until a root. Parents are replaced by what was
+    // found, which shortens the long walks of flat images.
     {
         bool bad = false;
-#pragma unroll 4
-        for (int j = 0; j < 16; ++j) {
-            const int r = rs + j, idx = (r + 1) * kStride + c + 4;
-            uint32_t w = VW[idx];
-            if (!w) continue;
-            if (!(w & kIn)) {
-                int x = idx;
-                uint32_t v = w;
-                for (int n = 0; n < kCtPx && !(v & kIn); ++n) {
-                    x += (int)(v & 0xffu) - 128;
-                    v = VW[x];
+#pragma unroll 2
+        for (int j = 0; j < kRows; ++j) {
+            const int at = (rs + j) * kCtSide + cl;
+            const uint2 ow = *reinterpret_cast<const uint2 *>(W + at);
+            const uint32_t pp = reinterpret_cast<volatile uint32_t *>(P)[at / 2];
+            uint32_t x[2] = {pp & 0xfffu, (pp >> 16) & 0xfffu}, v[2], own[2] = {ow.x, ow.y};
+#pragma unroll
+            for (int n = 0; n < 3; ++n) x[0] = P[x[0]] & 0xfffu, x[1] = P[x[1]] & 0xfffu;
+            reinterpret_cast<volatile uint32_t *>(P)[at / 2] = (pp & 0xf000f000u) | x[0] | x[1] << 16;
+            v[0] = VW[x[0]], v[1] = VW[x[1]];
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll 1
+                for (int n = 0; n < kCtPx && own[q] && !(v[q] & kIn); ++n) {
+                    x[q] = P[x[q]] & 0xfffu;
+                    v[q] = VW[x[q]];
                 }
-                w = (w & ~kLow) | (v & kLow);
-                VW[idx] = w;
-            }
-            const uint32_t k = w & kIdx, I = w >> 24;
-            const int gr = r0 + r, gc = c0 + c;
-            uint32_t *sk = const_cast<uint32_t *>(nlink + k);
-            if (MARKER) {
-                const uint32_t J = __ldg(d.marker + (int64_t)gr * d.ld_marker + gc);
-                bad |= J > I;
-                const uint32_t v = kRootBit | min(J, I);
-                if (nlink[k] < v) atomicMax(sk, v);
-            } else if (gr == 0 || gr == d.H - 1 || gc == 0 || gc == d.W - 1) {
-                atomicMax(sk, kRootBit | I);
+            uint2 nw = ow;
+            if (ow.x) nw.x = ow.x | (v[0] & kLabel);
+            if (ow.y) nw.y = ow.y | (v[1] & kLabel);
+            *reinterpret_cast<uint2 *>(W + at) = nw;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int r = rs + j, c = cl + q;
+                if (!own[q]) continue;
+                const uint32_t k = v[q] & kIdx, I = own[q] >> 24;
+                const int gr = r0 + r, gc = c0 + c;
+                uint32_t *sk = const_cast<uint32_t *>(nlink + k);
+                if (MARKER) {
+                    const uint32_t J = __ldg(d.marker + (int64_t)gr * d.ld_marker + gc);
+                    bad |= J > I;
+                    const uint32_t s = kRootBit | min(J, I);
+                    if (nlink[k] < s) atomicMax(sk, s);
+                } else if (gr == 0 || gr == d.H - 1 || gc == 0 || gc == d.W - 1) {
+                    atomicMax(sk, kRootBit | I);
+                }
             }
         }
         if (MARKER && bad) raise_status(b.err, RT_EMARKER);
     }
     __syncthreads();
 
-    // ---- edges between clusters that pass the triangle rule. The owner of
-    // an edge is the window whose upper left pixel is (r, c).
-    {
-        // larger pixel hi, smaller lo; x: a common neighbour. The edge can go
-        // if x is above both, or above lo and in lo's cluster.
-        auto drops = [&](uint32_t x, uint32_t lo, uint32_t hi) {
-            return x > (((x ^ lo) & kLow) == 0u ? lo : hi);
-        };
-        auto joins = [&](uint32_t lo, uint32_t hi) {   // both exist, one in the tile, not one cluster
-            return lo && ((lo | hi) & kIn) && ((lo ^ hi) & kLow);
-        };
-        auto diagonal = [&](uint32_t m, uint32_t mr, uint32_t dn, uint32_t dr) -> uint32_t {
-            const bool main = max(m, dr) > max(mr, dn);
-            const uint32_t p = main ? m : mr, q = main ? dr : dn;   // p in the upper row
-            const uint32_t x = main ? mr : m, y = main ? dn : dr;
-            const uint32_t lo = min(p, q), hi = max(p, q);
-            if (!joins(lo, hi) || drops(x, lo, hi) || drops(y, lo, hi)) return 0u;
-            const uint32_t dir = lo == p ? (main ? 7u : 5u) : (main ? 0u : 2u);
-            return edge_key(lo, hi, dir);
-        };
-        auto straight = [&](uint32_t p, uint32_t q, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
-                            uint32_t dp, uint32_t dq) -> uint32_t {
-            const uint32_t lo = min(p, q), hi = max(p, q);
-            if (!joins(lo, hi) || drops(x0, lo, hi) || drops(x1, lo, hi) || drops(x2, lo, hi) || drops(x3, lo, hi))
-                return 0u;
-            return edge_key(lo, hi, lo == p ? dp : dq);
-        };
-        auto append = [&](uint32_t e0, uint32_t e1, uint32_t e2) {   // whole warp
-            const int n = (e0 != 0u) + (e1 != 0u) + (e2 != 0u);
-            const uint32_t b0 = __ballot_sync(0xffffffffu, n & 1), b1 = __ballot_sync(0xffffffffu, n & 2);
-            const int total = __popc(b0) + 2 * __popc(b1);
-            if (total == 0) return;
-            int at = 0;
-            if (lane == 0) at = atomicAdd(&s_edges, total);
-            at = __shfl_sync(0xffffffffu, at, 0) + __popc(b0 & below) + 2 * __popc(b1 & below);
-            if (at + n > kList) return;   // cannot happen (see kList)
-            if (e0) list[at++] = e0;
-            if (e1) list[at++] = e1;
-            if (e2) list[at] = e2;
-        };
-        const int first = rs == 0 ? -1 : rs;
-        const uint32_t *x = W + (first + 1) * kStride + c + 4;
-        uint32_t u = 0, ur = 0;                       // row above (only rows >= 0 use it)
-        if (first > 0) u = x[-kStride], ur = x[1 - kStride];
-        uint32_t ml = x[-1], m = x[0], mr = x[1];
-        for (int r = first; r < rs + 16; ++r) {
-            x += kStride;
-            const uint32_t dl = x[-1], dn = x[0], dr = x[1];
-            const uint32_t e0 = diagonal(m, mr, dn, dr);
-            const uint32_t e1 = straight(m, mr, u, ur, dn, dr, 4u, 3u);
-            const uint32_t e2 = straight(m, dn, ml, mr, dl, dr, 6u, 1u);
-            append(e0, e1, e2);
-            u = m, ur = mr;
-            ml = dl, m = dn, mr = dr;
-        }
-        // the windows left of the tile (c = -1)
-        if (warp < 3) {
-            const int r = t - 1;
-            uint32_t e0 = 0, e1 = 0;
-            if (r < kCtSide) {
-                const uint32_t *y = W + (r + 1) * kStride + 3;
-                e0 = diagonal(y[0], y[1], y[kStride], y[kStride + 1]);
-                if (r >= 0) e1 = straight(y[0], y[1], y[-kStride], y[1 - kStride], y[kStride], y[kStride + 1], 4u, 3u);
-            }
-            append(e0, e1, 0u);
+    // ---- the pixels' edges, as index | (code + 1) << 12, and the best edge of
+    // every rim cluster that leaves the tile
+    if (halo) {
+        const uint32_t w = W[rim];
+        if (w) {
+            const uint32_t k = w & kIdx, old = nlink[k], v = kRootBit | min((w >> 24) + 1u, halo) << 8 | (old & 0xffu);
+            if (old < v) atomicMax(const_cast<uint32_t *>(nlink + k), v);
         }
     }
+    {
+        // rows of words >> 4 (only their order counts), with the columns beside the lane's two
+        auto load = [&](int r, uint32_t (&o)[4]) {
+            const uint2 v = row_of(r);
+            o[1] = v.x >> 4;
+            o[2] = v.y >> 4;
+            o[0] = __shfl_up_sync(0xffffffffu, o[2], 1);
+            o[3] = __shfl_down_sync(0xffffffffu, o[1], 1);
+            if (lane == 0) o[0] = 0u;
+            if (lane == 31) o[3] = 0u;
+        };
+        uint32_t u[4], m[4], n[4];
+        load(rs - 1, u);
+        load(rs, m);
+        // a pixel's second and third edge (rare) wait in `more`, 16 bits each
+        unsigned long long more = 0;
+        auto put = [&](uint32_t e0, uint32_t e1) {   // whole warp
+            const uint32_t b0 = __ballot_sync(0xffffffffu, e0 != 0u), b1 = __ballot_sync(0xffffffffu, e1 != 0u);
+            const int n0 = __popc(b0);
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&s_edges, n0 + __popc(b1));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            const int p0 = at + __popc(b0 & below), p1 = at + n0 + __popc(b1 & below);
+            if (e0 && p0 < kList) list[p0] = e0;   // p < kList: always (see kList)
+            if (e1 && p1 < kList) list[p1] = e1;
+        };
+        auto flush = [&]() {
+            do {
+                put((uint32_t)more & 0xffffu, (uint32_t)(more >> 16) & 0xffffu);
+                more >>= 32;
+            } while (__any_sync(0xffffffffu, more != 0ull));
+        };
+#pragma unroll 1   // the loops over rows stay rolled: the kernel's time is lost to instruction fetch otherwise
+        for (int j = 0; j < kRows; ++j) {
+            const int r = rs + j;
+            load(r + 1, n);
+            const uint32_t pp = reinterpret_cast<volatile uint32_t *>(P)[(r * kCtSide + cl) / 2];
+            uint32_t g[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                // bit j of the set: kNear[j] is larger (the sign of a difference, shifted in)
+                const uint32_t near[8] = {u[q], u[q + 1], u[q + 2], m[q], m[q + 2], n[q], n[q + 1], n[q + 2]};
+                uint32_t set = 0;
+#pragma unroll
+                for (int j = 7; j >= 0; --j) set = __funnelshift_l(m[q + 1] - near[j], set, 1);
+                const uint32_t code = q ? pp >> 28 : (pp >> 12) & 0xfu;
+                g[q] = table[code * 256u + (set & 0xffu)];
+                if (m[q + 1] == 0u) g[q] = 0u;
+            }
+            const uint32_t at0 = (uint32_t)(r * kCtSide + cl);
+            put(g[0] ? at0 | (g[0] & 0xfu) << 12 : 0u, g[1] ? (at0 + 1u) | (g[1] & 0xfu) << 12 : 0u);
+            if ((g[0] | g[1]) >> 4) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+#pragma unroll 1
+                    for (uint32_t f = g[q] >> 4; f; f >>= 4) more = more << 16 | (at0 + q) | (f & 0xfu) << 12;
+            }
+            // of two adjacent pixels one at most has four groups (its corners
+            // larger, its edge neighbours not): a row adds at most 2 + 1
+            if (__any_sync(0xffffffffu, more >> 16 != 0ull)) flush();
+#pragma unroll
+            for (int q = 0; q < 4; ++q) u[q] = m[q], m[q] = n[q];
+        }
+        if (__any_sync(0xffffffffu, more != 0ull)) flush();
+    }
+    __syncthreads();
+
+#pragma unroll 1
+    for (int k = t; k < nr; k += NT) best[k] = 0u;   // in the parents' memory
     __syncthreads();
 
     // ---- contraction rounds. Each warp keeps a range of the list and
@@ -340,97 +411,146 @@ __global__ void __launch_bounds__(kT, 4) ct_local_kernel(const __grid_constant__
         start = min(warp * per, n);
         cnt = min(per, n - start);
     }
-    auto edge_pass = [&]() {
+    auto edge_pass = [&](bool first) {
         int kept = 0;
-        for (int i = 0; i < cnt; i += 32) {
-            const bool have = i + lane < cnt;
-            const uint32_t key = have ? list[start + i + lane] : 0u;
-            uint32_t ra = ~0u, rb = ~0u;
-            if (have) {
-                const int lo = (int)((key >> 11) & 0x1fffu);
-                const uint32_t wl = W[lo], wh = W[lo + step_of(key)];
-                if (wl & kIn) ra = root_of(nlink, wl & kIdx);
-                if (wh & kIn) rb = root_of(nlink, wh & kIdx);
+#pragma unroll 1
+        for (int i = lane; i < cnt + lane; i += 32) {
+            uint32_t e = 0, ra = 0, rb = 0;
+            if (i < cnt) {
+                e = list[start + i];
+                if (first) {
+                    const uint32_t p = e & 0xfffu, code = (e >> 12) - 1u;
+                    const uint32_t wp = W[p], wq = W[p + code + 61u * (code * 11u >> 5) - 65u];   // 64 row + column
+                    e = wp;
+                    ra = wp & kIdx;
+                    rb = wq & kIdx;
+                } else {
+                    ra = root_of(nlink, e & kIdx);
+                    rb = root_of(nlink, (e >> 12) & kIdx);
+                }
             }
             const bool keep = ra != rb;
             const uint32_t m = __ballot_sync(0xffffffffu, keep);
             if (keep) {
-                list[start + kept + __popc(m & below)] = key;
-                if (ra != ~0u && best[ra] < key) atomicMax(const_cast<uint32_t *>(best + ra), key);
-                if (rb != ~0u && best[rb] < key) atomicMax(const_cast<uint32_t *>(best + rb), key);
+                const uint32_t pos = start + kept + __popc(m & below);
+                list[pos] = (e & 0xff000000u) | rb << 12 | ra;
+                const uint32_t key = ((e >> 24) << 13) + pos + 1u;
+                atomicMax(const_cast<uint32_t *>(best + ra), key);
+                atomicMax(const_cast<uint32_t *>(best + rb), key);
             }
             kept += __popc(m);
             __syncwarp();
         }
         cnt = kept;
     };
-    edge_pass();
+    edge_pass(true);
     __syncthreads();
-    for (;;) {
+    // Only open roots are visited (round 0: all; then the list that the round
+    // before left). A root that is final, or whose best edge leaves the tile,
+    // stays: another may still join it.
+    int nl = nr;
+#pragma unroll 1
+    for (int round = 0;; ++round) {
+        const volatile uint16_t *from = live + (round & 1) * kRoots;
+        volatile uint16_t *to = live + (~round & 1) * kRoots;
         // decide: S << 24 | weight << 16 | parent, parent 0xffff: stays
-        uint32_t dec[kRoots / kT];
+        uint32_t dec[kPer], id[kPer];
         int any = 0;
 #pragma unroll
-        for (int q = 0; q < kRoots / kT; ++q) {
-            const uint32_t k = t + q * kT;
+        for (int q = 0; q < kPer; ++q) {
             dec[q] = 0xffffu;
-            if (k >= (uint32_t)nr) continue;
-            const uint32_t v = nlink[k], key = best[k];
-            if (!(v & kRootBit) || !key) continue;
-            const uint32_t w = key >> 24, S = v & 0xffu;
-            if (S >= w) continue;                                  // final
-            const int lo = (int)((key >> 11) & 0x1fffu);
-            const uint32_t wl = W[lo], wh = W[lo + step_of(key)];
-            if (!(wl & wh & kIn)) continue;                        // its best edge leaves the tile
-            const uint32_t ra = root_of(nlink, wl & kIdx);
-            const uint32_t o = ra == k ? root_of(nlink, wh & kIdx) : ra;
-            if (k < o && best[o] == key && (nlink[o] & 0xffu) < w) continue;   // o joins this one
+            id[q] = 0u;
+            if (t + q * NT >= nl) continue;
+            const uint32_t k = round ? from[t + q * NT] : (uint32_t)(t + q * NT);
+            id[q] = k;
+            const uint32_t key = best[k];
+            if (!key) continue;
+            const uint32_t w = (key - 1u) >> 13, v = nlink[k], S = v & 0xffu;
+            if (S >= w || ((v >> 8) & 0x1ffu) > w + 1u) continue;
+            const uint32_t e = list[(key - 1u) & 0x1fffu];
+            const uint32_t ra = e & kIdx, o = ra == k ? (e >> 12) & kIdx : ra;
+            const uint32_t vo = nlink[o];
+            if (k < o && best[o] == key && (vo & 0xffu) < w && ((vo >> 8) & 0x1ffu) <= w + 1u) continue;   // o joins this one
             dec[q] = S << 24 | w << 16 | o;
+            id[q] = k | (v & 0x1ff00u) << 8;
             any = 1;
         }
+        if (t == 0) s_live[~round & 1] = 0;
         if (!__syncthreads_or(any)) break;
 #pragma unroll
-        for (int q = 0; q < kRoots / kT; ++q)
-            if ((dec[q] & 0xffffu) != 0xffffu) nlink[t + q * kT] = dec[q] & 0xffffffu;
+        for (int q = 0; q < kPer; ++q)
+            if ((dec[q] & 0xffffu) != 0xffffu) nlink[id[q] & 0xffffu] = dec[q] & 0xffffffu;
         __syncthreads();
+        // joined: find the new root, with the smallest weight on the way, and
+        // hand it the sources; the others make the next list
 #pragma unroll
-        for (int q = 0; q < kRoots / kT; ++q) {
-            const uint32_t k = t + q * kT;
-            if (k >= (uint32_t)nr) continue;
-            uint32_t v = nlink[k];
-            if (v & kRootBit) {
+        for (int q = 0; q < kPer; ++q) {
+            if (warp * 32 + q * NT >= nl) continue;   // whole warp
+            const bool in = t + q * NT < nl, joined = (dec[q] & 0xffffu) != 0xffffu;
+            const uint32_t k = id[q] & 0xffffu;
+            if (joined) {
+                uint32_t w = (dec[q] >> 16) & 0xffu, x = dec[q] & 0xffffu;
+#pragma unroll 1
+                for (int n = 0; n < kRoots; ++n) {
+                    const uint32_t v = nlink[x];
+                    if (v & kRootBit) break;
+                    w = min(w, v >> 16);
+                    x = v & 0xffffu;
+                }
+                nlink[k] = w << 16 | x;
+#pragma unroll 1
+                for (uint32_t v = nlink[x];;) {   // both maxima at once; ends when nobody else raised them between
+                    const uint32_t m = kRootBit | max(v & 0x1ff00u, id[q] >> 8 & 0x1ff00u) | max(v & 0xffu, dec[q] >> 24);
+                    if (m == v) break;
+                    const uint32_t old = atomicCAS(const_cast<uint32_t *>(nlink + x), v, m);
+                    if (old == v) break;
+                    v = old;
+                }
+            } else if (in) {
                 best[k] = 0u;
-                continue;
             }
-            uint32_t w = v >> 16, x = v & 0xffffu;
-            for (int n = 0; n < kRoots; ++n) {
-                v = nlink[x];
-                if (v & kRootBit) break;
-                w = min(w, v >> 16);
-                x = v & 0xffffu;
-            }
-            nlink[k] = w << 16 | x;
-            if ((dec[q] & 0xffffu) != 0xffffu) atomicMax(const_cast<uint32_t *>(nlink + x), kRootBit | dec[q] >> 24);
+            const bool stays = in && !joined;
+            const uint32_t m = __ballot_sync(0xffffffffu, stays);
+            int base = 0;
+            if (lane == 0 && m) base = atomicAdd(&s_live[~round & 1], __popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (stays) to[base + __popc(m & below)] = (uint16_t)k;
         }
         __syncthreads();
-        edge_pass();
+        nl = s_live[~round & 1];
+        edge_pass(false);
         __syncthreads();
     }
 
     // ---- nodes: the clusters with a pixel on a side that has a neighbour
     // tile. best[k] becomes 1 + the node of root k, 0 for the others (which
     // are final: no edge of theirs leaves the tile).
-    for (int k = t; k < nr; k += kT) best[k] = 0u;
-    __syncthreads();
-    {
-        const int side = t >> 6, i = t & 63;
-        const bool open = side == 0 ? ty > 0 : side == 1 ? ty + 1 < d.ny : side == 2 ? tx > 0 : tx + 1 < d.nx;
-        const int r = side == 0 ? 0 : side == 1 ? kCtSide - 1 : i, cc = side < 2 ? i : side == 2 ? 0 : kCtSide - 1;
-        const uint32_t w = W[(r + 1) * kStride + cc + 4];
-        if (open && w) best[root_of(nlink, w & kIdx)] = 1u;
+#pragma unroll 1
+    for (int k = t; k < nr; k += NT) {
+        best[k] = 0u;
+        uint32_t v = nlink[k];
+        if (v & kRootBit) {
+            nlink[k] = v & (kRootBit | 0xffu);
+            continue;
+        }
+        uint32_t w = v >> 16, x = v & 0xffffu;   // links of earlier rounds: one step per round
+#pragma unroll 1
+        for (int n = 0; n < kRoots; ++n) {
+            v = nlink[x];
+            if (v & kRootBit) break;
+            w = min(w, v >> 16);
+            x = v & 0xffffu;
+        }
+        nlink[k] = w << 16 | x;
     }
     __syncthreads();
-    for (int k0 = warp * 32; k0 < nr; k0 += kT) {
+    if (halo) {
+        const uint32_t w = W[rim];
+        if (w) best[root_of(nlink, w & kIdx)] = 1u;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int k0 = warp * 32; k0 < nr; k0 += NT) {
         const int k = k0 + lane;
         const bool f = k < nr && best[k] != 0u;
         const uint32_t m = __ballot_sync(0xffffffffu, f);
@@ -447,21 +567,18 @@ __global__ void __launch_bounds__(kT, 4) ct_local_kernel(const __grid_constant__
     // as a source of its own
     {
         int kept = 0;
+#pragma unroll 1
         for (int i = 0; i < cnt; i += 32) {
             uint32_t e = 0;
             bool keep = false;
             if (i + lane < cnt) {
-                const uint32_t key = list[start + i + lane];
-                const int lo = (int)((key >> 11) & 0x1fffu);
-                const uint32_t wl = W[lo], wh = W[lo + step_of(key)];
-                if (wl & wh & kIn) {
-                    const uint32_t ra = root_of(nlink, wl & kIdx), rb = root_of(nlink, wh & kIdx);
-                    const uint32_t na = best[ra], nb = best[rb], w = key >> 24;
-                    keep = na && nb;
-                    e = (na - 1u) | (nb - 1u) << 8 | w << 16;
-                    if (na && !nb) atomicMax(const_cast<uint32_t *>(nlink + ra), kRootBit | min(w, nlink[rb] & 0xffu));
-                    if (nb && !na) atomicMax(const_cast<uint32_t *>(nlink + rb), kRootBit | min(w, nlink[ra] & 0xffu));
-                }
+                const uint32_t f = list[start + i + lane];
+                const uint32_t ra = f & kIdx, rb = (f >> 12) & kIdx, w = f >> 24;
+                const uint32_t na = best[ra], nb = best[rb];
+                keep = na && nb;
+                e = (na - 1u) | (nb - 1u) << 8 | w << 16;
+                if (na && !nb) atomicMax(const_cast<uint32_t *>(nlink + ra), kRootBit | min(w, nlink[rb] & 0xffu));
+                if (nb && !na) atomicMax(const_cast<uint32_t *>(nlink + rb), kRootBit | min(w, nlink[ra] & 0xffu));
             }
             const uint32_t m = __ballot_sync(0xffffffffu, keep);
             if (keep) list[start + kept + __popc(m & below)] = e;
@@ -473,10 +590,10 @@ __global__ void __launch_bounds__(kT, 4) ct_local_kernel(const __grid_constant__
     __syncthreads();
     // per cluster: node << 8 | bound (kCtNoNode: the value itself)
     {
-        uint32_t tab[kRoots / kT];
+        uint32_t tab[kPer];
 #pragma unroll
-        for (int q = 0; q < kRoots / kT; ++q) {
-            const uint32_t k = t + q * kT;
+        for (int q = 0; q < kPer; ++q) {
+            const uint32_t k = t + q * NT;
             tab[q] = 0u;
             if (k >= (uint32_t)nr) continue;
             uint32_t v = nlink[k], w = 255u, x = k;
@@ -489,36 +606,38 @@ __global__ void __launch_bounds__(kT, 4) ct_local_kernel(const __grid_constant__
             tab[q] = n ? (n - 1u) << 8 | w : kCtNoNode << 8 | min(w, v & 0xffu);
             if (n && x == k) {
                 const uint32_t g = (uint32_t)tile * kCtNodes + n - 1u;
-                b.S[g] = v & 0xffu;
-                b.link[g] = 255ull << 32 | g;
+                b.link[g] = kNodeRoot | (unsigned long long)(v & 0xffu) << 40 | g;
                 b.best[g] = 0ull;
             }
         }
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < kRoots / kT; ++q) {
-            const uint32_t k = t + q * kT;
+        for (int q = 0; q < kPer; ++q) {
+            const uint32_t k = t + q * NT;
             if (k < (uint32_t)nr) nlink[k] = tab[q];
         }
-        // the forest rounds below use best as two arrays of 256 words
+        // the forest rounds below use best and what follows as arrays per node
         if (t < nn) best[t] = t;
-        best[kT + t] = 0u;
+        if (t < kCtNodes) best[kRoots + t] = 0u;
     }
     __syncthreads();
     {
-        uint16_t *o = b.plane + (int64_t)tile * kCtPx + rs * kCtSide + c;
-#pragma unroll 4
-        for (int j = 0; j < 16; ++j) {
-            const uint32_t w = W[(rs + j + 1) * kStride + c + 4];
-            const uint32_t e = nlink[w & kIdx];
-            if (w) o[j * kCtSide] = (uint16_t)((e & 0xff00u) | min(e & 0xffu, w >> 24));
+        uint16_t *o = b.plane + (int64_t)tile * kCtPx + rs * kCtSide + cl;
+#pragma unroll 2
+        for (int j = 0; j < kRows; ++j) {
+            const uint2 v = row_of(rs + j);
+            const uint32_t e0 = nlink[v.x & kIdx], e1 = nlink[v.y & kIdx];
+            *reinterpret_cast<uint32_t *>(o + j * kCtSide) = (e0 & 0xff00u) | min(e0 & 0xffu, v.x >> 24) |
+                                                             (e1 & 0xff00u) << 16 | min(e1 & 0xffu, v.y >> 24) << 16;
         }
     }
 
     // ---- maximum spanning forest of the nodes (only these edges can matter)
-    volatile uint32_t *comp = best, *fb = best + kT;
+    volatile uint32_t *comp = best, *fb = best + kRoots;
+#pragma unroll 1
     for (;;) {
         int kept = 0;
+#pragma unroll 1
         for (int i = 0; i < cnt; i += 32) {
             const bool have = i + lane < cnt;
             const uint32_t e = have ? list[start + i + lane] : 0u;
@@ -544,10 +663,10 @@ __global__ void __launch_bounds__(kT, 4) ct_local_kernel(const __grid_constant__
             const uint32_t ca = comp[e & 0xffu], o = ca == (uint32_t)t ? comp[(e >> 8) & 0xffu] : ca;
             if (!((uint32_t)t < o && fb[o] == key)) {
                 join = o;
-                const int64_t g = (int64_t)tile * kCtEdges + atomicAdd(&s_forest, 1);
-                b.ea[g] = (uint32_t)tile * kCtNodes + (e & 0xffu);
-                b.eb[g] = (uint32_t)tile * kCtNodes + ((e >> 8) & 0xffu);
-                b.ew[g] = (uint8_t)(e >> 16);
+                const int i = atomicAdd(&s_forest, 1);   // dealt to the tile's units in turn
+                b.edge[((int64_t)tile * kCtUnits + i % kCtUnits) * kCtUnitEdges + i / kCtUnits] =
+                    node_edge((uint32_t)tile * kCtNodes + (e & 0xffu), (uint32_t)tile * kCtNodes + ((e >> 8) & 0xffu),
+                              e >> 16);
             }
         }
         if (!__syncthreads_or(join != ~0u)) break;
@@ -555,6 +674,7 @@ __global__ void __launch_bounds__(kT, 4) ct_local_kernel(const __grid_constant__
         __syncthreads();
         if (t < nn) {
             uint32_t x = comp[t];
+#pragma unroll 1
             for (int n = 0; n < kCtNodes && comp[x] != x; ++n) x = comp[x];
             comp[t] = x;
             fb[t] = 0u;
@@ -567,9 +687,11 @@ __global__ void __launch_bounds__(kT, 4) ct_local_kernel(const __grid_constant__
 // ----------------------------------------------------------------- global
 namespace {
 
-constexpr int kGT = 256;
+constexpr int kGT = 1024;
+constexpr int kGCluster = 8;
+constexpr int64_t kGClusterUnits = 512;
+constexpr int kFewTiles = 304;
 constexpr uint32_t kMix = 2654435761u, kUnmix = 244002641u;   // inverses mod 2^32: ties in no geometric order
-constexpr uint32_t kDone = 0x80000000u;
 constexpr int kMaxRounds = 64;
 static_assert(kMix * kUnmix == 1u, "inverse");
 
@@ -580,33 +702,48 @@ __device__ __forceinline__ uint32_t ct_node(const CtBatch &b, const CtImage &d, 
     return (uint32_t)t * kCtNodes + (e >> 8);
 }
 
-__device__ __forceinline__ uint32_t ct_root(const CtBatch &b, uint32_t x)
+// The root above node x and its link word.
+__device__ __forceinline__ uint32_t ct_root(const CtBatch &b, uint32_t x, unsigned long long &l)
 {
-    for (int n = 0; n < (1 << 20); ++n) {
-        const uint32_t p = (uint32_t)__ldcg(b.link + x);
-        if (p == x) break;
-        x = p;
+    l = __ldcg(b.link + x);
+#pragma unroll 1
+    for (int n = 0; n < (1 << 20) && !(l & kNodeRoot); ++n) {
+        x = (uint32_t)l;
+        l = __ldcg(b.link + x);
     }
     return x;
 }
 
 }  // namespace
 
-// Contraction of the nodes of the batch. Every warp owns the tiles [t0, t1),
-// with their nodes and the edges of their slots, which it keeps compacted at
-// the start of its range; so no list is shared. A round: (1) the edges find
-// their clusters and raise the clusters' best edges; (2) every open root
-// takes its decision. A grid barrier follows each. Roots that joined are
-// pointed at their new root, with the smallest weight on the way, at the
-// start of the next round's (1); readers that come first walk on.
-__global__ void __launch_bounds__(kGT, 4) ct_global_kernel(const __grid_constant__ CtBatch b, uint64_t timeout_ns)
+// Contraction of the nodes of the batch. The work is cut into units, four a
+// tile (a quarter of its nodes and forest, half a seam); every warp owns the
+// units [u0, u1) and keeps their nodes and edges compacted at the start of
+// their slots, so no list is shared. A round: (1) the edges find their
+// clusters and raise the clusters' best edges; (2) every open root takes its
+// decision. A grid barrier follows each. Roots that joined are pointed at
+// their new root, with the smallest weight on the way, at the start of the
+// next round's (1); readers that come first walk on. One CTA an SM: a
+// barrier's cost is its arrivals at one address. CLUSTER: the grid is one
+// cluster, and the barrier the hardware's.
+template <bool CLUSTER>
+__global__ void __launch_bounds__(kGT, 1) ct_global_kernel(const __grid_constant__ CtBatch b, uint64_t timeout_ns)
 {
+    auto barrier = [&]() -> bool {
+        if (CLUSTER) {
+            __threadfence();
+            asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+            return true;
+        }
+        return grid_barrier(b.ctl + kCtCtlBar, gridDim.x, b.err, timeout_ns);
+    };
     const int lane = threadIdx.x & 31;
     const int64_t gw = (int64_t)blockIdx.x * (kGT / 32) + (threadIdx.x >> 5), nw = (int64_t)gridDim.x * (kGT / 32);
-    const int t0 = (int)(gw * b.ntiles / nw), t1 = (int)((gw + 1) * b.ntiles / nw);
+    const int64_t units = (int64_t)b.ntiles * kCtUnits;
+    const int u0 = (int)(gw * units / nw), u1 = (int)((gw + 1) * units / nw);
     const uint32_t below = (1u << lane) - 1u;
-    const int64_t ebase = (int64_t)t0 * kCtEdges;
-    uint32_t *act = b.act + (int64_t)t0 * kCtNodes;
+    unsigned long long *edge = b.edge + (int64_t)u0 * kCtUnitEdges;
+    uint32_t *act = b.act + (int64_t)u0 * kCtUnitNodes;
     int ne = 0, na = 0;
     __shared__ uint32_t s_open;
 
@@ -617,93 +754,90 @@ __global__ void __launch_bounds__(kGT, 4) ct_global_kernel(const __grid_constant
         const uint32_t wm = __reduce_max_sync(peers, w);
         const bool lead = valid && lane == __ffs(peers) - 1;
         const uint32_t m = __ballot_sync(0xffffffffu, lead);
-        if (lead) {
-            const int64_t g = ebase + ne + __popc(m & below);
-            b.ea[g] = a;
-            b.eb[g] = c;
-            b.ew[g] = (uint8_t)wm;
-        }
+        if (lead) edge[ne + __popc(m & below)] = node_edge(a, c, wm);
         ne += __popc(m);
     };
-    for (int t = t0; t < t1; ++t) {
+#pragma unroll 1
+    for (int u = u0; u < u1; ++u) {
+        const int t = u / kCtUnits, part = u % kCtUnits;
         const CtImage &d = ct_image(b, t);
         const int lt = t - d.tile_base;
         const int ty = lt / d.nx, tx = lt - ty * d.nx;
         const uint32_t cn = __ldcg(b.cnt + t);
-        const int nn = (int)(cn & 0xffffu), nf = (int)(cn >> 16);
-        for (int i = lane; i < nn; i += 32) act[na + i] = (uint32_t)t * kCtNodes + i;
+        const int nn = ((int)(cn & 0xffffu) - part + kCtUnits - 1) / kCtUnits,
+                  nf = ((int)(cn >> 16) - part + kCtUnits - 1) / kCtUnits;
+#pragma unroll 1
+        for (int i = lane; i < nn; i += 32) act[na + i] = (uint32_t)(t * kCtNodes + part + i * kCtUnits);
         na += nn;
-        // the tile's forest moves up (never past its own slots)
+        // the unit's part of the forest moves up (never past its own slots)
+        const unsigned long long *from = b.edge + (int64_t)u * kCtUnitEdges;
+#pragma unroll 1
         for (int i = 0; i < nf; i += 32) {
-            const int64_t from = (int64_t)t * kCtEdges + i + lane, to = ebase + ne + i + lane;
-            uint32_t a = 0, c = 0;
-            uint8_t w = 0;
-            if (i + lane < nf) a = b.ea[from], c = b.eb[from], w = b.ew[from];
+            const unsigned long long e = i + lane < nf ? from[i + lane] : 0ull;
             __syncwarp();
-            if (i + lane < nf) b.ea[to] = a, b.eb[to] = c, b.ew[to] = w;
+            if (i + lane < nf) edge[ne + i + lane] = e;
             __syncwarp();
         }
         ne += nf;
-        // seams: keys order the pixels of a window by (I, raster order), 0 = outside
-        auto key = [&](int r, int c, uint32_t at) -> uint32_t {
-            if (r < 0 || r >= d.H || c < 0 || c >= d.W) return 0u;
-            return ((uint32_t)__ldg(d.mask + (int64_t)r * d.ld_mask + c) + 1u) << 4 | at;
-        };
-        auto weight = [&](uint32_t k1, uint32_t k2) { return (min(k1, k2) >> 4) - 1u; };
-        if (tx + 1 < d.nx) {
-            const int c = tx * kCtSide + kCtSide - 1;
-            for (int h = 0; h < kCtSide; h += 32) {
-                const int r = ty * kCtSide + h + lane;
-                const uint32_t u0 = key(r - 1, c, 0), u1 = key(r - 1, c + 1, 1), m0 = key(r, c, 2),
-                               m1 = key(r, c + 1, 3), d0 = key(r + 1, c, 4), d1 = key(r + 1, c + 1, 5);
-                const bool in = m0 && m1;
-                const bool s = in && max(m0, m1) > max(max(u0, u1), max(d0, d1));
-                emit(s, s ? ct_node(b, d, r, c) : 0u, s ? ct_node(b, d, r, c + 1) : 0u, s ? weight(m0, m1) : 0u);
-                const bool q = in && d0 && d1, main = max(m0, d1) > max(m1, d0);
-                emit(q, q ? ct_node(b, d, main ? r : r + 1, c) : 0u, q ? ct_node(b, d, main ? r + 1 : r, c + 1) : 0u,
-                     q ? (main ? weight(m0, d1) : weight(m1, d0)) : 0u);
+        // half a seam (parts 0, 1: the right one, 2, 3: the lower one): a lane
+        // takes the pixel m0 on this side, the one across m1, and the window
+        // of both and their next neighbours n0, n1; p0, p1 are their previous
+        // neighbours. Keys order the pixels by (I, raster order), 0 = outside.
+        const bool down = part >= 2;
+        const int i = (part & 1) * 32 + lane;
+        if (down ? ty + 1 < d.ny : tx + 1 < d.nx) {   // whole warp
+            const int r = ty * kCtSide + (down ? kCtSide - 1 : i), c = tx * kCtSide + (down ? i : kCtSide - 1);
+            auto key = [&](int along, int across) -> uint32_t {
+                const int y = r + (down ? across : along), x = c + (down ? along : across);
+                if (y < 0 || y >= d.H || x < 0 || x >= d.W) return 0u;
+                return ((uint32_t)__ldg(d.mask + (int64_t)y * d.ld_mask + x) + 1u) << 4 |
+                       (uint32_t)(down ? across * 3 + along + 1 : (along + 1) * 2 + across);
+            };
+            auto node = [&](int along, int across) {
+                return ct_node(b, d, r + (down ? across : along), c + (down ? along : across));
+            };
+            const uint32_t p0 = key(-1, 0), p1 = key(-1, 1), m0 = key(0, 0), m1 = key(0, 1), n0 = key(1, 0),
+                           n1 = key(1, 1);
+            const bool in = m0 && m1;
+            const bool s = in && max(m0, m1) > max(max(p0, p1), max(n0, n1));
+            // the window at the tile's corner belongs to the right seam
+            const bool q = in && n0 && n1 && !(down && i == kCtSide - 1), main = max(m0, n1) > max(m1, n0);
+            uint32_t a0 = 0, a1 = 0, c0 = 0, c1 = 0;
+            if (s || q) {
+                a0 = node(0, 0), a1 = node(0, 1);
+                if (q) c0 = node(1, 0), c1 = node(1, 1);
             }
-        }
-        if (ty + 1 < d.ny) {
-            const int r = ty * kCtSide + kCtSide - 1;
-            for (int h = 0; h < kCtSide; h += 32) {
-                const int c = tx * kCtSide + h + lane;
-                const uint32_t l0 = key(r, c - 1, 0), m0 = key(r, c, 1), r0 = key(r, c + 1, 2),
-                               l1 = key(r + 1, c - 1, 3), m1 = key(r + 1, c, 4), r1 = key(r + 1, c + 1, 5);
-                const bool in = m0 && m1;
-                const bool s = in && max(m0, m1) > max(max(l0, l1), max(r0, r1));
-                emit(s, s ? ct_node(b, d, r, c) : 0u, s ? ct_node(b, d, r + 1, c) : 0u, s ? weight(m0, m1) : 0u);
-                // the window at the tile's corner belongs to the right seam
-                const bool q = in && r0 && r1 && h + lane < kCtSide - 1, main = max(m0, r1) > max(m1, r0);
-                emit(q, q ? ct_node(b, d, r, main ? c : c + 1) : 0u, q ? ct_node(b, d, r + 1, main ? c + 1 : c) : 0u,
-                     q ? (main ? weight(m0, r1) : weight(m1, r0)) : 0u);
-            }
+            emit(s, a0, a1, s ? (min(m0, m1) >> 4) - 1u : 0u);
+            emit(q, main ? a0 : c0, main ? c1 : a1, q ? ((main ? min(m0, n1) : min(m1, n0)) >> 4) - 1u : 0u);
         }
         __syncwarp();
     }
 
+#pragma unroll 1
     for (int round = 0; round < kMaxRounds; ++round) {
         // (0) roots that joined: final links of the last round; the others stay open
         if (round > 0) {
             int kept = 0;
+#pragma unroll 1
             for (int i = 0; i < na; i += 32) {
                 bool open = false;
                 uint32_t r = 0;
                 if (i + lane < na) {
                     r = act[i + lane];
-                    const unsigned long long l = __ldcg(b.link + r);
-                    uint32_t x = (uint32_t)l;
-                    open = x == r;
+                    unsigned long long l = __ldcg(b.link + r);
+                    open = (l & kNodeRoot) != 0ull;
                     if (!open) {
-                        uint32_t w = (uint32_t)(l >> 32);
+                        uint32_t w = (uint32_t)(l >> 32), x = (uint32_t)l;
+#pragma unroll 1
                         for (int n = 0; n < (1 << 20); ++n) {
-                            const unsigned long long lx = __ldcg(b.link + x);
-                            if ((uint32_t)lx == x) break;
-                            w = min(w, (uint32_t)(lx >> 32));
-                            x = (uint32_t)lx;
+                            l = __ldcg(b.link + x);
+                            if (l & kNodeRoot) break;
+                            w = min(w, (uint32_t)(l >> 32));
+                            x = (uint32_t)l;
                         }
                         __stcg(b.link + r, (unsigned long long)w << 32 | x);
-                        atomicMax(b.S + x, __ldcg(b.S + r) & 0xffu);
+                        const uint32_t S = b.S[r];   // stored by this warp when it joined
+                        if (node_S(l) < S) atomicMax(b.link + x, kNodeRoot | (unsigned long long)S << 40 | x);
                     }
                 }
                 const uint32_t m = __ballot_sync(0xffffffffu, open);
@@ -715,32 +849,31 @@ __global__ void __launch_bounds__(kGT, 4) ct_global_kernel(const __grid_constant
         }
         // (1) edges; a key holds the round, so the last round's bests count as none
         int kept = 0;
+#pragma unroll 1
         for (int i = 0; i < ne; i += 32) {
             uint32_t a = 0, c = 0, w = 0;
-            bool keep = false, oa = false, oc = false;
+            bool keep = false, oa = true, oc = true;
             if (i + lane < ne) {
-                const int64_t g = ebase + i + lane;
-                a = b.ea[g];
-                c = b.eb[g];
-                w = b.ew[g];
+                const unsigned long long e = edge[i + lane];
+                a = (uint32_t)(e >> 28) & kNodeId;
+                c = (uint32_t)e & kNodeId;
+                w = (uint32_t)(e >> 56);
                 if (round > 0) {
-                    a = ct_root(b, a);
-                    c = ct_root(b, c);
-                    oa = !(__ldcg(b.S + a) & kDone);
-                    oc = !(__ldcg(b.S + c) & kDone);
-                } else {
-                    oa = oc = true;
+                    unsigned long long la, lc;
+                    a = ct_root(b, a, la);
+                    c = ct_root(b, c, lc);
+                    oa = !(la & kNodeDone);
+                    oc = !(lc & kNodeDone);
                 }
                 keep = a != c && (oa || oc);
             }
             const uint32_t m = __ballot_sync(0xffffffffu, keep);
             if (keep) {
-                const int64_t g = ebase + kept + __popc(m & below);
-                b.ea[g] = a;
-                b.eb[g] = c;
-                b.ew[g] = (uint8_t)w;
+                const int at = kept + __popc(m & below);
+                edge[at] = node_edge(a, c, w);
+                const uint32_t g = (uint32_t)u0 * kCtUnitEdges + at;
                 const unsigned long long k =
-                    (unsigned long long)(round + 1) << 48 | (unsigned long long)(w + 1u) << 32 | (uint32_t)g * kMix;
+                    (unsigned long long)(round + 1) << 48 | (unsigned long long)(w + 1u) << 32 | g * kMix;
                 if (oa && __ldcg(b.best + a) < k) atomicMax(b.best + a, k);
                 if (oc && __ldcg(b.best + c) < k) atomicMax(b.best + c, k);
             }
@@ -752,29 +885,38 @@ __global__ void __launch_bounds__(kGT, 4) ct_global_kernel(const __grid_constant
         uint32_t *open_cnt = b.ctl + kCtCtlOpen + round % 3;
         if (lane == 0 && na) atomicAdd(open_cnt, (uint32_t)na);
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(b.ctl + kCtCtlOpen + (round + 1) % 3, 0u);
-        if (!grid_barrier(b.ctl + kCtCtlBar, gridDim.x, b.err, timeout_ns)) return;
+        if (!barrier()) return;
         if (threadIdx.x == 0) s_open = ld_acquire(open_cnt);
         __syncthreads();
         if (s_open == 0u) return;
         // (2) decisions
         kept = 0;
+#pragma unroll 1
         for (int i = 0; i < na; i += 32) {
             bool open = false;
             uint32_t r = 0;
             if (i + lane < na) {
                 r = act[i + lane];
-                const unsigned long long k = __ldcg(b.best + r);
-                const uint32_t S = __ldcg(b.S + r) & 0xffu;
+                const unsigned long long k = __ldcg(b.best + r), l = __ldcg(b.link + r);
                 const bool some = (uint32_t)(k >> 48) == (uint32_t)(round + 1);
-                const uint32_t w = ((uint32_t)(k >> 32) & 0xffffu) - 1u;
+                const uint32_t w = ((uint32_t)(k >> 32) & 0xffffu) - 1u, S = node_S(l);
                 if (!some || S >= w) {
-                    atomicOr(b.S + r, kDone);
+                    atomicOr(b.link + r, kNodeDone);
                 } else {
                     open = true;
-                    const uint32_t g = (uint32_t)k * kUnmix;
-                    const uint32_t a = __ldcg(b.ea + g), c = __ldcg(b.eb + g), o = a == r ? c : a;
-                    const bool mutual = __ldcg(b.best + o) == k && (__ldcg(b.S + o) & 0xffu) < w;
-                    if (!(mutual && r < o)) __stcg(b.link + r, (unsigned long long)w << 32 | o);
+                    const unsigned long long e = __ldcg(b.edge + (uint32_t)k * kUnmix);
+                    const uint32_t a = (uint32_t)(e >> 28) & kNodeId, c = (uint32_t)e & kNodeId, o = a == r ? c : a;
+                    // o joins r by the same edge: the smaller of the two stays
+                    // (o may have joined already; its link word is no root's then)
+                    bool mutual = false;
+                    if (r < o && __ldcg(b.best + o) == k) {
+                        const unsigned long long lo = __ldcg(b.link + o);
+                        mutual = !(lo & kNodeRoot) || node_S(lo) < w;
+                    }
+                    if (!mutual) {
+                        b.S[r] = S;
+                        __stcg(b.link + r, (unsigned long long)w << 32 | o);
+                    }
                 }
             }
             const uint32_t m = __ballot_sync(0xffffffffu, open);
@@ -783,7 +925,7 @@ __global__ void __launch_bounds__(kGT, 4) ct_global_kernel(const __grid_constant
             __syncwarp();
         }
         na = kept;
-        if (!grid_barrier(b.ctl + kCtCtlBar, gridDim.x, b.err, timeout_ns)) return;
+        if (!barrier()) return;
     }
     raise_status(b.err, RT_ETIMEOUT);   // not reached: every round at least halves the open roots of a component
 }
@@ -799,14 +941,13 @@ __global__ void __launch_bounds__(256) ct_out_kernel(const __grid_constant__ CtB
     const int nn = (int)(b.cnt[tile] & 0xffffu);
     uint32_t v = 255u;
     if (t < nn) {
-        uint32_t x = (uint32_t)tile * kCtNodes + t;
-        for (int n = 0; n < (1 << 20); ++n) {
-            const unsigned long long l = b.link[x];
-            if ((uint32_t)l == x) break;
+        unsigned long long l = b.link[(uint32_t)tile * kCtNodes + t];
+#pragma unroll 1
+        for (int n = 0; n < (1 << 20) && !(l & kNodeRoot); ++n) {
             v = min(v, (uint32_t)(l >> 32));
-            x = (uint32_t)l;
+            l = b.link[(uint32_t)l];
         }
-        v = min(v, b.S[x] & 0xffu);
+        v = min(v, node_S(l));
     }
     val[t] = v;
     __syncthreads();
@@ -860,22 +1001,39 @@ void ct_plan_image(CtBatch &b, const uint8_t *marker, int64_t ld_marker, const u
 cudaError_t launch_contract(const CtBatch &b, int num_sms, uint64_t timeout_ns, cudaStream_t s)
 {
     const bool given = b.img[0].marker != nullptr;   // all images of a batch, or none
-    const void *fn = given ? (const void *)ct_local_kernel<true> : (const void *)ct_local_kernel<false>;
+    // With two tiles per SM or fewer little hides a tile's latency: then 512
+    // threads share it (512 x 512: 75 us against 87 for both stages, 1024 x
+    // 1024: 112 against 117; equal from 1536 x 1536 on, and above that the
+    // barriers of larger CTAs cost more: 247 us against 220 at 4096 x 4096).
+    const bool few = b.ntiles <= kFewTiles;
+    auto *fn = few ? (given ? ct_local_kernel<true, 512> : ct_local_kernel<false, 512>)
+                   : (given ? ct_local_kernel<true, 256> : ct_local_kernel<false, 256>);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalSmem);
     if (e != cudaSuccess) return e;
-    if (given) ct_local_kernel<true><<<(unsigned)b.ntiles, kT, kLocalSmem, s>>>(b);
-    else ct_local_kernel<false><<<(unsigned)b.ntiles, kT, kLocalSmem, s>>>(b);
+    fn<<<(unsigned)b.ntiles, few ? 512 : 256, kLocalSmem, s>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ct_global_kernel, kGT, 0);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    int grid = per_sm * num_sms;
-    const int need = (int)ceil_div(b.ntiles, kGT / 32);
-    if (grid > need) grid = need;
+    const int64_t units = (int64_t)b.ntiles * kCtUnits;
+    const int need = (int)ceil_div(units, kGT / 32);
+    // One cluster of eight CTAs while its 256 warps hold two units each at
+    // most (512 x 512: 90 us against 110 for both stages; 768 x 768: equal).
+    if (units <= kGClusterUnits) {
+        auto *gfn = ct_global_kernel<true>;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kGCluster);
+        cfg.blockDim = dim3(kGT);
+        cfg.stream = s;
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = kGCluster;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, gfn, b, timeout_ns);
+    }
     CtBatch bb = b;
     void *args[] = {&bb, &timeout_ns};
-    return cudaLaunchCooperativeKernel((const void *)ct_global_kernel, dim3((unsigned)grid), dim3(kGT), args, 0, s);
+    return cudaLaunchCooperativeKernel((const void *)ct_global_kernel<false>, dim3((unsigned)(need < num_sms ? need : num_sms)),
+                                       dim3(kGT), args, 0, s);
 }
 
 cudaError_t launch_contract_out(const CtBatch &b, int threshold, cudaStream_t s)

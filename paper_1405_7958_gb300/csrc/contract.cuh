@@ -12,12 +12,14 @@ constexpr int kCtPx = kCtSide * kCtSide;
 // rim, which has 252 pixels; slot 255 of a pixel's entry means "no node".
 constexpr int kCtNodes = 256;
 constexpr uint32_t kCtNoNode = 255u;
-// Edge slots per tile: at most 251 edges of the forest between its nodes,
-// and at most 257 across its right and lower seams (per seam one diagonal
-// for each of its 2 x 2 windows and one straight pair per pixel).
-constexpr int kCtEdges = 512;
+// The global stage's units: a quarter of a tile's nodes (at most 63) and of
+// the forest between them (at most 63 edges), and half of its right or lower
+// seam (at most 32 diagonals, one per 2 x 2 window, and 32 straight pairs).
+constexpr int kCtUnits = 4;
+constexpr int kCtUnitNodes = kCtNodes / kCtUnits;
+constexpr int kCtUnitEdges = 128;
 constexpr int kCtMaxImgs = 32;
-constexpr int64_t kCtMaxTiles = int64_t(1) << 23;   // edge slots are numbered in 32 bits
+constexpr int64_t kCtMaxTiles = int64_t(1) << 20;   // an edge names its nodes in 28 bits each
 
 struct CtImage {
     const uint8_t *marker;   // NULL: derived from the mask with h_offset
@@ -39,12 +41,11 @@ struct CtBatch {
     int n, ntiles;
     uint16_t *plane;         // per pixel (tile by tile): node of the tile << 8 | bound
     uint32_t *cnt;           // per tile: nodes | forest edges << 16
-    uint32_t *S;             // per node: best marker value that reaches it; bit 31: final
-    unsigned long long *link;   // per node: weight << 32 | parent (itself: a root)
+    unsigned long long *link;   // per node: its parent and link weight, or a root's state (contract.cu)
     unsigned long long *best;   // per node: its best edge of the round
+    uint32_t *S;             // per node that joined another: its sources' best value
     uint32_t *act;           // per node slot: the warps' lists of roots still open
-    uint32_t *ea, *eb;       // per edge slot: its nodes
-    uint8_t *ew;             //                its weight
+    unsigned long long *edge;   // per edge slot: weight and nodes
     uint32_t *ctl;           // kCtCtlWords control words, zeroed before the launches
     int32_t *err;            // device status word
     CtImage img[kCtMaxImgs];
