@@ -37,9 +37,9 @@
  *    calls. Calls on one context must be serialised by the caller (one
  *    stream at a time); use one context per concurrent stream.
  *  - Iterative steps are bounded: the reconstruction's propagation by a
- *    number of tile visits (max_iters, see rt_set_limits), and every
- *    propagation (reconstruction and hole filling) by device time (20 s
- *    unless set otherwise). A bound that is reached stops the step short of
+ *    number of tile visits (max_iters, see rt_set_limits) and by device time
+ *    (20 s unless set otherwise; hole filling joins components and has
+ *    nothing to bound). A bound that is reached stops the step short of
  *    its fixed point, reports RT_ETIMEOUT in the device status, and leaves
  *    the context usable for the next call.
  *  - Strides are in elements, not bytes (a reading of the boundary: every

@@ -6,15 +6,14 @@
 #include <new>
 #include <vector>
 
-#include "ccl.cuh"
 #include "common.cuh"
 #include "contract.cuh"
 #include "edt.cuh"
 #include "features.cuh"
-#include "fill.cuh"
 #include "mlp.cuh"
 #include "objects.cuh"
 #include "recon.cuh"
+#include "runs.cuh"
 #include "synth.cuh"
 
 using namespace rtk;
@@ -406,6 +405,22 @@ rt_status run_contract(rt_ctx *ctx, CtBatch &b, int32_t *err, cudaStream_t s, co
     return RT_OK;
 }
 
+// Workspace of the hole filling and labeling stages: the bits first, then
+// what no stage before them uses (carve_runs_late).
+void carve_bits(Carve &cv, RunBatch &b) { b.bits = cv.take<unsigned long long>((size_t)b.ntiles * kRunSide); }
+void carve_runs_late(Carve &cv, RunBatch &b, bool fill, bool label)
+{
+    const size_t nt = (size_t)b.ntiles, nodes = 1 + nt * kRunSlots;
+    b.sides = cv.take<uint8_t>(nt * kRunSides);
+    b.cnt = cv.take<uint8_t>(nt);
+    b.lcnt = cv.take<uint8_t>(nt);
+    b.outside = fill ? cv.take<uint32_t>(nodes) : nullptr;
+    b.U = label ? cv.take<uint32_t>(nodes) : nullptr;
+    b.A = label ? cv.take<uint32_t>(nodes) : nullptr;
+    b.M = label ? cv.take<uint32_t>(nodes) : nullptr;
+    b.words = cv.take<uint32_t>(nt * kRunWords);
+}
+
 void add_image(ReconBatch &b, const uint8_t *marker, int64_t ld_marker, const uint8_t *mask, int64_t ld_mask,
                int H, int W, int h_offset)
 {
@@ -465,9 +480,9 @@ bool bad_tile(const rt_tile &t)
 
 // Workspace of one chunk (up to kMaxImgs tiles) of rt_segment_batch. Every
 // stage runs once for the whole chunk, so every tile has its own buffers:
-// padded reconstruction copies, the binary image, the fill's bit planes, the
-// union-find arrays, the kept-pixel bit plane and the distance transform's
-// column masks.
+// the reconstruction's, the foreground bits, the component slots, the
+// kept-pixel bit plane and the distance transform's column masks.
+constexpr size_t kWsBytesPerPx = 13;
 struct Chunk {
     bool contract = false;   // reconstruction by contraction (cb), else by propagation (b, w)
     CtBatch cb;
@@ -477,9 +492,7 @@ struct Chunk {
     FeatBatch fb;
     float *feat = nullptr;
     int32_t *picks = nullptr;
-    FillBatch fill;
-    uint32_t *fill_flags = nullptr, *fill_pending = nullptr;
-    UfBatch uf;
+    RunBatch rb;
     EdtBitsBatch eb;
 };
 
@@ -524,33 +537,38 @@ void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, con
         c.feat = cv.take<float>((size_t)cn * kNumFeatures);
         c.picks = cv.take<int32_t>((size_t)cn);
     }
-    c.fill.n = 0;
-    c.uf.n = 0;
+    c.rb.n = c.rb.ntiles = 0;
+    c.rb.amin = P.min_area;
+    c.rb.amax = P.max_area;
     c.eb.n = 0;
-    int fill_tiles = 0;
+    size_t px = 0;
     for (int i = 0; i < cn; ++i) {
         const rt_tile &t = tiles[c0 + i];
-        const int H = t.H, W = t.W;
-        // B = (R < threshold); F replaces it in place unless the caller wants F
-        uint8_t *B = cv.take<uint8_t>((size_t)H * W);
-        auto outputs = [&](auto &d) {
+        RunImage &u = run_add(c.rb, t.H, t.W);
+        u.filled = t.filled;
+        u.ld_filled = t.ld_filled;
+        u.labels = t.labels;
+        u.ld_lab = t.ld_labels;
+        u.n_kept = t.n_kept;
+        px += (size_t)t.H * t.W;
+        if (c.contract) {   // B = (R < threshold) goes straight to the bits
+            c.cb.img[i].out = t.recon;
+            c.cb.img[i].ld_out = t.ld_recon;
+        } else {
+            uint8_t *B = cv.take<uint8_t>((size_t)t.H * t.W);
+            ReconImage &d = c.b.img[i];
             d.out = t.recon;
             d.ld_out = t.ld_recon;
             d.bin = B;
-            d.ld_bin = W;
-        };
-        if (c.contract) outputs(c.cb.img[i]);
-        else outputs(c.b.img[i]);
-        uint8_t *F = t.filled ? t.filled : B;
-        const int64_t ldF = t.filled ? t.ld_filled : W;
-        char *fws = cv.take<char>(fill_image_bytes(H, W));
-        if (real) fill_add(c.fill, B, W, F, ldF, H, W, fws);
-        fill_tiles += (int)(ceil_div(H, kFillTH) * ceil_div(W, kFillTW));
+            d.ld_bin = t.W;
+            u.in = B;
+            u.ld_in = t.W;
+        }
     }
-    c.fill_flags = cv.take<uint32_t>((size_t)fill_tiles);
-    c.fill_pending = cv.take<uint32_t>(1);
-    // The contraction's arrays are dead once R and B are written; the stages
-    // from the labeling on reuse their memory.
+    carve_bits(cv, c.rb);
+    c.cb.bits = c.contract ? c.rb.bits : nullptr;
+    // The contraction's arrays are dead once R and the bits are written; the
+    // later stages reuse their memory.
     size_t contract_end = 0;
     if (c.contract) {
         const size_t off = cv.off;
@@ -558,29 +576,41 @@ void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, con
         contract_end = cv.off;
         cv.off = off;
     }
+    carve_runs_late(cv, c.rb, true, true);
     for (int i = 0; i < cn; ++i) {
         const rt_tile &t = tiles[c0 + i];
-        const int H = t.H, W = t.W;
-        char *uws = cv.take<char>(uf_workspace_bytes(H, W));
-        uint32_t *kept = cv.take<uint32_t>((size_t)H * ceil_div(W, 32));
-        char *ews = cv.take<char>(edt_bits_workspace_bytes(H, W));
+        uint32_t *kept = cv.take<uint32_t>((size_t)t.H * ceil_div(t.W, 32));
+        char *ews = cv.take<char>(edt_bits_workspace_bytes(t.H, t.W));
         if (real) {
-            UfImage u;
-            std::memset(&u, 0, sizeof(u));
-            uf_carve(u, uws, H, W);
-            u.in = c.fill.img[i].out;
-            u.ld_in = c.fill.img[i].ld_out;
-            u.labels = t.labels;
-            u.ld_lab = t.ld_labels;
-            u.n_kept = t.n_kept;
-            u.fgbits = kept;
-            uf_add(c.uf, u);
-            edt_bits_add(c.eb, kept, H, W, t.d2, t.ld_d2, ews);
+            c.rb.img[i].kept = kept;
+            edt_bits_add(c.eb, kept, t.H, t.W, t.d2, t.ld_d2, ews);
         }
     }
     if (cv.off < contract_end) cv.off = contract_end;
-    c.uf.amin = P.min_area;
-    c.uf.amax = P.max_area;
+    // The figure callers size their budgets by has always been at least 13
+    // bytes per pixel, with the frontier queues on top; it stays so.
+    const size_t floor = kWsBytesPerPx * px + (c.contract || !c.w.fq_cap ? 0 : 8 * (size_t)c.w.fq_cap + 4 * kFqCtlWords);
+    if (cv.off < floor) cv.off = floor;
+}
+
+// Workspace bytes rt_segment_batch needs for these tiles (the largest chunk).
+size_t segment_ws_bytes(const rt_tile *tiles, int n, const rt_seg_params &P, bool learned, const rt_ctx *ctx)
+{
+    const Limits lim = seg_limits(ctx, P);
+    size_t most = 0;
+    for (int c0 = 0; c0 < n; c0 += kMaxImgs) {
+        const int cn = n - c0 < kMaxImgs ? n - c0 : kMaxImgs;
+        // A call that contracts fits where the same call with a bound on its
+        // propagation fits: a reservation serves both.
+        for (bool may_contract : {true, false}) {
+            Carve cv;
+            Chunk c;
+            layout_chunk(cv, c, tiles, c0, cn, P, learned, ctx, lim, may_contract);
+            most = cv.off > most ? cv.off : most;
+            if (!c.contract) break;
+        }
+    }
+    return most;
 }
 
 // The picker's features and network on a chunk, into its picks.
@@ -608,26 +638,6 @@ rt_status report_picks(rt_ctx *ctx, const int32_t *picks, int cn, cudaStream_t s
     if (ctx->picks_ev_valid) RT_CUDA_TRY(cudaEventRecord(ctx->picks_ev, s));
     ctx->n_last_picks = cn;
     return RT_OK;
-}
-
-// Workspace bytes rt_segment_batch needs for these tiles (the largest chunk).
-size_t segment_ws_bytes(const rt_tile *tiles, int n, const rt_seg_params &P, bool learned, const rt_ctx *ctx)
-{
-    const Limits lim = seg_limits(ctx, P);
-    size_t most = 0;
-    for (int c0 = 0; c0 < n; c0 += kMaxImgs) {
-        const int cn = n - c0 < kMaxImgs ? n - c0 : kMaxImgs;
-        // A call that contracts fits where the same call with a bound on its
-        // propagation fits: a reservation serves both.
-        for (bool may_contract : {true, false}) {
-            Carve cv;
-            Chunk c;
-            layout_chunk(cv, c, tiles, c0, cn, P, learned, ctx, lim, may_contract);
-            most = cv.off > most ? cv.off : most;
-            if (!c.contract) break;
-        }
-    }
-    return most;
 }
 
 }  // namespace
@@ -820,6 +830,7 @@ rt_status rt_reconstruct(rt_ctx *ctx, const uint8_t *marker, int64_t ld_marker, 
         ct_plan_image(cb, marker, ld_marker, mask, ld_mask, H, W, h_offset);
         cb.img[0].out = out;
         cb.img[0].ld_out = ld_out;
+        cb.bits = nullptr;
         int32_t *cerr = nullptr;
         rt_status cst = RT_OK;
         for (int pass = 0; pass < 2; ++pass) {   // size, then carve
@@ -871,34 +882,26 @@ rt_status rt_fill_holes(rt_ctx *ctx, const uint8_t *in, int64_t ld_in, uint8_t *
     if ((const void *)in == (const void *)out && ld_in != ld_out) return RT_EINVAL;
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
-    Carve cv;
-    auto layout = [&](Carve &c, char *&fws, uint32_t *&flags, uint32_t *&pend, int32_t *&err) {
-        fws = c.take<char>(fill_image_bytes(H, W));
-        flags = c.take<uint32_t>((size_t)(ceil_div(H, kFillTH) * ceil_div(W, kFillTW)));
-        pend = c.take<uint32_t>(1);
-        err = c.take<int32_t>(1);
-    };
-    char *fws;
-    uint32_t *flags, *pend;
-    int32_t *err;
-    layout(cv, fws, flags, pend, err);
-    rt_status st = ensure_ws(ctx, cv.off);
-    if (st != RT_OK) return st;
-    cv = Carve();
-    cv.base = (char *)ctx->ws;
-    layout(cv, fws, flags, pend, err);
+    RunBatch b;
+    b.n = b.ntiles = 0;
+    RunImage &u = run_add(b, H, W);
+    u.in = in;
+    u.ld_in = ld_in;
+    u.filled = out;
+    u.ld_filled = ld_out;
+    for (bool real : {false, true}) {   // size, then carve
+        Carve cv;
+        if (real) cv.base = (char *)ctx->ws;
+        carve_bits(cv, b);
+        carve_runs_late(cv, b, true, false);
+        rt_status st = RT_OK;
+        if (!real && (st = ensure_ws(ctx, cv.off)) != RT_OK) return st;
+    }
     if (dev_status) RT_CUDA_TRY(cudaMemsetAsync(dev_status, 0, sizeof(int32_t), s));
-    FillBatch fb;
-    fb.n = 0;
-    fill_add(fb, in, ld_in, out, ld_out, H, W, fws);
-    fb.conn = conn;
-    fb.flags = flags;
-    fb.pending = pend;
-    fb.err = dev_status ? dev_status : err;
-    fb.timeout_ns = ctx_limits(ctx).timeout_ns;
     Phase ph(ctx, RT_PHASE_FILL, s);
-    ctx->launches += 3;
-    return cuda_status(launch_fill(fb, ctx->num_sms, s));
+    ctx->launches += 4;
+    RT_CUDA_TRY(launch_run_pack(b, s));
+    return cuda_status(launch_run_fill(b, conn, 0, s));
 }
 
 rt_status rt_label_area(rt_ctx *ctx, const uint8_t *bin, int64_t ld_bin, int32_t *labels, int64_t ld_lab, int H,
@@ -910,25 +913,30 @@ rt_status rt_label_area(rt_ctx *ctx, const uint8_t *bin, int64_t ld_bin, int32_t
     if (overlaps(bin, span(H, ld_bin, 1, W), labels, span(H, ld_lab, 4, W))) return RT_EINVAL;
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
-    rt_status st = ensure_ws(ctx, uf_workspace_bytes(H, W));
-    if (st != RT_OK) return st;
-    UfImage u;
-    std::memset(&u, 0, sizeof(u));
-    uf_carve(u, (char *)ctx->ws, H, W);
+    RunBatch b;
+    b.n = b.ntiles = 0;
+    b.amin = min_area;
+    b.amax = max_area;
+    RunImage &u = run_add(b, H, W);
     u.in = bin;
     u.ld_in = ld_bin;
     u.labels = labels;
     u.ld_lab = ld_lab;
     u.n_kept = dev_n_kept;
-    UfBatch b;
-    b.n = 0;
-    uf_add(b, u);
-    b.amin = min_area;
-    b.amax = max_area;
+    for (bool real : {false, true}) {   // size, then carve
+        Carve cv;
+        if (real) cv.base = (char *)ctx->ws;
+        carve_bits(cv, b);
+        carve_runs_late(cv, b, false, true);
+        rt_status st = RT_OK;
+        if (!real && (st = ensure_ws(ctx, cv.off)) != RT_OK) return st;
+    }
     if (dev_status) RT_CUDA_TRY(cudaMemsetAsync(dev_status, 0, sizeof(int32_t), s));
     Phase ph(ctx, RT_PHASE_LABEL, s);
-    ctx->launches += 4;
-    return cuda_status(launch_label_batch(b, conn, s));
+    ctx->launches += 5;
+    RT_CUDA_TRY(launch_run_pack(b, s));
+    RT_CUDA_TRY(launch_run_local(b, conn, s));
+    return cuda_status(launch_run_label(b, conn, s));
 }
 
 rt_status rt_edt(rt_ctx *ctx, const uint8_t *fg, int64_t ld_fg, int32_t *d2, int64_t ld_d2, int H, int W,
@@ -1272,19 +1280,15 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
             RT_CUDA_TRY(c.contract ? launch_contract_out(c.cb, P.threshold, s) : launch_recon_out(c.b, P.threshold, s));
         }
         {
-            c.fill.conn = P.conn_fill;
-            c.fill.flags = c.fill_flags;
-            c.fill.pending = c.fill_pending;
-            c.fill.err = c.err;
-            c.fill.timeout_ns = lim.timeout_ns;
             Phase ph(ctx, RT_PHASE_FILL, s);
-            ctx->launches += 3;
-            RT_CUDA_TRY(launch_fill(c.fill, ctx->num_sms, s));
+            if (!c.contract) RT_CUDA_TRY(launch_run_pack(c.rb, s));
+            RT_CUDA_TRY(launch_run_fill(c.rb, P.conn_fill, 8, s));
+            ctx->launches += c.contract ? 3 : 4;
         }
         {
             Phase ph(ctx, RT_PHASE_LABEL, s);
-            ctx->launches += 4;
-            RT_CUDA_TRY(launch_label_batch(c.uf, 8, s));
+            ctx->launches += 3;
+            RT_CUDA_TRY(launch_run_label(c.rb, 8, s));
         }
         {
             Phase ph(ctx, RT_PHASE_EDT, s);

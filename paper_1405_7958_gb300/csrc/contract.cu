@@ -952,31 +952,29 @@ __global__ void __launch_bounds__(256) ct_out_kernel(const __grid_constant__ CtB
     val[t] = v;
     __syncthreads();
     const int r = ty * kCtSide + (t >> 2), c = tx * kCtSide + (t & 3) * 16;
-    const int n = min(16, d.W - c);
-    if (r >= d.H || n <= 0) return;
+    const int n = r < d.H ? min(16, d.W - c) : 0;   // may be negative: none
     const uint4 *src = reinterpret_cast<const uint4 *>(b.plane + (int64_t)tile * kCtPx + (t >> 2) * kCtSide + (t & 3) * 16);
     const uint4 s0 = __ldcs(src), s1 = __ldcs(src + 1);
     const uint32_t e[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-    uint32_t R[4] = {0, 0, 0, 0}, B[4] = {0, 0, 0, 0};
+    uint32_t R[4] = {0, 0, 0, 0}, B = 0;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
-        if (k >= n) break;   // entries past the image are not written
+        if (k >= n) break;   // nothing past the image
         const uint32_t x = (e[k >> 1] >> (16 * (k & 1))) & 0xffffu;
         const uint32_t p = min(x & 0xffu, val[x >> 8]);
         R[k >> 2] |= p << (8 * (k & 3));
-        B[k >> 2] |= (uint32_t)((int)p < threshold) << (8 * (k & 3));
+        B |= (uint32_t)((int)p < threshold) << k;
     }
-    auto store = [&](uint8_t *o, const uint32_t *w) {
-        if (n == 16 && ((uintptr_t)o & 15u) == 0) {
-            *reinterpret_cast<uint4 *>(o) = make_uint4(w[0], w[1], w[2], w[3]);
-        } else {
+    if (b.bits) reinterpret_cast<uint16_t *>(b.bits + (int64_t)tile * kCtSide)[t] = (uint16_t)B;
+    if (!d.out || n <= 0) return;
+    uint8_t *o = d.out + (int64_t)r * d.ld_out + c;
+    if (n == 16 && ((uintptr_t)o & 15u) == 0) {
+        *reinterpret_cast<uint4 *>(o) = make_uint4(R[0], R[1], R[2], R[3]);
+    } else {
 #pragma unroll
-            for (int k = 0; k < 16; ++k)
-                if (k < n) o[k] = (uint8_t)(w[k >> 2] >> (8 * (k & 3)));
-        }
-    };
-    if (d.out) store(d.out + (int64_t)r * d.ld_out + c, R);
-    if (d.bin) store(d.bin + (int64_t)r * d.ld_bin + c, B);
+        for (int k = 0; k < 16; ++k)
+            if (k < n) o[k] = (uint8_t)(R[k >> 2] >> (8 * (k & 3)));
+    }
 }
 
 void ct_plan_image(CtBatch &b, const uint8_t *marker, int64_t ld_marker, const uint8_t *mask, int64_t ld_mask, int H,
@@ -993,8 +991,8 @@ void ct_plan_image(CtBatch &b, const uint8_t *marker, int64_t ld_marker, const u
     d.ny = (int)ceil_div(H, kCtSide);
     d.tile_base = b.ntiles;
     d.h_offset = h_offset;
-    d.out = d.bin = nullptr;
-    d.ld_out = d.ld_bin = 0;
+    d.out = nullptr;
+    d.ld_out = 0;
     b.ntiles += d.nx * d.ny;
 }
 

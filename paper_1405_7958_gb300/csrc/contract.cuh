@@ -32,8 +32,6 @@ struct CtImage {
     int h_offset;
     uint8_t *out;            // nullable: R, H x W, stride ld_out
     int64_t ld_out;
-    uint8_t *bin;            // nullable: B = (R < threshold), H x W, stride ld_bin
-    int64_t ld_bin;
 };
 
 // Up to kCtMaxImgs images and the workspace of the batch, passed by value.
@@ -46,6 +44,7 @@ struct CtBatch {
     uint32_t *S;             // per node that joined another: its sources' best value
     uint32_t *act;           // per node slot: the warps' lists of roots still open
     unsigned long long *edge;   // per edge slot: weight and nodes
+    unsigned long long *bits;   // nullable: B = (R < threshold), per tile 64 rows, bit = column
     uint32_t *ctl;           // kCtCtlWords control words, zeroed before the launches
     int32_t *err;            // device status word
     CtImage img[kCtMaxImgs];
@@ -59,7 +58,7 @@ void ct_plan_image(CtBatch &b, const uint8_t *marker, int64_t ld_marker, const u
                    int W, int h_offset);
 // local contraction of every tile, then the global contraction (cooperative)
 cudaError_t launch_contract(const CtBatch &b, int num_sms, uint64_t timeout_ns, cudaStream_t s);
-// R and B = (R < threshold) into every image's out / bin (either may be NULL)
+// R into every image's out and B = (R < threshold) into bits (either may be NULL)
 cudaError_t launch_contract_out(const CtBatch &b, int threshold, cudaStream_t s);
 
 }  // namespace rtk
