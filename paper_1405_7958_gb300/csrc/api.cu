@@ -414,6 +414,7 @@ void carve_runs_late(Carve &cv, RunBatch &b, bool fill, bool label)
     b.sides = cv.take<uint8_t>(nt * kRunSides);
     b.cnt = cv.take<uint8_t>(nt);
     b.lcnt = cv.take<uint8_t>(nt);
+    b.kept = nullptr;
     b.outside = fill ? cv.take<uint32_t>(nodes) : nullptr;
     b.U = label ? cv.take<uint32_t>(nodes) : nullptr;
     b.A = label ? cv.take<uint32_t>(nodes) : nullptr;
@@ -478,6 +479,21 @@ bool bad_tile(const rt_tile &t)
     return false;
 }
 
+// Starts an EDT batch: takes its control words with the status word before
+// them (`words` in all, to be cleared), for images of `bands` bands of rows.
+int32_t *take_edt_ctl(Carve &cv, EdtBitsBatch &b, size_t bands, int &words)
+{
+    b.n = b.ntiles = b.nbands = b.maxW = 0;
+    words = (int)(6 + 2 * bands);
+    uint32_t *w = cv.take<uint32_t>((size_t)words);
+    b.err = reinterpret_cast<int32_t *>(w);
+    b.far_any = w ? w + 1 : nullptr;
+    b.has_bg = w ? w + 2 : nullptr;
+    b.bar = w ? w + 4 : nullptr;
+    b.far_rows = reinterpret_cast<unsigned long long *>(w ? w + 6 : nullptr);
+    return b.err;
+}
+
 // Workspace of one chunk (up to kMaxImgs tiles) of rt_segment_batch. Every
 // stage runs once for the whole chunk, so every tile has its own buffers:
 // the reconstruction's, the foreground bits, the component slots, the
@@ -488,7 +504,8 @@ struct Chunk {
     CtBatch cb;
     ReconBatch b;
     ReconWs w;
-    int32_t *err = nullptr;
+    int32_t *err = nullptr;   // first of the ctl_words words that a call clears
+    int ctl_words = 0;
     FeatBatch fb;
     float *feat = nullptr;
     int32_t *picks = nullptr;
@@ -502,7 +519,9 @@ void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, con
                   const rt_ctx *ctx, const Limits &lim, bool may_contract = true)
 {
     const bool real = cv.base != nullptr;
-    c.err = cv.take<int32_t>(1);
+    size_t bands = 0;
+    for (int i = 0; i < cn; ++i) bands += (size_t)ceil_div(tiles[c0 + i].H, kEdtSide);
+    c.err = take_edt_ctl(cv, c.eb, bands, c.ctl_words);
     c.cb.n = c.cb.ntiles = 0;
     for (int i = 0; i < cn; ++i) {
         const rt_tile &t = tiles[c0 + i];
@@ -540,7 +559,6 @@ void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, con
     c.rb.n = c.rb.ntiles = 0;
     c.rb.amin = P.min_area;
     c.rb.amax = P.max_area;
-    c.eb.n = 0;
     size_t px = 0;
     for (int i = 0; i < cn; ++i) {
         const rt_tile &t = tiles[c0 + i];
@@ -577,14 +595,12 @@ void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, con
         cv.off = off;
     }
     carve_runs_late(cv, c.rb, true, true);
+    c.rb.kept = cv.take<unsigned long long>((size_t)c.rb.ntiles * kRunSide);
+    c.eb.bits = c.rb.kept;
     for (int i = 0; i < cn; ++i) {
         const rt_tile &t = tiles[c0 + i];
-        uint32_t *kept = cv.take<uint32_t>((size_t)t.H * ceil_div(t.W, 32));
         char *ews = cv.take<char>(edt_bits_workspace_bytes(t.H, t.W));
-        if (real) {
-            c.rb.img[i].kept = kept;
-            edt_bits_add(c.eb, kept, t.H, t.W, t.d2, t.ld_d2, ews);
-        }
+        if (real) edt_bits_add(c.eb, t.H, t.W, t.d2, t.ld_d2, ews);
     }
     if (cv.off < contract_end) cv.off = contract_end;
     // The figure callers size their budgets by has always been at least 13
@@ -946,27 +962,33 @@ rt_status rt_edt(rt_ctx *ctx, const uint8_t *fg, int64_t ld_fg, int32_t *d2, int
     if (overlaps(fg, span(H, ld_fg, 1, W), d2, span(H, ld_d2, 4, W))) return RT_EINVAL;
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
-    Carve cv;
-    cv.take<char>(edt_workspace_bytes(H, W));
-    rt_status st = ensure_ws(ctx, cv.off + 1024);
-    if (st != RT_OK) return st;
-    cv = Carve();
-    cv.base = (char *)ctx->ws;
-    EdtArgs a;
-    a.fg8 = fg;
-    a.lab32 = nullptr;
-    a.ld_in = ld_fg;
-    a.H = H;
-    a.W = W;
-    a.d2 = d2;
-    a.ld_d2 = ld_d2;
-    a.g = cv.take<uint16_t>((size_t)H * W);
-    a.seg = cv.take<int32_t>((size_t)2 * ceil_div(H, 32) * W);
-    a.any_bg = cv.take<uint32_t>(1);
-    if (dev_status) RT_CUDA_TRY(cudaMemsetAsync(dev_status, 0, sizeof(int32_t), s));
+    RunBatch r;
+    r.n = r.ntiles = 0;
+    RunImage &u = run_add(r, H, W);
+    u.in = fg;
+    u.ld_in = ld_fg;
+    EdtBitsBatch b;
+    int words = 0;
+    for (bool real : {false, true}) {   // size, then carve
+        Carve cv;
+        if (real) cv.base = (char *)ctx->ws;
+        take_edt_ctl(cv, b, (size_t)ceil_div(H, kEdtSide), words);
+        carve_bits(cv, r);
+        char *ews = cv.take<char>(edt_bits_workspace_bytes(H, W));
+        rt_status st = RT_OK;
+        if (!real && (st = ensure_ws(ctx, cv.off)) != RT_OK) return st;
+        if (real) edt_bits_add(b, H, W, d2, ld_d2, ews);
+    }
+    b.bits = r.bits;
+    RT_CUDA_TRY(cudaMemsetAsync(b.err, 0, (size_t)words * 4, s));
+    if (dev_status) {
+        RT_CUDA_TRY(cudaMemsetAsync(dev_status, 0, sizeof(int32_t), s));
+        b.err = dev_status;
+    }
     Phase ph(ctx, RT_PHASE_EDT, s);
     ctx->launches += 3;
-    return cuda_status(launch_edt(a, s));
+    RT_CUDA_TRY(launch_run_pack(r, s));
+    return cuda_status(launch_edt_bits_batch(b, ctx->num_sms, ctx_limits(ctx).timeout_ns, s));
 }
 
 rt_status rt_watershed(rt_ctx *ctx, const int32_t *labels, int64_t ld_lab, const int32_t *d2, int64_t ld_d2, int H,
@@ -1241,7 +1263,7 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
         Carve cv;
         cv.base = (char *)ctx->ws;
         layout_chunk(cv, c, tiles, c0, cn, P, learned, ctx, lim);
-        RT_CUDA_TRY(zero_words(c.err, 1, s));
+        RT_CUDA_TRY(zero_words(c.err, c.ctl_words, s));
         ctx->launches += 1;
         auto reconstruct = [&](const int32_t *pick) {
             return c.contract ? run_contract(ctx, c.cb, c.err, s, lim)
@@ -1292,8 +1314,8 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
         }
         {
             Phase ph(ctx, RT_PHASE_EDT, s);
-            ctx->launches += 3;
-            RT_CUDA_TRY(launch_edt_bits_batch(c.eb, s));
+            ctx->launches += 2;
+            RT_CUDA_TRY(launch_edt_bits_batch(c.eb, ctx->num_sms, lim.timeout_ns, s));
         }
         if (aside) {   // enqueued last: its launches delay none of the chain's
             RT_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork, 0));

@@ -276,8 +276,9 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
     const int nr = s_roots;
 
     // ---- every pixel's cluster: four steps uphill without a test (nearly
-    // always enough), then until a root. Parents are replaced by what was
-    // found, which shortens the long walks of flat images.
+    // always enough), then until a root or a pixel that has found its own.
+    // Parents are replaced by what was found, which shortens the long walks
+    // of flat images.
     {
         bool bad = false;
 #pragma unroll 2
@@ -288,7 +289,6 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
             uint32_t x[2] = {pp & 0xfffu, (pp >> 16) & 0xfffu}, v[2], own[2] = {ow.x, ow.y};
 #pragma unroll
             for (int n = 0; n < 3; ++n) x[0] = P[x[0]] & 0xfffu, x[1] = P[x[1]] & 0xfffu;
-            reinterpret_cast<volatile uint32_t *>(P)[at / 2] = (pp & 0xf000f000u) | x[0] | x[1] << 16;
             v[0] = VW[x[0]], v[1] = VW[x[1]];
 #pragma unroll
             for (int q = 0; q < 2; ++q)
@@ -297,6 +297,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
                     x[q] = P[x[q]] & 0xfffu;
                     v[q] = VW[x[q]];
                 }
+            reinterpret_cast<volatile uint32_t *>(P)[at / 2] = (pp & 0xf000f000u) | x[0] | x[1] << 16;
             uint2 nw = ow;
             if (ow.x) nw.x = ow.x | (v[0] & kLabel);
             if (ow.y) nw.y = ow.y | (v[1] & kLabel);

@@ -67,7 +67,6 @@ extern "C" rt_status rt_edt_noalloc(const uint8_t *fg, int64_t ld_fg, int32_t *d
     cudaStream_t s = (cudaStream_t)stream;
     rtk::EdtArgs a;
     a.fg8 = fg;
-    a.lab32 = nullptr;
     a.ld_in = ld_fg;
     a.H = H;
     a.W = W;

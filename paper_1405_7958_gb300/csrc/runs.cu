@@ -729,17 +729,8 @@ __global__ void __launch_bounds__(kWarps * 32) run_label_kernel(const __grid_con
             store(i, v[0], v[1]);
         }
     }
-    if (d.kept && i0 == 0) {   // 32-bit words of the rows
-        const int wpr = (d.W + 31) / 32, w0 = 2 * p.tx;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int r = p.r0 + 2 * lane + j;
-            if (r >= d.H) continue;
-            uint32_t *o = d.kept + (int64_t)r * wpr + w0;
-            o[0] = (uint32_t)keep[j];
-            if (w0 + 1 < wpr) o[1] = (uint32_t)(keep[j] >> 32);
-        }
-    }
+    if (b.kept && i0 == 0)
+        *(reinterpret_cast<ulonglong2 *>(b.kept + (int64_t)tile * kRunSide) + lane) = make_ulonglong2(keep[0], keep[1]);
 }
 
 // --------------------------------------------------------------------- host

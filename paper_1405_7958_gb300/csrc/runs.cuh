@@ -24,7 +24,6 @@ struct RunImage {
     int32_t *labels;       // stride ld_lab
     int64_t ld_lab;
     int32_t *n_kept;       // nullable: number of components kept (zeroed by the local stage)
-    uint32_t *kept;        // nullable: kept pixels as a bit plane, ceil(W / 32) words per row
 };
 
 // Up to kRunMaxImgs images and the batch's workspace, passed by value.
@@ -32,6 +31,7 @@ struct RunBatch {
     int n, ntiles;
     int32_t amin, amax;              // area range kept, inclusive
     unsigned long long *bits;        // per tile: 64 rows, bit = column; foreground
+    unsigned long long *kept;        // nullable: the kept pixels, in the same layout
     uint8_t *sides;                  // per tile: slot (255: none) of the top, bottom, left, right pixels
     uint8_t *cnt;                    // per tile: slots of the fill's background components
     uint32_t *outside;               // forest over 1 + tile * kRunSlots + slot; 0 = outside
