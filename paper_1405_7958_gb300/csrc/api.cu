@@ -6,6 +6,7 @@
 #include <new>
 #include <vector>
 
+#include "ccl.cuh"
 #include "common.cuh"
 #include "contract.cuh"
 #include "edt.cuh"
@@ -695,10 +696,7 @@ rt_status rt_create(rt_ctx **ctx, int device, size_t workspace_bytes)
     if (cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         cudaHostAlloc((void **)&c->picks_host, kMaxImgs * sizeof(int32_t), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer((void **)&c->picks_mapped, c->picks_host, 0) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->picks_ev, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaEventCreateWithFlags(&c->picks_ev, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         free_host_side(c);
         delete c;
@@ -929,6 +927,27 @@ rt_status rt_label_area(rt_ctx *ctx, const uint8_t *bin, int64_t ld_bin, int32_t
     if (overlaps(bin, span(H, ld_bin, 1, W), labels, span(H, ld_lab, 4, W))) return RT_EINVAL;
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
+    if ((int64_t)run_tiles(H, W) <= kUfMaxTiles) {
+        rt_status st = ensure_ws(ctx, uf_workspace_bytes(H, W));
+        if (st != RT_OK) return st;
+        UfImage u;
+        std::memset(&u, 0, sizeof(u));
+        uf_carve(u, (char *)ctx->ws, H, W);
+        u.in = bin;
+        u.ld_in = ld_bin;
+        u.labels = labels;
+        u.ld_lab = ld_lab;
+        u.n_kept = dev_n_kept;
+        UfBatch b;
+        b.n = 0;
+        uf_add(b, u);
+        b.amin = min_area;
+        b.amax = max_area;
+        if (dev_status) RT_CUDA_TRY(cudaMemsetAsync(dev_status, 0, sizeof(int32_t), s));
+        Phase ph(ctx, RT_PHASE_LABEL, s);
+        ctx->launches += 4;
+        return cuda_status(launch_label_batch(b, conn, s));
+    }
     RunBatch b;
     b.n = b.ntiles = 0;
     b.amin = min_area;
@@ -1218,6 +1237,15 @@ int rt_last_picks(const rt_ctx *ctx, int *classes, int cap)
 rt_status rt_set_picker(rt_ctx *ctx, const uint16_t *wb, const float *norm)
 {
     if (!ctx || (!wb) != (!norm)) return RT_EINVAL;
+    if (wb && !ctx->side) {   // a learned call may run the picker beside the chain
+        DeviceGuard g(ctx->device);
+        if ((!ctx->fork && cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) != cudaSuccess) ||
+            (!ctx->join && cudaEventCreateWithFlags(&ctx->join, cudaEventDisableTiming) != cudaSuccess) ||
+            cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            return RT_ECUDA;
+        }
+    }
     ctx->picker_wb = wb;
     ctx->picker_norm = norm;
     return RT_OK;

@@ -1,4 +1,5 @@
-"""GPU tests of hole filling and labeling on runs of bit rows: sizes around
+"""GPU tests of hole filling and labeling on runs of bit rows (and of the pixel
+union-find that labels small images): sizes around
 their 64 x 64 tiles, both connectivities, images with the most runs and pairs
 a tile can hold, holes and components across many tiles, against the CPU
 oracle (whole numbers: no tolerance)."""
@@ -44,6 +45,18 @@ def masks(H, W):
     return {k: np.asarray(v).astype(np.uint8) for k, v in out.items()}
 
 
+def test_chain_labels_of_dense_masks(rt):
+    """The chain labels bit planes at every size: masks with the most runs,
+    thresholded from two grey values (dark = foreground)."""
+    for H, W in ((1, 130), (64, 65), (191, 193)):
+        for name, m in masks(H, W).items():
+            I = np.where(m > 0, 20, 220).astype(np.uint8)
+            out = rt.segment_batch([dev(I)], rt.SegParams(min_area=2, max_area=10 ** 6))[0]
+            want = oracle.chain(I, min_area=2, max_area=10 ** 6)
+            for k in ("F", "L", "D"):
+                assert np.array_equal(host(out[k]), want[k]), (name, k)
+
+
 @pytest.mark.parametrize("conn", [4, 8])
 @pytest.mark.parametrize("H,W", SIZES)
 def test_fill_and_label_equal_the_oracle(rt, H, W, conn):
@@ -76,9 +89,11 @@ def test_unaligned_views(rt):
 def test_many_tiles(rt):
     """Thousands of tiles: one background and one component across all of
     them, and the tiles' order must not matter."""
-    r, c = np.mgrid[0:3000, 0:3100]
+    r, c = np.mgrid[0:3000, 0:3301]
     grid = ((r % 97 < 2) | (c % 89 < 2)).astype(np.uint8)          # meshes: every cell a hole
     grid[1500:, 1550] = 0                                            # some of them open
-    for m in (grid, 1 - grid, synth.random_binary(3000, 3100, 8, 420)):
+    for m in (grid, 1 - grid, synth.random_binary(3000, 3301, 8, 420)):
         assert np.array_equal(host(rt.fill_holes(dev(m))), oracle.fill_holes(m, 4))
-        assert np.array_equal(host(rt.label_area(dev(m), 0, 2 ** 31 - 1)), oracle.label_area(m, 0, 2 ** 31 - 1, 8))
+        for conn in (4, 8):   # large enough for the union-find over runs
+            got = host(rt.label_area(dev(m), 2, 2 ** 31 - 1, conn=conn))
+            assert np.array_equal(got, oracle.label_area(m, 2, 2 ** 31 - 1, conn)), conn
