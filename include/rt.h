@@ -255,7 +255,7 @@ RT_API rt_status rt_recon_stats(rt_ctx *ctx, int64_t *visits, int64_t *iteration
  * d2: int32 H x W (ld_d2). h >= 0. basins: int32 H x W (ld_b), the basin
  * label of every object pixel, -1 elsewhere; must not overlap the inputs.
  * dev_n_basins (device int32, nullable) receives the number of markers.
- * The workspace holds about 37 bytes per pixel.
+ * The workspace holds about 41 bytes per pixel.
  */
 RT_API rt_status rt_watershed(rt_ctx *ctx, const int32_t *labels, int64_t ld_lab, const int32_t *d2,
                               int64_t ld_d2, int H, int W, int h, int32_t *basins, int64_t ld_b,
@@ -264,11 +264,11 @@ RT_API rt_status rt_watershed(rt_ctx *ctx, const int32_t *labels, int64_t ld_lab
 /*
  * Feature computation stage (Section 5.1): per object of `labels` (as for
  * rt_watershed), over the intensities `img`, RT_NOBJFEAT features, computed
- * as the paper organises it: one thread block per object's minimum bounding
+ * as the paper organises it: one group of threads per object's minimum bounding
  * box accumulates the intermediate results (pixel count, perimeter,
  * coordinate and intensity moments, the 256-bin histogram, the 8-level
- * co-occurrence matrix of horizontally adjacent pixels), then one thread
- * per object computes the features. In order: area; perimeter (pixel edges
+ * co-occurrence matrix of horizontally adjacent pixels), then a few threads
+ * per object compute the features. In order: area; perimeter (pixel edges
  * between the object and a 4-neighbour outside it, the image border
  * included); bounding box height, width; centroid row, column; major and
  * minor axis 4 sqrt(l1), 4 sqrt(l2) (l1 >= l2 >= 0 the eigenvalues of the
@@ -282,7 +282,7 @@ RT_API rt_status rt_watershed(rt_ctx *ctx, const int32_t *labels, int64_t ld_lab
  * obj_labels: int32[cap], feat: double[cap][RT_NOBJFEAT], both device,
  * written for the first min(cap, number of objects) objects in increasing
  * label order; dev_n_obj (device int32, nullable) receives the number of
- * objects. The workspace holds about 28 bytes per pixel plus 1.4 KB per
+ * objects. The workspace holds about 28 bytes per pixel plus 128 bytes per
  * output slot.
  */
 #define RT_NOBJFEAT 20

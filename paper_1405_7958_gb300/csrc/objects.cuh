@@ -11,12 +11,15 @@ constexpr int kObjFeat = 20;         // features per object
 constexpr int kObjChunk = 1024;      // pixels per enumeration chunk (raster order)
 constexpr int kWsSmemPx = 4096;      // largest bounding box a watershed block holds in shared memory
 
-// Per-object intermediate results of the feature computation (one block
-// per object writes them, one thread per object turns them into features).
+// Per-object intermediate results of the feature computation (one group of
+// threads per object writes them, one thread per object turns them into
+// features): moments, co-occurrence sums (hom over 840) and what is taken
+// from the histogram.
 struct ObjInter {
     int64_t area, per, sr, sc, srr, scc, src, si, sii;
-    uint32_t hist[256];
-    uint32_t glcm[64];
+    int64_t n2, con, en, hom;
+    double ent;
+    int32_t vmin, vmax, med;
 };
 
 struct ObjArgs {
@@ -28,15 +31,14 @@ struct ObjArgs {
     int64_t ld_D;
     int H, W;
     // workspace
-    uint32_t *chunk_cnt;   // per chunk: objects whose first pixel lies in it, then their prefix sum
-    uint32_t *ctl;         // [0] objects, [1] next object of the per-object blocks, [2] basins,
-                           // [3] objects with a large box, [4] the others (watershed)
-    int32_t *order;        // watershed: objects by box size class (large first from the front, small
-                           // from the back)
-    int32_t *idx_of;       // per pixel index (sparse): object index of the label it is the first pixel of
-    int32_t *olabel;       // per object: label
-    int32_t *box;          // per object: r0, c0, r1, c1
-    int64_t max_obj;       // capacity of olabel / box
+    uint32_t *chunk_cnt;   // per chunk: its records, and << 16 the objects whose first pixel lies in it
+    uint32_t *block_cnt;   // per block of the scan: the objects of its chunks
+    uint32_t *ctl;         // [0] objects, [1] next and [3] number of the large ones, [4] and [5] next
+                           // object for the warps of the medium and the small boxes (watershed)
+    uint2 *rec;            // per chunk, kObjChunk slots: label; offset in the chunk, length - 1 << 16
+    int32_t *big;          // objects left to the blocks (large boxes); where the records were
+    int32_t *olabel;       // per object: label, increasing
+    int32_t *box;          // per label (sparse): r0, c0, r1, c1
     ObjInter *inter;       // per written object (features)
     int32_t *R;            // watershed, image-sized (stride W): large objects' working copies
     unsigned long long *st;
