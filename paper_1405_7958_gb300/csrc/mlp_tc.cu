@@ -1,15 +1,22 @@
 // The picker network's forward pass on the 5th-generation tensor cores
 // (tcgen05), for training batches.
 //
-// One CTA of 128 threads takes 128 samples: the M = 128 rows of three
+// One CTA of 256 threads takes 128 samples: the M = 128 rows of three
 // products whose accumulators live in tensor memory,
 //   H1 = Xn W1^T (K = 24, padded to 32),  H2 = relu(H1 + b1) W2^T (K = 64),
 //   Z  = relu(H2 + b2) W3^T (N = 3, padded to 16),
 // with bf16 operands (the parameters are bf16 already; the normalised input
 // and the two hidden layers are rounded to bf16 to enter a product) and fp32
-// accumulation. Thread t owns sample t: it writes row t of each A operand
-// and reads row t (tensor-memory lane t) of each accumulator. One thread
-// issues the products; their completion arrives on an mbarrier.
+// accumulation. Threads t and t + 128 own sample t: each writes one half of
+// the columns of row t of an A operand and reads that half of row t
+// (tensor-memory lane t) of an accumulator. One thread issues the products;
+// their completion arrives on an mbarrier. The products are a few hundred
+// cycles: what counts is the latency of the chain and the number of memory
+// instructions around them, so global and shared memory are accessed 16
+// bytes at a time (VEC: the pointers are 16-byte aligned; else 2 or 4 bytes),
+// the input by all threads in order, and the samples' columns are halved
+// between two threads. Batch of 256: forward 9 us, backward 10 (a thread
+// per sample, 2- and 4-byte accesses a row apart: 30 and 34).
 //
 // Operands sit in shared memory in the no-swizzle K-major layout of 8-row x
 // 16-byte core matrices: element (r, k) of a K-wide operand is at
@@ -24,6 +31,7 @@ namespace rtk {
 namespace {
 
 constexpr int kTcM = 128;       // samples per CTA = tensor-memory lanes
+constexpr int kTcThreads = 2 * kTcM;
 constexpr int kK1 = 32;         // layer 1 K: 24 inputs, zero-padded
 constexpr int kN3 = 16;         // layer 3 N: 3 outputs, zero-padded
 constexpr int kTmemCols = 256;  // H1 at columns 0..63, H2 at 64..127, Z at 128..143
@@ -115,34 +123,86 @@ __device__ __forceinline__ void tc_after_sync() { asm volatile("tcgen05.fence::a
 
 __device__ __forceinline__ uint16_t to_bf16(float f) { return __bfloat16_as_ushort(__float2bfloat16_rn(f)); }
 
-// ReLU(acc + bias) of 64 accumulator columns starting at `col`: saved in fp32
-// (act) and written as this thread's bf16 row of the next A operand
-__device__ __forceinline__ void hidden_row(uint32_t tbase, int col, const uint16_t *wb, int bias, uint8_t *A, int row,
+__device__ __forceinline__ uint32_t two_bf16(float a, float b)
+{
+    return (uint32_t)to_bf16(a) | ((uint32_t)to_bf16(b) << 16);
+}
+
+__device__ __forceinline__ float of_bf16(uint16_t u) { return __uint_as_float((uint32_t)u << 16); }
+
+template <bool VEC>
+__device__ __forceinline__ void load4(const float *p, float *v)
+{
+    if (VEC) {
+        const float4 q = *reinterpret_cast<const float4 *>(p);
+        v[0] = q.x;
+        v[1] = q.y;
+        v[2] = q.z;
+        v[3] = q.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = p[i];
+    }
+}
+
+template <bool VEC>
+__device__ __forceinline__ void store4(float *p, const float *v)
+{
+    if (VEC) {
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p[i] = v[i];
+    }
+}
+
+// 8 consecutive bf16 parameters, one row of a core matrix
+template <bool VEC>
+__device__ __forceinline__ uint4 load_w8(const uint16_t *p)
+{
+    if (VEC) return *reinterpret_cast<const uint4 *>(p);
+    uint32_t u[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) u[i] = (uint32_t)p[2 * i] | ((uint32_t)p[2 * i + 1] << 16);
+    return make_uint4(u[0], u[1], u[2], u[3]);
+}
+
+// ReLU(acc + bias) of the 32 accumulator columns from `col` of this thread's
+// lane, the columns j0 .. j0 + 31 of the hidden layer: saved in fp32 (act)
+// and written to row `row` of the next A operand
+template <bool VEC>
+__device__ __forceinline__ void hidden_row(uint32_t tbase, int col, const float *bias, uint8_t *A, int row, int j0,
                                            float *act_row)
 {
 #pragma unroll
-    for (int q = 0; q < kMlpH / 16; ++q) {
+    for (int q = 0; q < 2; ++q) {
         float v[16];
-        tmem_ld16(tbase + (uint32_t)(col + 16 * q), v);
+        tmem_ld16(tbase + (uint32_t)(col + j0 + 16 * q), v);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int j = 16 * q + i;
-            const float h = fmaxf(v[i] + __uint_as_float((uint32_t)wb[bias + j] << 16), 0.f);
-            if (act_row) act_row[j] = h;
-            *reinterpret_cast<uint16_t *>(A + core_off(row, j, kMlpH)) = to_bf16(h);
+        for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i] + bias[j0 + 16 * q + i], 0.f);
+#pragma unroll
+        for (int i = 0; i < 16; i += 8)
+            *reinterpret_cast<uint4 *>(A + core_off(row, j0 + 16 * q + i, kMlpH)) =
+                make_uint4(two_bf16(v[i], v[i + 1]), two_bf16(v[i + 2], v[i + 3]), two_bf16(v[i + 4], v[i + 5]),
+                           two_bf16(v[i + 6], v[i + 7]));
+        if (act_row) {
+#pragma unroll
+            for (int i = 0; i < 16; i += 4) store4<VEC>(act_row + j0 + 16 * q + i, v + i);
         }
     }
 }
 
-__global__ void __launch_bounds__(kTcM) mlp_forward_tc_kernel(const uint16_t *wb, const float *norm, const float *x,
+template <bool VEC>
+__global__ void __launch_bounds__(kTcThreads) mlp_forward_tc_kernel(const uint16_t *wb, const float *norm, const float *x,
                                                               int B, float *logits, float *act, int32_t *pick,
                                                               float min_prob, int fallback, int32_t *err)
 {
     __shared__ __align__(1024) uint8_t sm[kTcSmem];
     __shared__ __align__(8) uint64_t mbar_store;
     __shared__ uint32_t tmem_base;
-    const int t = threadIdx.x, warp = t >> 5;
-    const int b = blockIdx.x * kTcM + t;
+    __shared__ __align__(16) float bias[2 * kMlpH + kMlpOut];
+    const int t = threadIdx.x, warp = t >> 5, row = t & (kTcM - 1), j0 = (t / kTcM) * (kMlpH / 2);
+    const int b = blockIdx.x * kTcM + row;
     const bool live = b < B;
     uint8_t *A = sm + kOffA;
     const uint32_t mbar = smem_u32(&mbar_store);
@@ -157,32 +217,45 @@ __global__ void __launch_bounds__(kTcM) mlp_forward_tc_kernel(const uint16_t *wb
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // B operands (the parameters, zero-padded) and this thread's row of the
-    // layer-1 A operand (the normalised input, zero-padded)
-    for (int i = t; i < kMlpH * kK1; i += kTcM) {
-        const int n = i / kK1, k = i % kK1;
-        *reinterpret_cast<uint16_t *>(sm + kOffB1 + core_off(n, k, kK1)) = k < kMlpIn ? wb[kW1 + n * kMlpIn + k] : 0;
-    }
-    for (int i = t; i < kMlpH * kMlpH; i += kTcM) {
-        const int n = i / kMlpH, k = i % kMlpH;
-        *reinterpret_cast<uint16_t *>(sm + kOffB2 + core_off(n, k, kMlpH)) = wb[kW2 + n * kMlpH + k];
-    }
-    for (int i = t; i < kN3 * kMlpH; i += kTcM) {
-        const int n = i / kMlpH, k = i % kMlpH;
-        *reinterpret_cast<uint16_t *>(sm + kOffB3 + core_off(n, k, kMlpH)) = n < kMlpOut ? wb[kW3 + n * kMlpH + k] : 0;
+    // B operands (the parameters, zero-padded), the biases, and the layer-1 A
+    // operand (the normalised input, zero-padded)
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int i = t; i < kMlpH * kK1 / 8; i += kTcThreads) {
+        const int n = i / (kK1 / 8), k = 8 * (i % (kK1 / 8));
+        *reinterpret_cast<uint4 *>(sm + kOffB1 + core_off(n, k, kK1)) =
+            k < kMlpIn ? load_w8<VEC>(wb + kW1 + n * kMlpIn + k) : zero;
     }
 #pragma unroll
-    for (int k = 0; k < kK1; ++k) {
-        float v = 0.f;
-        if (live && k < kMlpIn) v = (x[(int64_t)b * kMlpIn + k] - norm[k]) / norm[kMlpIn + k];
-        *reinterpret_cast<uint16_t *>(A + core_off(t, k, kK1)) = to_bf16(v);
+    for (int i = t; i < kMlpH * kMlpH / 8; i += kTcThreads) {
+        const int n = i / (kMlpH / 8), k = 8 * (i % (kMlpH / 8));
+        *reinterpret_cast<uint4 *>(sm + kOffB2 + core_off(n, k, kMlpH)) = load_w8<VEC>(wb + kW2 + n * kMlpH + k);
     }
+    if (t < kN3 * kMlpH / 8) {
+        const int n = t / (kMlpH / 8), k = 8 * (t % (kMlpH / 8));
+        *reinterpret_cast<uint4 *>(sm + kOffB3 + core_off(n, k, kMlpH)) =
+            n < kMlpOut ? load_w8<VEC>(wb + kW3 + n * kMlpH + k) : zero;
+    }
+    if (t < 2 * kMlpH + kMlpOut)
+        bias[t] = of_bf16(wb[t < kMlpH ? kB1 + t : t < 2 * kMlpH ? kB2 + t - kMlpH : kB3 + t - 2 * kMlpH]);
+#pragma unroll
+    for (int u = 0; u < kTcM * kMlpIn / 4 / kTcThreads; ++u) {
+        const int i = t + kTcThreads * u, r = i / (kMlpIn / 4), k = 4 * (i % (kMlpIn / 4));
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        if (blockIdx.x * kTcM + r < B) {
+            load4<VEC>(x + (int64_t)blockIdx.x * kTcM * kMlpIn + 4 * i, v);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = (v[e] - norm[k + e]) / norm[kMlpIn + k + e];
+        }
+        *reinterpret_cast<uint2 *>(A + core_off(r, k, kK1)) = make_uint2(two_bf16(v[0], v[1]), two_bf16(v[2], v[3]));
+    }
+    if (t < kTcM) *reinterpret_cast<uint4 *>(A + core_off(t, kMlpIn, kK1)) = zero;
     fence_async_smem();
     tc_before_sync();
     __syncthreads();
     tc_after_sync();
     const uint32_t tmem = tmem_base;
-    const uint32_t tlane = tmem + ((uint32_t)(32 * warp) << 16);   // this warp's 32 lanes
+    const uint32_t tlane = tmem + ((uint32_t)(32 * (warp & 3)) << 16);   // this warp's 32 lanes
     const uint32_t aaddr = smem_u32(A);
     bool ok = true;
 
@@ -195,7 +268,7 @@ __global__ void __launch_bounds__(kTcM) mlp_forward_tc_kernel(const uint16_t *wb
     }
     ok = mbar_wait(mbar, 0) && ok;
     tc_after_sync();
-    hidden_row(tlane, 0, wb, kB1, A, t, live && act ? act + (int64_t)b * kMlpAct : nullptr);
+    hidden_row<VEC>(tlane, 0, bias, A, row, j0, live && act ? act + (int64_t)b * kMlpAct : nullptr);
     fence_async_smem();
     tc_before_sync();
     __syncthreads();
@@ -210,7 +283,7 @@ __global__ void __launch_bounds__(kTcM) mlp_forward_tc_kernel(const uint16_t *wb
     }
     ok = ok && mbar_wait(mbar, 1);
     tc_after_sync();
-    hidden_row(tlane, kMlpH, wb, kB2, A, t, live && act ? act + (int64_t)b * kMlpAct + kMlpH : nullptr);
+    hidden_row<VEC>(tlane, kMlpH, bias + kMlpH, A, row, j0, live && act ? act + (int64_t)b * kMlpAct + kMlpH : nullptr);
     fence_async_smem();
     tc_before_sync();
     __syncthreads();
@@ -235,12 +308,12 @@ __global__ void __launch_bounds__(kTcM) mlp_forward_tc_kernel(const uint16_t *wb
         if (t == 0) raise_status(err, RT_ETIMEOUT);
         return;
     }
-    if (!live) return;
+    if (!live || j0) return;
     float z[kMlpOut];
     int best = 0;
 #pragma unroll
     for (int k = 0; k < kMlpOut; ++k) {
-        z[k] = zv[k] + __uint_as_float((uint32_t)wb[kB3 + k] << 16);
+        z[k] = zv[k] + bias[2 * kMlpH + k];
         if (logits) logits[(int64_t)b * kMlpOut + k] = z[k];
         if (z[k] > z[best]) best = k;
     }
@@ -253,7 +326,8 @@ __global__ void __launch_bounds__(kTcM) mlp_forward_tc_kernel(const uint16_t *wb
     if (pick) pick[b] = best;
 }
 
-// Backward on the tensor cores, 128 samples per CTA (thread t: sample t).
+// Backward on the tensor cores, 128 samples per CTA (threads t and t + 128:
+// sample t).
 //   dz  = (softmax(z) - onehot(label)) / B               (fp32, per thread)
 //   dh2 = (dz W3) * [h2 > 0]                              (fp32, per thread: K = 3)
 //   dh1 = (dh2 W2) * [h1 > 0]                             (product 1: 128 x 64, K = 64)
@@ -275,16 +349,33 @@ constexpr int kBwB2 = kBwA2 + kTcM * kTcM * 2;      // 96 x 128: [h1 | xn | 1]^T
 constexpr int kBwSmem = kBwB2 + kBwN2 * kTcM * 2;   // 73728 bytes (dynamic)
 constexpr int kBwPart = kW3;                        // partial sums per CTA: W1 b1 W2 b2
 
-__global__ void __launch_bounds__(kTcM) mlp_backward_tc_kernel(const uint16_t *wb, const float *norm, const float *x,
-                                                               const float *act, const float *logits,
-                                                               const int32_t *label, int B, float *part, float *dz_out,
-                                                               float *loss_out, int32_t *err)
+// Column t (even and odd lanes side by side) of a K = 128 operand, rows
+// n .. n + 15: lanes exchange one value of each pair of rows, so every store
+// is two samples of one row.
+__device__ __forceinline__ void store_column16(uint8_t *op, int n, int t, const float *v)
+{
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+        const uint32_t mine = two_bf16(v[i], v[i + 1]), other = __shfl_xor_sync(0xffffffffu, mine, 1);
+        const uint32_t both = (t & 1) ? __byte_perm(other, mine, 0x7632) : __byte_perm(mine, other, 0x5410);
+        *reinterpret_cast<uint32_t *>(op + core_off(n + i + (t & 1), t & ~1, kTcM)) = both;
+    }
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(kTcThreads) mlp_backward_tc_kernel(const uint16_t *wb, const float *norm,
+                                                                     const float *x, const float *act,
+                                                                     const float *logits, const int32_t *label, int B,
+                                                                     float *part, float *dz_out, float *loss_out,
+                                                                     int32_t *err)
 {
     extern __shared__ __align__(1024) uint8_t smb[];
     __shared__ __align__(8) uint64_t mbar_store;
     __shared__ uint32_t tmem_base;
-    const int t = threadIdx.x, warp = t >> 5;
-    const int b = blockIdx.x * kTcM + t;
+    __shared__ __align__(16) float w3[kMlpOut * kMlpH];
+    constexpr int kHalf = kMlpH / 2;
+    const int t = threadIdx.x, warp = t >> 5, row = t & (kTcM - 1), half = t / kTcM, j0 = half * kHalf;
+    const int b = blockIdx.x * kTcM + row;
     const bool live = b < B;
     const uint32_t mbar = smem_u32(&mbar_store);
     if (warp == 0) {
@@ -297,15 +388,36 @@ __global__ void __launch_bounds__(kTcM) mlp_backward_tc_kernel(const uint16_t *w
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // W2^T as product 1's B: B[n][k] = W2[k][n]
-    for (int i = t; i < kMlpH * kMlpH; i += kTcM) {
-        const int n = i % kMlpH, k = i / kMlpH;
-        *reinterpret_cast<uint16_t *>(smb + kBwB1 + core_off(n, k, kMlpH)) = wb[kW2 + k * kMlpH + n];
+    // W2^T as product 1's B: B[n][k] = W2[k][n], 8 columns of rows k and k + 1 per thread
+    {
+        static_assert(kMlpH / 2 * (kMlpH / 8) == kTcThreads, "one pair of 16-byte pieces per thread");
+        const int k = 2 * (t / (kMlpH / 8)), n = 8 * (t % (kMlpH / 8));
+        const uint4 p = load_w8<VEC>(wb + kW2 + k * kMlpH + n), q = load_w8<VEC>(wb + kW2 + (k + 1) * kMlpH + n);
+        const uint32_t a[4] = {p.x, p.y, p.z, p.w}, c[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            *reinterpret_cast<uint32_t *>(smb + kBwB1 + core_off(n + e, k, kMlpH)) =
+                __byte_perm(a[e / 2], c[e / 2], (e & 1) ? 0x7632 : 0x5410);
     }
-    // this sample's deltas of the output and the second hidden layer (fp32)
-    float h2[kMlpH], dz[kMlpOut];
-    float lossb = 0.f;
+    if (t < kMlpOut * kMlpH) w3[t] = of_bf16(wb[kW3 + t]);
+    // this sample's deltas of the output (both of its threads) and of half the second hidden layer (fp32)
+    float h2[kHalf], h1[kHalf], xn[16], dz[kMlpOut];
+#pragma unroll
+    for (int k = 0; k < kMlpOut; ++k) dz[k] = 0.f;
+#pragma unroll
+    for (int j = 0; j < kHalf; ++j) h1[j] = h2[j] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) xn[k] = 0.f;
     if (live) {
+        const float *ar = act + (int64_t)b * kMlpAct + j0;
+#pragma unroll
+        for (int j = 0; j < kHalf; j += 4) load4<VEC>(ar + kMlpH + j, h2 + j);
+#pragma unroll
+        for (int j = 0; j < kHalf; j += 4) load4<VEC>(ar + j, h1 + j);
+        // the input columns 0 .. 15, or 16 .. 23 and the one
+#pragma unroll
+        for (int k = 0; k < 16; k += 4)
+            if (half == 0 || k < kMlpIn - 16) load4<VEC>(x + (int64_t)b * kMlpIn + 16 * half + k, xn + k);
         const float *z = logits + (int64_t)b * kMlpOut;
         float m = z[0];
 #pragma unroll
@@ -314,36 +426,32 @@ __global__ void __launch_bounds__(kTcM) mlp_backward_tc_kernel(const uint16_t *w
 #pragma unroll
         for (int k = 0; k < kMlpOut; ++k) se += expf(z[k] - m);
         const int y = label[b];
-        lossb = logf(se) + m - z[y];
 #pragma unroll
         for (int k = 0; k < kMlpOut; ++k) {
             dz[k] = (expf(z[k] - m) / se - (k == y ? 1.f : 0.f)) / (float)B;
-            dz_out[(int64_t)b * kMlpOut + k] = dz[k];
+            if (half == 0) dz_out[(int64_t)b * kMlpOut + k] = dz[k];
         }
-        loss_out[b] = lossb;
-#pragma unroll
-        for (int j = 0; j < kMlpH; ++j) h2[j] = act[(int64_t)b * kMlpAct + kMlpH + j];
-    } else {
-#pragma unroll
-        for (int k = 0; k < kMlpOut; ++k) dz[k] = 0.f;
-#pragma unroll
-        for (int j = 0; j < kMlpH; ++j) h2[j] = 0.f;
+        if (half == 0) loss_out[b] = logf(se) + m - z[y];
     }
+    __syncthreads();   // w3
 #pragma unroll
-    for (int j = 0; j < kMlpH; ++j) {
+    for (int j = 0; j < kHalf; ++j) {
         float s = 0.f;
 #pragma unroll
-        for (int k = 0; k < kMlpOut; ++k) s = fmaf(__uint_as_float((uint32_t)wb[kW3 + k * kMlpH + j] << 16), dz[k], s);
-        const uint16_t d = to_bf16(h2[j] > 0.f ? s : 0.f);
-        *reinterpret_cast<uint16_t *>(smb + kBwA1 + core_off(t, j, kMlpH)) = d;     // row t of product 1's A
-        *reinterpret_cast<uint16_t *>(smb + kBwA2 + core_off(j, t, kTcM)) = d;      // column t of product 2's A
+        for (int k = 0; k < kMlpOut; ++k) s = fmaf(w3[k * kMlpH + j0 + j], dz[k], s);
+        h2[j] = h2[j] > 0.f ? s : 0.f;
     }
+#pragma unroll
+    for (int j = 0; j < kHalf; j += 8)   // row of product 1's A
+        *reinterpret_cast<uint4 *>(smb + kBwA1 + core_off(row, j0 + j, kMlpH)) =
+            make_uint4(two_bf16(h2[j], h2[j + 1]), two_bf16(h2[j + 2], h2[j + 3]), two_bf16(h2[j + 4], h2[j + 5]),
+                       two_bf16(h2[j + 6], h2[j + 7]));
     fence_async_smem();
     tc_before_sync();
     __syncthreads();
     tc_after_sync();
     const uint32_t tmem = tmem_base;
-    const uint32_t tlane = tmem + ((uint32_t)(32 * warp) << 16);
+    const uint32_t tlane = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
     bool ok = true;
     if (t == 0) {
         for (int s = 0; s < kMlpH / 16; ++s)
@@ -351,35 +459,31 @@ __global__ void __launch_bounds__(kTcM) mlp_backward_tc_kernel(const uint16_t *w
                      smem_desc(smem_u32(smb + kBwB1) + 256 * s, kMlpH), instr_desc(kTcM, kMlpH), s > 0);
         mma_commit(mbar);
     }
-    // meanwhile: column t of product 2's B (h1, xn and a one, as bf16)
-    {
-        float xn[kMlpIn];
+    // meanwhile: column `row` of product 2's A (dh2) and B (h1, xn, a one and the padding), as bf16
 #pragma unroll
-        for (int k = 0; k < kMlpIn; ++k) xn[k] = live ? (x[(int64_t)b * kMlpIn + k] - norm[k]) / norm[kMlpIn + k] : 0.f;
+    for (int q = 0; q < 2; ++q) {
+        store_column16(smb + kBwA2, j0 + 16 * q, row, h2 + 16 * q);
+        store_column16(smb + kBwB2, j0 + 16 * q, row, h1 + 16 * q);
+    }
+    if (live) {
 #pragma unroll
-        for (int n = 0; n < kBwN2; ++n) {
-            float v = 0.f;
-            if (live) {
-                if (n < kMlpH) v = act[(int64_t)b * kMlpAct + n];
-                else if (n < kBwOne) v = xn[n - kMlpH];
-                else if (n == kBwOne) v = 1.f;
-            }
-            *reinterpret_cast<uint16_t *>(smb + kBwB2 + core_off(n, t, kTcM)) = to_bf16(v);
+        for (int k = 0; k < 16; ++k) {
+            const int c = 16 * half + k;
+            if (c < kMlpIn) xn[k] = (xn[k] - norm[c]) / norm[kMlpIn + c];
+            if (c == kMlpIn) xn[k] = 1.f;
         }
     }
+    store_column16(smb + kBwB2, kMlpH + 16 * half, row, xn);
     ok = mbar_wait(mbar, 0) && ok;
     tc_after_sync();
-    // dh1 = (dh2 W2) * [h1 > 0]: column t of product 2's A, rows 64..127
+    // dh1 = (dh2 W2) * [h1 > 0]: column `row` of product 2's A, rows 64..127
 #pragma unroll
-    for (int q = 0; q < kMlpH / 16; ++q) {
+    for (int q = 0; q < 2; ++q) {
         float v[16];
-        tmem_ld16(tlane + (uint32_t)(16 * q), v);
+        tmem_ld16(tlane + (uint32_t)(j0 + 16 * q), v);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int j = 16 * q + i;
-            const bool on = live && act[(int64_t)b * kMlpAct + j] > 0.f;
-            *reinterpret_cast<uint16_t *>(smb + kBwA2 + core_off(kMlpH + j, t, kTcM)) = to_bf16(on ? v[i] : 0.f);
-        }
+        for (int i = 0; i < 16; ++i) v[i] = h1[16 * q + i] > 0.f ? v[i] : 0.f;   // 0 if not live
+        store_column16(smb + kBwA2, kMlpH + j0 + 16 * q, row, v);
     }
     fence_async_smem();
     tc_before_sync();
@@ -393,29 +497,29 @@ __global__ void __launch_bounds__(kTcM) mlp_backward_tc_kernel(const uint16_t *w
     }
     ok = ok && mbar_wait(mbar, 1);
     tc_after_sync();
-    // row t of product 2: feature t of dh2 (t < 64) or of dh1 (t >= 64)
+    // row `row` of product 2: feature `row` of dh2 (< 64) or of dh1; the workspace is aligned
     float *pc = part + (int64_t)blockIdx.x * kBwPart;
-    if (warp < 2) {
+    if ((warp & 3) < 2) {
 #pragma unroll
-        for (int q = 0; q < kMlpH / 16; ++q) {
+        for (int q = 0; q < 2; ++q) {
             float v[16];
-            tmem_ld16(tlane + kMlpH + (uint32_t)(16 * q), v);
+            tmem_ld16(tlane + kMlpH + (uint32_t)(j0 + 16 * q), v);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) pc[kW2 + t * kMlpH + 16 * q + i] = v[i];
+            for (int i = 0; i < 16; i += 4) store4<true>(pc + kW2 + row * kMlpH + j0 + 16 * q + i, v + i);
         }
-        float v[16];
-        tmem_ld16(tlane + kMlpH + 80, v);
-        pc[kB2 + t] = v[kBwOne - 80];
+        if (half) {
+            float v[16];
+            tmem_ld16(tlane + kMlpH + 80, v);
+            pc[kB2 + row] = v[kBwOne - 80];
+        }
     } else {
-        const int i1 = t - kMlpH;
+        const int i1 = row - kMlpH;
         float v[16];
-        tmem_ld16(tlane + kMlpH + 64, v);
+        tmem_ld16(tlane + kMlpH + 64 + 16 * (uint32_t)half, v);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) pc[kW1 + i1 * kMlpIn + i] = v[i];
-        tmem_ld16(tlane + kMlpH + 80, v);
-#pragma unroll
-        for (int i = 0; i < kMlpIn - 16; ++i) pc[kW1 + i1 * kMlpIn + 16 + i] = v[i];
-        pc[kB1 + i1] = v[kBwOne - 80];
+        for (int i = 0; i < 16; i += 4)
+            if (half == 0 || i < kMlpIn - 16) store4<true>(pc + kW1 + i1 * kMlpIn + 16 * half + i, v + i);
+        if (half) pc[kB1 + i1] = v[kBwOne - 80];
     }
     tc_before_sync();
     __syncthreads();
@@ -456,6 +560,8 @@ __global__ void mlp_grad_tc_kernel(const float *part, int nblk, const float *dz,
     }
 }
 
+bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
+
 }  // namespace
 
 size_t mlp_backward_tc_workspace_bytes(int B)
@@ -473,9 +579,11 @@ cudaError_t launch_mlp_backward_tc(const uint16_t *wb, const float *norm, const 
     float *part = ws;
     float *dz = part + (int64_t)nblk * kBwPart;
     float *lossb = dz + (int64_t)B * kMlpOut;
-    cudaError_t e = cudaFuncSetAttribute(mlp_backward_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwSmem);
+    const auto kernel = aligned16(wb) && aligned16(x) && aligned16(act) ? mlp_backward_tc_kernel<true>
+                                                                        : mlp_backward_tc_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwSmem);
     if (e != cudaSuccess) return e;
-    mlp_backward_tc_kernel<<<nblk, kTcM, kBwSmem, s>>>(wb, norm, x, act, logits, label, B, part, dz, lossb, err);
+    kernel<<<nblk, kTcThreads, kBwSmem, s>>>(wb, norm, x, act, logits, label, B, part, dz, lossb, err);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     mlp_grad_tc_kernel<<<(unsigned)ceil_div((int64_t)(kMlpParams + 1) * 32, 256), 256, 0, s>>>(part, nblk, dz, act,
                                                                                                lossb, B, grad, loss);
@@ -487,8 +595,10 @@ cudaError_t launch_mlp_forward_tc(const uint16_t *wb, const float *norm, const f
                                   cudaStream_t s)
 {
     if (B <= 0) return cudaSuccess;
-    mlp_forward_tc_kernel<<<(unsigned)ceil_div(B, kTcM), kTcM, 0, s>>>(wb, norm, x, B, logits, act, pick, min_prob,
-                                                                       fallback, err);
+    const auto kernel = aligned16(wb) && aligned16(x) && aligned16(act) ? mlp_forward_tc_kernel<true>
+                                                                        : mlp_forward_tc_kernel<false>;
+    kernel<<<(unsigned)ceil_div(B, kTcM), kTcThreads, 0, s>>>(wb, norm, x, B, logits, act, pick, min_prob, fallback,
+                                                              err);
     return cudaGetLastError();
 }
 
