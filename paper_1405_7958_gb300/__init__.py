@@ -49,8 +49,15 @@ def _check(code: int, where: str):
         raise RtError(code, where)
 
 
+# torch.cuda.current_stream() builds a Stream object, 2.9 us of each call; the
+# raw handle of the current device's current stream takes 0.2
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream
 
