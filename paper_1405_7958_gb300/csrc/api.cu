@@ -392,6 +392,8 @@ void carve_contract(Carve &cv, CtBatch &b)
     b.best = cv.take<unsigned long long>(nt * kCtNodes);
     b.act = cv.take<uint32_t>(nt * kCtNodes);
     b.edge = cv.take<unsigned long long>(nt * kCtUnits * kCtUnitEdges);
+    b.ecnt = cv.take<uint8_t>(nt * kCtUnits);
+    b.rim = cv.take<uint16_t>(nt * 4 * kCtSide);
 }
 
 // Enqueue the contraction of a carved batch; launch_contract_out writes R.
@@ -402,7 +404,7 @@ rt_status run_contract(rt_ctx *ctx, CtBatch &b, int32_t *err, cudaStream_t s, co
     RT_CUDA_TRY(zero_words(b.ctl, kCtCtlWords, s));
     Phase ph(ctx, RT_PHASE_RECON_SWEEP, s);
     RT_CUDA_TRY(launch_contract(b, ctx->num_sms, lim.timeout_ns, s));
-    ctx->launches += 3;
+    ctx->launches += 4;
     return RT_OK;
 }
 

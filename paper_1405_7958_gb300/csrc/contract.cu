@@ -34,15 +34,16 @@
 // until each open cluster's best edge leaves the tile; what is left of a
 // tile are its nodes (clusters that touch its rim, about 50 of 4096 pixels
 // on nuclei tiles), the forest between them, and 2 bytes per pixel (node,
-// bound). ct_global_kernel adds the edges across the seams and contracts
-// the nodes of the whole batch (one persistent cooperative launch).
+// bound). ct_seam_kernel adds the edges across the seams; ct_global_kernel
+// contracts the nodes of the whole batch (one persistent cooperative launch).
 // ct_out_kernel writes R.
 //
 // Measured on one GB300 against the directional sweeps (rt_segment_batch or
-// rt_reconstruct, whole call): 512 x 512 reconstruction 85 us against 357;
-// one 4096 x 4096 tile 0.66 ms against 1.37; eight of them 3.55 ms against
-// 5.65; a 16384 x 16384 slide 6.9 ms against 10.4. So the contraction runs
-// wherever the call leaves the schedule to the library.
+// rt_reconstruct, whole call; the chain's other stages are the same):
+// 512 x 512 reconstruction 78 us against 357; one 4096 x 4096 tile 0.47 ms
+// against 1.17; eight of them 2.6 ms against 4.7; a 16384 x 16384 slide 5.0
+// ms against 8.5. So the contraction runs wherever the call leaves the
+// schedule to the library.
 #include "contract.cuh"
 
 namespace rtk {
@@ -622,6 +623,10 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
         if (t < kCtNodes) best[kRoots + t] = 0u;
     }
     __syncthreads();
+    if (t < 4 * kCtSide) {
+        const uint32_t w = W[rim];
+        b.rim[(int64_t)tile * 4 * kCtSide + t] = (uint16_t)(w ? (nlink[w & kIdx] & 0xff00u) | w >> 24 : kCtNoNode << 8);
+    }
     {
         uint16_t *o = b.plane + (int64_t)tile * kCtPx + rs * kCtSide + cl;
 #pragma unroll 2
@@ -696,129 +701,295 @@ constexpr uint32_t kMix = 2654435761u, kUnmix = 244002641u;   // inverses mod 2^
 constexpr int kMaxRounds = 64;
 static_assert(kMix * kUnmix == 1u, "inverse");
 
-__device__ __forceinline__ uint32_t ct_node(const CtBatch &b, const CtImage &d, int r, int c)
+// A barrier of the cooperative grid that also adds up a number per CTA: word
+// counts arrivals in its low half and the numbers in its high half (zero
+// before the launch), `target` is all arrivals up to this barrier. An
+// arrival is one release without an answer and the wait one polled word, 1.5
+// us; counting down, a generation and separate fences took 3.7. The wait is
+// bounded: RT_ETIMEOUT and false.
+__device__ __forceinline__ bool sum_barrier(unsigned long long *word, uint32_t target, uint32_t add, uint32_t &sum,
+                                            int32_t *err, uint64_t timeout_ns)
 {
-    const int t = d.tile_base + (r / kCtSide) * d.nx + c / kCtSide;
-    const uint32_t e = __ldcg(b.plane + (int64_t)t * kCtPx + (r % kCtSide) * kCtSide + c % kCtSide);
-    return (uint32_t)t * kCtNodes + (e >> 8);
+    __shared__ uint32_t s_sum;
+    __shared__ int s_ok;
+    if (threadIdx.x == 0) {   // the caller has synchronised the CTA
+        const unsigned long long one = 1ull | (unsigned long long)add << 32;
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(word), "l"(one) : "memory");
+        unsigned long long v;
+        int ok = 1;
+        uint64_t t0 = 0;
+        for (uint32_t spins = 1;; ++spins) {
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
+            if ((int32_t)((uint32_t)v - target) >= 0) break;
+            if ((spins & 255u) != 0) continue;
+            __nanosleep(64);
+            const uint64_t now = globaltimer_ns();
+            if (!t0) t0 = now;
+            if (now - t0 > timeout_ns) {
+                raise_status(err, RT_ETIMEOUT);
+                ok = 0;
+                break;
+            }
+        }
+        s_sum = (uint32_t)(v >> 32);
+        s_ok = ok;
+    }
+    __syncthreads();
+    sum = s_sum;
+    return s_ok != 0;
 }
 
-// The root above node x and its link word.
-__device__ __forceinline__ uint32_t ct_root(const CtBatch &b, uint32_t x, unsigned long long &l)
+// The roots above the ends of two edges and their link words, the walks side
+// by side.
+__device__ __forceinline__ void ct_roots(const CtBatch &b, uint32_t (&x)[4], unsigned long long (&l)[4],
+                                         const bool (&have)[2])
 {
-    l = __ldcg(b.link + x);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) l[k] = have[k / 2] ? __ldcg(b.link + x[k]) : kNodeRoot;
 #pragma unroll 1
-    for (int n = 0; n < (1 << 20) && !(l & kNodeRoot); ++n) {
-        x = (uint32_t)l;
-        l = __ldcg(b.link + x);
+    for (int n = 0; n < (1 << 20); ++n) {
+        bool more = false;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (!(l[k] & kNodeRoot)) {
+                x[k] = (uint32_t)l[k];
+                l[k] = __ldcg(b.link + x[k]);
+                more = true;
+            }
+        if (!more) break;
     }
-    return x;
+}
+
+// An edge's key in round `round`: later rounds first, then heavier ones, then
+// by the edge's slot g, mixed.
+__device__ __forceinline__ unsigned long long edge_key(int round, uint32_t w, uint32_t g)
+{
+    return (unsigned long long)(round + 1) << 48 | (unsigned long long)(w + 1u) << 32 | g * kMix;
 }
 
 }  // namespace
 
+// ------------------------------------------------------------------- seams
+// The edges across the seams and round 0's best edge of every node, a CTA
+// per tile. A tile has four units, each a quarter of its nodes and forest and
+// half a seam (parts 0, 1: the right one, 2, 3: the lower one); warp w writes
+// the edges of part w behind the part's forest edges. The pixels come from
+// the tiles' rims, a few words a lane. The best edges are first found in
+// shared memory, for the nodes of the tile and of its right and its lower
+// neighbour: by weight, then among equals by the mixed slot, which is what
+// edge_key orders by; then one global maximum a node. (The global kernel's
+// warps built the seams and raced for the bests one unit after the other:
+// 240 us of 505 for eight 4096 x 4096 tiles; this kernel takes 15 per tile.)
+__global__ void __launch_bounds__(kCtUnits * 32) ct_seam_kernel(const __grid_constant__ CtBatch b)
+{
+    __shared__ __align__(16) uint32_t bw[3 * kCtNodes], bg[3 * kCtNodes];
+    const int tile = blockIdx.x, t = threadIdx.x, lane = t & 31, part = t >> 5;
+    const uint32_t all = 0xffffffffu, below = (1u << lane) - 1u;
+    const CtImage &d = ct_image(b, tile);
+    const int lt = tile - d.tile_base;
+    const int ty = lt / d.nx, tx = lt - ty * d.nx;
+    const bool down = part >= 2;
+    const int u = tile * kCtUnits + part;
+    // this lane's edges: up to two of the forest, two of the seam
+    uint32_t ea[4], ec[4], ew[4], eg[4];
+    bool have[4] = {false, false, false, false};
+    const int nf = ((int)(__ldcg(b.cnt + tile) >> 16) - part + kCtUnits - 1) / kCtUnits;
+    unsigned long long *edge = b.edge + (int64_t)u * kCtUnitEdges;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        have[k] = lane + 32 * k < nf;
+        const unsigned long long e = have[k] ? __ldcg(edge + lane + 32 * k) : 0ull;
+        ea[k] = (uint32_t)(e >> 28) & kNodeId;
+        ec[k] = (uint32_t)e & kNodeId;
+        ew[k] = (uint32_t)(e >> 56);
+        eg[k] = (uint32_t)u * kCtUnitEdges + lane + 32 * k;
+    }
+    for (int i = t; i < 3 * kCtNodes / 4; i += kCtUnits * 32) {
+        reinterpret_cast<uint4 *>(bw)[i] = make_uint4(0u, 0u, 0u, 0u);
+        reinterpret_cast<uint4 *>(bg)[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    // half a seam: a lane takes the pixel m0 on this side, the one across m1,
+    // and the window of both and their next neighbours n0, n1; p0, p1 are
+    // their previous neighbours. Rim words: node << 8 | I, node kCtNoNode
+    // outside the image. Keys order the pixels by (I, raster order), 0 =
+    // outside.
+    int ne = nf;
+    if (down ? ty + 1 < d.ny : tx + 1 < d.nx) {   // whole warp
+        const int i = (part & 1) * 32 + lane;
+        const int t1 = down ? tile + d.nx : tile + 1;           // the tile across
+        const int step = down ? 1 : d.nx;                       // to the next tile along the seam
+        const int s0 = down ? 1 : 3, s1 = down ? 0 : 2;         // the sides that meet
+        auto rim = [&](int ut, int side, int at) { return (uint32_t)__ldg(b.rim + ((int64_t)ut * 4 + side) * kCtSide + at); };
+        const uint32_t none = kCtNoNode << 8;
+        const uint32_t m0 = rim(tile, s0, i), m1 = rim(t1, s1, i);
+        // the ends' neighbours along the seam may be the next tiles'
+        const bool end = lane == 0 || lane == 31;
+        const int ni = lane == 0 ? i - 1 : i + 1;
+        const int hop = ni < 0 ? -step : ni >= kCtSide ? step : 0;
+        const bool there = hop == 0 || (hop < 0 ? (down ? tx > 0 : ty > 0) : (down ? tx + 1 < d.nx : ty + 1 < d.ny));
+        uint32_t x0 = none, x1 = none;
+        if (end && there) {
+            x0 = rim(tile + hop, s0, ni & (kCtSide - 1));
+            x1 = rim(t1 + hop, s1, ni & (kCtSide - 1));
+        }
+        uint32_t p0 = __shfl_up_sync(all, m0, 1), p1 = __shfl_up_sync(all, m1, 1), n0 = __shfl_down_sync(all, m0, 1),
+                 n1 = __shfl_down_sync(all, m1, 1);
+        if (lane == 0) p0 = x0, p1 = x1;
+        if (lane == 31) n0 = x0, n1 = x1;
+        auto key = [&](uint32_t w, uint32_t along, uint32_t across) {
+            return w >= none ? 0u : ((w & 0xffu) + 1u) << 4 | (down ? across * 3u + along : along * 2u + across);
+        };
+        const uint32_t k0 = key(m0, 1, 0), k1 = key(m1, 1, 1), l0 = key(n0, 2, 0), l1 = key(n1, 2, 1);
+        const bool in = k0 && k1;
+        have[2] = in && max(k0, k1) > max(max(key(p0, 0, 0), key(p1, 0, 1)), max(l0, l1));
+        // the window at the tile's corner belongs to the right seam
+        have[3] = in && l0 && l1 && !(down && i == kCtSide - 1);
+        const bool main = max(k0, l1) > max(k1, l0);
+        const int nt = lane == 31 ? hop : 0;   // the next neighbours' tiles
+        const uint32_t a0 = (uint32_t)tile * kCtNodes + (m0 >> 8), a1 = (uint32_t)t1 * kCtNodes + (m1 >> 8),
+                       c0 = (uint32_t)(tile + nt) * kCtNodes + (n0 >> 8), c1 = (uint32_t)(t1 + nt) * kCtNodes + (n1 >> 8);
+        ea[2] = a0, ec[2] = a1, ew[2] = (min(k0, k1) >> 4) - 1u;
+        ea[3] = main ? a0 : c0, ec[3] = main ? c1 : a1, ew[3] = (main ? min(k0, l1) : min(k1, l0)) / 16u - 1u;
+#pragma unroll
+        for (int k = 2; k < 4; ++k) {
+            // of neighbouring lanes' edges between the same nodes the heaviest (the first of equals): a vote on all
+            // equal pairs of the warp takes longer than the few edges more
+            const uint32_t w = have[k] ? ew[k] + 1u : 0u;
+            const uint32_t pa = __shfl_up_sync(all, ea[k], 1), pc = __shfl_up_sync(all, ec[k], 1),
+                           pw = __shfl_up_sync(all, w, 1), na = __shfl_down_sync(all, ea[k], 1),
+                           nc = __shfl_down_sync(all, ec[k], 1), nw = __shfl_down_sync(all, w, 1);
+            if (lane > 0 && pa == ea[k] && pc == ec[k] && pw >= w) have[k] = false;
+            if (lane < 31 && na == ea[k] && nc == ec[k] && nw > w) have[k] = false;
+            const uint32_t m = __ballot_sync(all, have[k]);
+            const int at = ne + __popc(m & below);
+            eg[k] = (uint32_t)u * kCtUnitEdges + at;
+            if (have[k]) edge[at] = node_edge(ea[k], ec[k], ew[k]);
+            ne += __popc(m);
+        }
+    }
+    if (lane == 0) b.ecnt[u] = (uint8_t)ne;
+    // a node's place in bw and bg; elsewhere (over the corner): -1
+    auto place = [&](uint32_t x) {
+        const int ut = (int)(x >> 8);
+        return ut == tile ? (int)(x & 0xffu) : ut == tile + 1 ? kCtNodes + (int)(x & 0xffu)
+               : ut == tile + d.nx ? 2 * kCtNodes + (int)(x & 0xffu) : -1;
+    };
+    int pl[8];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        pl[k] = -1;
+        if (!have[k / 2]) continue;
+        const uint32_t x = k & 1 ? ec[k / 2] : ea[k / 2], w = ew[k / 2] + 1u;
+        pl[k] = place(x);
+        if (pl[k] < 0) atomicMax(b.best + x, edge_key(0, ew[k / 2], eg[k / 2]));
+        else if (bw[pl[k]] < w) atomicMax(bw + pl[k], w);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (pl[k] >= 0 && bw[pl[k]] == ew[k / 2] + 1u) atomicMax(bg + pl[k], eg[k / 2] * kMix);
+    __syncthreads();
+#pragma unroll
+    for (int i = t; i < 3 * kCtNodes; i += kCtUnits * 32) {
+        const uint32_t w = bw[i];
+        const int ut = i < kCtNodes ? tile : i < 2 * kCtNodes ? tile + 1 : tile + d.nx;
+        if (w) atomicMax(b.best + (uint32_t)ut * kCtNodes + (i & (kCtNodes - 1)),
+                         1ull << 48 | (unsigned long long)w << 32 | bg[i]);
+    }
+}
+
 // Contraction of the nodes of the batch. The work is cut into units, four a
-// tile (a quarter of its nodes and forest, half a seam); every warp owns the
-// units [u0, u1) and keeps their nodes and edges compacted at the start of
-// their slots, so no list is shared. A round: (1) the edges find their
-// clusters and raise the clusters' best edges; (2) every open root takes its
+// tile; every warp owns the units [u0, u1) and keeps their nodes and, from
+// round 1 on, edges compacted at the start of their slots, so no list is
+// shared. A round: (1) the edges find their clusters and raise the clusters'
+// best edges (round 0: by ct_seam_kernel); (2) every open root takes its
 // decision. A grid barrier follows each. Roots that joined are pointed at
 // their new root, with the smallest weight on the way, at the start of the
-// next round's (1); readers that come first walk on. One CTA an SM: a
-// barrier's cost is its arrivals at one address. CLUSTER: the grid is one
-// cluster, and the barrier the hardware's.
+// next round's (1); readers that come first walk on. Bound by the latency of
+// dependent reads in L2, so a lane has two edges or roots in flight, and by
+// the barriers (8 rounds); one CTA an SM: a barrier's cost is its arrivals at
+// one address. CLUSTER: the grid is one cluster, and the barrier the
+// hardware's. 1024 x 1024: 50 us (79 with the seams, one in flight and the
+// slower barrier), 4096 x 4096: 80 (138), eight of them: 190 (505).
 template <bool CLUSTER>
 __global__ void __launch_bounds__(kGT, 1) ct_global_kernel(const __grid_constant__ CtBatch b, uint64_t timeout_ns)
 {
-    auto barrier = [&]() -> bool {
-        if (CLUSTER) {
-            __threadfence();
-            asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-            return true;
-        }
-        return grid_barrier(b.ctl + kCtCtlBar, gridDim.x, b.err, timeout_ns);
-    };
     const int lane = threadIdx.x & 31;
     const int64_t gw = (int64_t)blockIdx.x * (kGT / 32) + (threadIdx.x >> 5), nw = (int64_t)gridDim.x * (kGT / 32);
     const int64_t units = (int64_t)b.ntiles * kCtUnits;
     const int u0 = (int)(gw * units / nw), u1 = (int)((gw + 1) * units / nw);
-    const uint32_t below = (1u << lane) - 1u;
+    const uint32_t all = 0xffffffffu, below = (1u << lane) - 1u;
     unsigned long long *edge = b.edge + (int64_t)u0 * kCtUnitEdges;
     uint32_t *act = b.act + (int64_t)u0 * kCtUnitNodes;
+    unsigned long long *word = reinterpret_cast<unsigned long long *>(b.ctl + kCtCtlBar);
     int ne = 0, na = 0;
-    __shared__ uint32_t s_open;
+    uint32_t target = 0, seen = 0;   // arrivals at the barriers so far, open roots handed in
+    // open roots: of the CTA, or (CLUSTER) of the cluster, in turn
+    __shared__ uint32_t s_open[3];
+    if (threadIdx.x < 3) s_open[threadIdx.x] = 0u;
+    __syncthreads();
+    if (CLUSTER)   // no CTA adds to another's before it is zero
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 
-    auto emit = [&](bool valid, uint32_t a, uint32_t c, uint32_t w) {   // whole warp: one edge per node pair
-        valid = valid && (a & 0xffu) != kCtNoNode && (c & 0xffu) != kCtNoNode;   // always: rim pixels are in nodes
-        const unsigned long long pair = valid ? (unsigned long long)a << 32 | c : ~0ull;
-        const uint32_t peers = __match_any_sync(0xffffffffu, pair);
-        const uint32_t wm = __reduce_max_sync(peers, w);
-        const bool lead = valid && lane == __ffs(peers) - 1;
-        const uint32_t m = __ballot_sync(0xffffffffu, lead);
-        if (lead) edge[ne + __popc(m & below)] = node_edge(a, c, wm);
-        ne += __popc(m);
-    };
+    // this warp's nodes, 32 units at a time
 #pragma unroll 1
-    for (int u = u0; u < u1; ++u) {
-        const int t = u / kCtUnits, part = u % kCtUnits;
-        const CtImage &d = ct_image(b, t);
-        const int lt = t - d.tile_base;
-        const int ty = lt / d.nx, tx = lt - ty * d.nx;
-        const uint32_t cn = __ldcg(b.cnt + t);
-        const int nn = ((int)(cn & 0xffffu) - part + kCtUnits - 1) / kCtUnits,
-                  nf = ((int)(cn >> 16) - part + kCtUnits - 1) / kCtUnits;
+    for (int ub = u0; ub < u1; ub += 32) {
+        const int u = ub + lane;
+        const int cn = u < u1 ? (int)(__ldcg(b.cnt + u / kCtUnits) & 0xffffu) : 0;
+        const int mine = max(0, (cn - u % kCtUnits + kCtUnits - 1) / kCtUnits);
 #pragma unroll 1
-        for (int i = lane; i < nn; i += 32) act[na + i] = (uint32_t)(t * kCtNodes + part + i * kCtUnits);
-        na += nn;
-        // the unit's part of the forest moves up (never past its own slots)
-        const unsigned long long *from = b.edge + (int64_t)u * kCtUnitEdges;
+        for (int j = 0; j < 32 && ub + j < u1; ++j) {
+            const int n = __shfl_sync(all, mine, j);
+            const uint32_t first = (uint32_t)((ub + j) / kCtUnits * kCtNodes + (ub + j) % kCtUnits);
 #pragma unroll 1
-        for (int i = 0; i < nf; i += 32) {
-            const unsigned long long e = i + lane < nf ? from[i + lane] : 0ull;
-            __syncwarp();
-            if (i + lane < nf) edge[ne + i + lane] = e;
-            __syncwarp();
+            for (int i = lane; i < n; i += 32) act[na + i] = first + (uint32_t)(i * kCtUnits);
+            na += n;
         }
-        ne += nf;
-        // half a seam (parts 0, 1: the right one, 2, 3: the lower one): a lane
-        // takes the pixel m0 on this side, the one across m1, and the window
-        // of both and their next neighbours n0, n1; p0, p1 are their previous
-        // neighbours. Keys order the pixels by (I, raster order), 0 = outside.
-        const bool down = part >= 2;
-        const int i = (part & 1) * 32 + lane;
-        if (down ? ty + 1 < d.ny : tx + 1 < d.nx) {   // whole warp
-            const int r = ty * kCtSide + (down ? kCtSide - 1 : i), c = tx * kCtSide + (down ? i : kCtSide - 1);
-            auto key = [&](int along, int across) -> uint32_t {
-                const int y = r + (down ? across : along), x = c + (down ? along : across);
-                if (y < 0 || y >= d.H || x < 0 || x >= d.W) return 0u;
-                return ((uint32_t)__ldg(d.mask + (int64_t)y * d.ld_mask + x) + 1u) << 4 |
-                       (uint32_t)(down ? across * 3 + along + 1 : (along + 1) * 2 + across);
-            };
-            auto node = [&](int along, int across) {
-                return ct_node(b, d, r + (down ? across : along), c + (down ? along : across));
-            };
-            const uint32_t p0 = key(-1, 0), p1 = key(-1, 1), m0 = key(0, 0), m1 = key(0, 1), n0 = key(1, 0),
-                           n1 = key(1, 1);
-            const bool in = m0 && m1;
-            const bool s = in && max(m0, m1) > max(max(p0, p1), max(n0, n1));
-            // the window at the tile's corner belongs to the right seam
-            const bool q = in && n0 && n1 && !(down && i == kCtSide - 1), main = max(m0, n1) > max(m1, n0);
-            uint32_t a0 = 0, a1 = 0, c0 = 0, c1 = 0;
-            if (s || q) {
-                a0 = node(0, 0), a1 = node(0, 1);
-                if (q) c0 = node(1, 0), c1 = node(1, 1);
-            }
-            emit(s, a0, a1, s ? (min(m0, m1) >> 4) - 1u : 0u);
-            emit(q, main ? a0 : c0, main ? c1 : a1, q ? ((main ? min(m0, n1) : min(m1, n0)) >> 4) - 1u : 0u);
+    }
+    __syncwarp();
+
+    // (1) on two edges a lane; they move to the front of the warp's slots
+    int kept = 0;
+    auto edges = [&](int round, const unsigned long long (&e)[2], const bool (&have)[2]) {   // whole warp
+        uint32_t x[4];
+        unsigned long long l[4];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            x[2 * k] = (uint32_t)(e[k] >> 28) & kNodeId;
+            x[2 * k + 1] = (uint32_t)e[k] & kNodeId;
+        }
+        ct_roots(b, x, l, have);
+        bool keep[2], oa[2], oc[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            oa[k] = !(l[2 * k] & kNodeDone);
+            oc[k] = !(l[2 * k + 1] & kNodeDone);
+            keep[k] = have[k] && x[2 * k] != x[2 * k + 1] && (oa[k] || oc[k]);
         }
         __syncwarp();
-    }
+        unsigned long long old[4], key[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint32_t m = __ballot_sync(all, keep[k]);
+            const int at = kept + __popc(m & below);
+            const uint32_t w = (uint32_t)(e[k] >> 56);
+            key[k] = edge_key(round, w, (uint32_t)u0 * kCtUnitEdges + at);
+            if (keep[k]) edge[at] = node_edge(x[2 * k], x[2 * k + 1], w);
+            kept += __popc(m);
+            old[2 * k] = keep[k] && oa[k] ? __ldcg(b.best + x[2 * k]) : ~0ull;
+            old[2 * k + 1] = keep[k] && oc[k] ? __ldcg(b.best + x[2 * k + 1]) : ~0ull;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (old[k] < key[k / 2]) atomicMax(b.best + x[k], key[k / 2]);
+    };
 
 #pragma unroll 1
     for (int round = 0; round < kMaxRounds; ++round) {
-        // (0) roots that joined: final links of the last round; the others stay open
         if (round > 0) {
-            int kept = 0;
+            // (0) roots that joined: final links of the last round; the others stay open
+            kept = 0;
 #pragma unroll 1
             for (int i = 0; i < na; i += 32) {
                 bool open = false;
@@ -828,6 +999,7 @@ __global__ void __launch_bounds__(kGT, 1) ct_global_kernel(const __grid_constant
                     unsigned long long l = __ldcg(b.link + r);
                     open = (l & kNodeRoot) != 0ull;
                     if (!open) {
+                        const uint32_t S = b.S[r];   // stored by this warp when it joined
                         uint32_t w = (uint32_t)(l >> 32), x = (uint32_t)l;
 #pragma unroll 1
                         for (int n = 0; n < (1 << 20); ++n) {
@@ -837,96 +1009,144 @@ __global__ void __launch_bounds__(kGT, 1) ct_global_kernel(const __grid_constant
                             x = (uint32_t)l;
                         }
                         __stcg(b.link + r, (unsigned long long)w << 32 | x);
-                        const uint32_t S = b.S[r];   // stored by this warp when it joined
                         if (node_S(l) < S) atomicMax(b.link + x, kNodeRoot | (unsigned long long)S << 40 | x);
                     }
                 }
-                const uint32_t m = __ballot_sync(0xffffffffu, open);
+                const uint32_t m = __ballot_sync(all, open);
                 if (open) act[kept + __popc(m & below)] = r;
                 kept += __popc(m);
                 __syncwarp();
             }
             na = kept;
-        }
-        // (1) edges; a key holds the round, so the last round's bests count as none
-        int kept = 0;
+            // (1) edges; a key holds the round, so the last round's bests count as none
+            kept = 0;
+            if (round == 1) {
+                // out of the units' own slots: their edges in a row, a lane finds its by the units' prefix sums
 #pragma unroll 1
-        for (int i = 0; i < ne; i += 32) {
-            uint32_t a = 0, c = 0, w = 0;
-            bool keep = false, oa = true, oc = true;
-            if (i + lane < ne) {
-                const unsigned long long e = edge[i + lane];
-                a = (uint32_t)(e >> 28) & kNodeId;
-                c = (uint32_t)e & kNodeId;
-                w = (uint32_t)(e >> 56);
-                if (round > 0) {
-                    unsigned long long la, lc;
-                    a = ct_root(b, a, la);
-                    c = ct_root(b, c, lc);
-                    oa = !(la & kNodeDone);
-                    oc = !(lc & kNodeDone);
+                for (int ub = u0; ub < u1; ub += 32) {
+                    const int n = ub + lane < u1 ? (int)__ldcg(b.ecnt + ub + lane) : 0;
+                    int end = n;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int v = __shfl_up_sync(all, end, o);
+                        if (lane >= o) end += v;
+                    }
+                    const int total = __shfl_sync(all, end, 31);
+#pragma unroll 1
+                    for (int i = 0; i < total; i += 64) {
+                        unsigned long long e[2];
+                        bool have[2];
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            const int f = i + 32 * k + lane;
+                            int j = 0;   // units that end at or before f
+#pragma unroll
+                            for (int o = 16; o > 0; o >>= 1)
+                                if (__shfl_sync(all, end, j + o - 1) <= f) j += o;
+                            const int first = __shfl_sync(all, end - n, j & 31);
+                            have[k] = f < total;
+                            e[k] = have[k] ? __ldcg(b.edge + (int64_t)(ub + j) * kCtUnitEdges + (f - first)) : 0ull;
+                        }
+                        edges(round, e, have);
+                        __syncwarp();
+                    }
                 }
-                keep = a != c && (oa || oc);
+            } else {
+#pragma unroll 1
+                for (int i = 0; i < ne; i += 64) {
+                    unsigned long long e[2];
+                    bool have[2];
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        have[k] = i + 32 * k + lane < ne;
+                        e[k] = have[k] ? edge[i + 32 * k + lane] : 0ull;
+                    }
+                    edges(round, e, have);
+                    __syncwarp();
+                }
             }
-            const uint32_t m = __ballot_sync(0xffffffffu, keep);
-            if (keep) {
-                const int at = kept + __popc(m & below);
-                edge[at] = node_edge(a, c, w);
-                const uint32_t g = (uint32_t)u0 * kCtUnitEdges + at;
-                const unsigned long long k =
-                    (unsigned long long)(round + 1) << 48 | (unsigned long long)(w + 1u) << 32 | g * kMix;
-                if (oa && __ldcg(b.best + a) < k) atomicMax(b.best + a, k);
-                if (oc && __ldcg(b.best + c) < k) atomicMax(b.best + c, k);
+            ne = kept;
+            // open roots of the batch: all of them hand in theirs with the barrier
+            const int slot = round % 3;
+            uint32_t open;
+            if (CLUSTER) {
+                if (na && lane < kGCluster) {
+                    uint32_t at = (uint32_t)__cvta_generic_to_shared(s_open + slot);
+                    asm volatile("mapa.shared::cluster.u32 %0, %0, %1;" : "+r"(at) : "r"(lane));
+                    asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(at), "r"(na) : "memory");
+                }
+                if (threadIdx.x == 0) s_open[(round + 1) % 3] = 0u;   // last read two rounds ago
+                __syncwarp();
+                asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+                open = *(volatile uint32_t *)(s_open + slot);
+            } else {
+                if (na && lane == 0) atomicAdd(s_open + slot, (uint32_t)na);
+                __syncthreads();
+                uint32_t sum;
+                if (!sum_barrier(word, target += gridDim.x, s_open[slot], sum, b.err, timeout_ns)) return;
+                if (threadIdx.x == 0) s_open[slot] = 0u;
+                open = sum - seen;
+                seen = sum;
             }
-            kept += __popc(m);
-            __syncwarp();
+            if (open == 0u) return;
         }
-        ne = kept;
-        // open roots of the batch: the round's counter (the next one's is cleared)
-        uint32_t *open_cnt = b.ctl + kCtCtlOpen + round % 3;
-        if (lane == 0 && na) atomicAdd(open_cnt, (uint32_t)na);
-        if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(b.ctl + kCtCtlOpen + (round + 1) % 3, 0u);
-        if (!barrier()) return;
-        if (threadIdx.x == 0) s_open = ld_acquire(open_cnt);
-        __syncthreads();
-        if (s_open == 0u) return;
-        // (2) decisions
+        // (2) decisions, two a lane
         kept = 0;
 #pragma unroll 1
-        for (int i = 0; i < na; i += 32) {
-            bool open = false;
-            uint32_t r = 0;
-            if (i + lane < na) {
-                r = act[i + lane];
-                const unsigned long long k = __ldcg(b.best + r), l = __ldcg(b.link + r);
-                const bool some = (uint32_t)(k >> 48) == (uint32_t)(round + 1);
-                const uint32_t w = ((uint32_t)(k >> 32) & 0xffffu) - 1u, S = node_S(l);
-                if (!some || S >= w) {
-                    atomicOr(b.link + r, kNodeDone);
-                } else {
-                    open = true;
-                    const unsigned long long e = __ldcg(b.edge + (uint32_t)k * kUnmix);
-                    const uint32_t a = (uint32_t)(e >> 28) & kNodeId, c = (uint32_t)e & kNodeId, o = a == r ? c : a;
+        for (int i = 0; i < na; i += 64) {
+            bool in[2], open[2];
+            uint32_t r[2], w[2], S[2];
+            unsigned long long key[2], e[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                in[k] = i + 32 * k + lane < na;
+                r[k] = in[k] ? act[i + 32 * k + lane] : 0u;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                key[k] = in[k] ? __ldcg(b.best + r[k]) : 0ull;
+                S[k] = in[k] ? node_S(__ldcg(b.link + r[k])) : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const bool some = (uint32_t)(key[k] >> 48) == (uint32_t)(round + 1);
+                w[k] = ((uint32_t)(key[k] >> 32) & 0xffffu) - 1u;
+                open[k] = in[k] && some && S[k] < w[k];
+                e[k] = open[k] ? __ldcg(b.edge + (uint32_t)key[k] * kUnmix) : 0ull;
+                if (in[k] && !open[k]) atomicOr(b.link + r[k], kNodeDone);
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (open[k]) {
+                    const uint32_t a = (uint32_t)(e[k] >> 28) & kNodeId, c = (uint32_t)e[k] & kNodeId,
+                                   o = a == r[k] ? c : a;
                     // o joins r by the same edge: the smaller of the two stays
                     // (o may have joined already; its link word is no root's then)
                     bool mutual = false;
-                    if (r < o && __ldcg(b.best + o) == k) {
+                    if (r[k] < o && __ldcg(b.best + o) == key[k]) {
                         const unsigned long long lo = __ldcg(b.link + o);
-                        mutual = !(lo & kNodeRoot) || node_S(lo) < w;
+                        mutual = !(lo & kNodeRoot) || node_S(lo) < w[k];
                     }
                     if (!mutual) {
-                        b.S[r] = S;
-                        __stcg(b.link + r, (unsigned long long)w << 32 | o);
+                        b.S[r[k]] = S[k];
+                        __stcg(b.link + r[k], (unsigned long long)w[k] << 32 | o);
                     }
                 }
+                const uint32_t m = __ballot_sync(all, open[k]);
+                if (open[k]) act[kept + __popc(m & below)] = r[k];
+                kept += __popc(m);
+                __syncwarp();
             }
-            const uint32_t m = __ballot_sync(0xffffffffu, open);
-            if (open) act[kept + __popc(m & below)] = r;
-            kept += __popc(m);
-            __syncwarp();
         }
         na = kept;
-        if (!barrier()) return;
+        if (CLUSTER) {
+            asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        } else {
+            __syncthreads();
+            uint32_t sum;
+            if (!sum_barrier(word, target += gridDim.x, 0u, sum, b.err, timeout_ns)) return;
+        }
     }
     raise_status(b.err, RT_ETIMEOUT);   // not reached: every round at least halves the open roots of a component
 }
@@ -1010,6 +1230,8 @@ cudaError_t launch_contract(const CtBatch &b, int num_sms, uint64_t timeout_ns, 
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalSmem);
     if (e != cudaSuccess) return e;
     fn<<<(unsigned)b.ntiles, few ? 512 : 256, kLocalSmem, s>>>(b);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    ct_seam_kernel<<<(unsigned)b.ntiles, kCtUnits * 32, 0, s>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int64_t units = (int64_t)b.ntiles * kCtUnits;
     const int need = (int)ceil_div(units, kGT / 32);

@@ -44,14 +44,15 @@ struct CtBatch {
     uint32_t *S;             // per node that joined another: its sources' best value
     uint32_t *act;           // per node slot: the warps' lists of roots still open
     unsigned long long *edge;   // per edge slot: weight and nodes
+    uint8_t *ecnt;           // per unit: its edges
+    uint16_t *rim;           // per tile: its upper row, lower row, left and right column: node << 8 | I
     unsigned long long *bits;   // nullable: B = (R < threshold), per tile 64 rows, bit = column
     uint32_t *ctl;           // kCtCtlWords control words, zeroed before the launches
     int32_t *err;            // device status word
     CtImage img[kCtMaxImgs];
 };
 
-constexpr int kCtCtlBar = 0;      // grid barrier: arrivals, generation
-constexpr int kCtCtlOpen = 2;     // three counters of open roots, used in turn
+constexpr int kCtCtlBar = 0;      // grid barrier: arrivals, open roots handed in (64 bits)
 constexpr int kCtCtlWords = 8;
 
 void ct_plan_image(CtBatch &b, const uint8_t *marker, int64_t ld_marker, const uint8_t *mask, int64_t ld_mask, int H,
