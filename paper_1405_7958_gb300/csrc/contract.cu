@@ -1159,6 +1159,9 @@ __global__ void __launch_bounds__(256) ct_out_kernel(const __grid_constant__ CtB
     const CtImage &d = ct_image(b, tile);
     const int lt = tile - d.tile_base;
     const int ty = lt / d.nx, tx = lt - ty * d.nx;
+    // the pixels' words are on their way while the nodes' values are found
+    const uint4 *src = reinterpret_cast<const uint4 *>(b.plane + (int64_t)tile * kCtPx + (t >> 2) * kCtSide + (t & 3) * 16);
+    const uint4 s0 = __ldcs(src), s1 = __ldcs(src + 1);
     const int nn = (int)(b.cnt[tile] & 0xffffu);
     uint32_t v = 255u;
     if (t < nn) {
@@ -1174,8 +1177,6 @@ __global__ void __launch_bounds__(256) ct_out_kernel(const __grid_constant__ CtB
     __syncthreads();
     const int r = ty * kCtSide + (t >> 2), c = tx * kCtSide + (t & 3) * 16;
     const int n = r < d.H ? min(16, d.W - c) : 0;   // may be negative: none
-    const uint4 *src = reinterpret_cast<const uint4 *>(b.plane + (int64_t)tile * kCtPx + (t >> 2) * kCtSide + (t & 3) * 16);
-    const uint4 s0 = __ldcs(src), s1 = __ldcs(src + 1);
     const uint32_t e[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
     uint32_t R[4] = {0, 0, 0, 0}, B = 0;
 #pragma unroll

@@ -22,9 +22,9 @@
 //     tile's run words back and writes labels, the kept bits and the count.
 //
 // Measured on one GB300, 4096 x 4096 nuclei tiles: filling eight of them takes
-// 0.26 ms (0.28 as bit-plane floods swept to a fixed point), labeling 0.19 ms
-// (0.66 as a union-find over pixels); one tile alone 67 us against 129 and 49
-// against 99, a 1024 x 1024 one 46 against 64 and 26 against 36. The local
+// 0.22 ms (0.28 as bit-plane floods swept to a fixed point), labeling 0.14 ms
+// (0.66 as a union-find over pixels); one tile alone 59 us against 129 and 43
+// against 99, a 1024 x 1024 one 45 against 64 and 26 against 36. The local
 // stages are bound by the latency of the tiles with the most runs, the label
 // stage by its stores (4 bytes a pixel).
 #include "runs.cuh"
@@ -36,13 +36,49 @@ namespace {
 typedef unsigned long long u64;
 
 constexpr int kFewTiles = 2048;
-constexpr int kWarps = 2;                 // tiles per CTA: a tile with many runs keeps few others' memory
+constexpr int kWarps = 4;                 // tiles per CTA; 1 while they fit in one wave (kFewTiles)
+// Shared memory: a warp's share holds a tile of up to kLightRuns runs (most
+// nuclei tiles) and lists the pairs of touching runs to join kLightPairs at a
+// time. A tile with more (up to kMaxRuns) waits until the other warps are done
+// and takes the whole block's. With room for the worst tile at every warp an
+// SM held 22 tiles; now it holds 32 or more, and 16 to 22 of an image of
+// nothing but heavy tiles. Eight 4096 x 4096 tiles: the local stages 80 and
+// 137 -> 63 and 114 us; one: 19 and 33 -> 17 and 27. Few tiles (kFewTiles)
+// fit all the same, and a heavy one would only wait, so there a block has one
+// warp (ALONE): 1024 x 1024 20 us against 22.
 constexpr int kMaxRuns = kRunWords;
-// Pairs of touching runs joined at a time: at most kPairSteps per lane. (The
-// lists of a seam fit too: 2 x 64 x 3 pairs.)
-constexpr int kPairSteps = 16, kPairs = 32 * kPairSteps;
-constexpr int kWarpWords = kMaxRuns + kPairs;   // shared memory of a warp
+constexpr int kLightRuns = 384, kLightPairs = 256, kWarpWords = kLightRuns + kLightPairs;
+constexpr int kHeavyPairs = kWarps * kWarpWords - kMaxRuns;
 constexpr size_t kRunSmem = sizeof(uint32_t) * kWarpWords * kWarps;
+template <bool ALONE>
+struct Mem {
+    bool heavy;
+    __device__ __forceinline__ volatile uint32_t *runs() const   // a word per run
+    {
+        extern __shared__ uint32_t run_smem[];
+        return run_smem + (ALONE || heavy ? 0 : (threadIdx.x >> 5) * kWarpWords);
+    }
+    __device__ __forceinline__ volatile uint32_t *pairs() const { return runs() + (ALONE || heavy ? kMaxRuns : kLightRuns); }
+    __device__ __forceinline__ int cap() const { return ALONE || heavy ? kHeavyPairs : kLightPairs; }
+};
+// Calls f(memory of the tile) for every warp of the block with its number of
+// runs; all threads of the block call it. ALONE: a block of one warp.
+template <bool ALONE, class F>
+__device__ __forceinline__ void with_memory(int runs, F &&f)
+{
+    if (ALONE) {
+        f(Mem<ALONE>{false});
+        return;
+    }
+    const bool heavy = runs > kLightRuns;
+    if (!heavy) f(Mem<ALONE>{false});
+    if (!__syncthreads_or(heavy)) return;
+#pragma unroll 1
+    for (int turn = 0; turn < kWarps; ++turn) {
+        if (heavy && turn == (int)(threadIdx.x >> 5)) f(Mem<ALONE>{true});
+        __syncthreads();
+    }
+}
 constexpr uint32_t kRim = 1u << 31, kBorder = 1u << 30, kParent = 0xffffu;
 constexpr int kSlotShift = 16;
 constexpr uint32_t kSlotMask = kRunSlots - 1;
@@ -69,15 +105,6 @@ static_assert(kMix * kUnmix == 1u, "inverse");
 __device__ __forceinline__ uint32_t mix(uint32_t x) { return x * kMix; }
 __device__ __forceinline__ uint32_t parent(const uint32_t *U, uint32_t v) { return __ldcg(U + v * kUnmix); }
 
-__device__ __forceinline__ uint32_t node_root(const uint32_t *U, uint32_t v)   // of and in mixed numbers
-{
-    uint32_t p = parent(U, v);
-    while (p != v) {
-        v = p;
-        p = parent(U, v);
-    }
-    return v;
-}
 __device__ __forceinline__ uint32_t node_find(uint32_t *U, uint32_t v)
 {
     uint32_t p = parent(U, v);
@@ -137,6 +164,11 @@ __device__ __forceinline__ void flatten(volatile uint32_t *P, int total, int lan
     }
 }
 
+__device__ __forceinline__ int count_runs(u64 m0, u64 m1)
+{
+    return (int)__reduce_add_sync(0xffffffffu, (uint32_t)(__popcll(m0 & ~(m0 << 1)) + __popcll(m1 & ~(m1 << 1))));
+}
+
 // The runs of (m0, m1).
 __device__ __forceinline__ Runs runs_of(u64 m0, u64 m1, int lane)
 {
@@ -161,7 +193,7 @@ __device__ __forceinline__ Runs runs_of(u64 m0, u64 m1, int lane)
 }
 
 // Components of the runs of (m0, m1): afterwards P[run] is its root run
-// (upper bits 0). Whole warp; pairs: kPairs words.
+// (upper bits 0). Whole warp.
 // The lanes list the places where two runs of adjacent rows first touch (the
 // first column of a stretch they share, or, for 8-connectivity, a corner),
 // then all lanes share the list: every pair whose roots differ hooks the
@@ -169,9 +201,11 @@ __device__ __forceinline__ Runs runs_of(u64 m0, u64 m1, int lane)
 // the next round), the trees are flattened, and at least half of the
 // components that can still join are gone. Unions by the rows' own lanes, one
 // after the other, kept a speckled nucleus's few lanes busy for 25 us a tile.
-template <int CONN>
-__device__ __forceinline__ Runs components(u64 m0, u64 m1, volatile uint32_t *P, volatile uint32_t *pairs, int lane)
+template <int CONN, bool ALONE>
+__device__ __forceinline__ Runs components(u64 m0, u64 m1, const Mem<ALONE> &mem, int lane)
 {
+    volatile uint32_t *P = mem.runs(), *pairs = mem.pairs();
+    const int cap = mem.cap();
     const Runs r = runs_of(m0, m1, lane);
     const uint32_t below = (1u << lane) - 1u;
     for (int i = lane; i < r.total; i += 32) P[i] = (uint32_t)i;
@@ -198,7 +232,7 @@ __device__ __forceinline__ Runs components(u64 m0, u64 m1, volatile uint32_t *P,
             const int ba = k < 3 ? r.base[0] : r.base[1], bb = k < 3 ? r.base[1] : dbase;
             constexpr int kStep[3] = {0, 1, -1};
 #pragma unroll 1
-            while (n + 32 <= kPairs && __any_sync(0xffffffffu, e[k] != 0ull)) {
+            while (n + 32 <= cap && __any_sync(0xffffffffu, e[k] != 0ull)) {
                 const bool some = e[k] != 0ull;
                 const uint32_t m = __ballot_sync(0xffffffffu, some);
                 if (some) {
@@ -345,11 +379,12 @@ __device__ __forceinline__ u64 run_bits(u64 m, int pos) { return m & ~(m + (1ull
 
 // Background components of a tile (foreground f0, f1), marked kRim and
 // kBorder (on the image border), the rim ones numbered.
-template <int CONN, class F>
-__device__ __forceinline__ Runs background(const RunImage &d, const Place &p, u64 f0, u64 f1, volatile uint32_t *P,
-                                           int lane, int &cnt, F &&f)
+template <int CONN, bool ALONE, class F>
+__device__ __forceinline__ Runs background(const RunImage &d, const Place &p, u64 f0, u64 f1, const Mem<ALONE> &mem, int lane,
+                                           int &cnt, F &&f)
 {
-    const Runs r = components<CONN>(exists(d, p, 2 * lane) & ~f0, exists(d, p, 2 * lane + 1) & ~f1, P, P + kMaxRuns, lane);
+    volatile uint32_t *P = mem.runs();
+    const Runs r = components<CONN>(exists(d, p, 2 * lane) & ~f0, exists(d, p, 2 * lane + 1) & ~f1, mem, lane);
     if (p.ty == 0) flag_runs(P, 0, __shfl_sync(0xffffffffu, r.n[0], 0), kBorder, lane);
     const int last = d.H - 1 - p.r0;
     if (last < kRunSide) {   // whole warp
@@ -399,38 +434,39 @@ __global__ void __launch_bounds__(256) run_pack_kernel(const __grid_constant__ R
 // --------------------------------------------------------------------- fill
 // Warp per tile: holes inside the tile are filled; the other background
 // components become slots.
-template <int CONN>
-__global__ void __launch_bounds__(kWarps * 32) run_fill_local_kernel(const __grid_constant__ RunBatch b)
+template <int CONN, bool ALONE>
+__global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_fill_local_kernel(const __grid_constant__ RunBatch b)
 {
-    extern __shared__ uint32_t run_smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int tile = blockIdx.x * kWarps + warp;
-    if (tile >= b.ntiles) return;
-    volatile uint32_t *P = run_smem + warp * kWarpWords;
+    const int lane = threadIdx.x & 31, at = blockIdx.x * (ALONE ? 1 : kWarps) + (threadIdx.x >> 5);
+    const bool mine = at < b.ntiles;
+    const int tile = mine ? at : 0;
     const RunImage &d = run_image(b, tile);
     const Place p = place_of(d, tile);
     const uint32_t node = 1u + (uint32_t)tile * kRunSlots;
     const ulonglong2 f = *(reinterpret_cast<const ulonglong2 *>(b.bits + (int64_t)tile * kRunSide) + lane);
-    if (!__any_sync(0xffffffffu, (f.x | f.y) != 0ull)) {   // nothing but background (no words): one component
-        const bool border = p.ty == 0 || p.tx == 0 || p.r0 + kRunSide >= d.H || p.c0 + kRunSide >= d.W;
-        const bool rim = p.open[0] || p.open[1] || p.open[2] || p.open[3];
-        uint16_t *s = reinterpret_cast<uint16_t *>(b.sides + (int64_t)tile * kRunSides) + lane;
-        const int nr = min(kRunSide, d.H - p.r0), nc = min(kRunSide, d.W - p.c0);
-        auto pair = [&](int n) { return (uint16_t)((2 * lane < n ? 0u : 255u) | (2 * lane + 1 < n ? 0u : 255u) << 8); };
-        if (p.open[0]) s[0] = pair(nc);
-        if (p.open[1]) s[kRunSide / 2] = pair(nc);
-        if (p.open[2]) s[2 * kRunSide / 2] = pair(nr);
-        if (p.open[3]) s[3 * kRunSide / 2] = pair(nr);
-        if (lane == 0) {
-            b.cnt[tile] = rim ? 1u : 0u;
-            if (rim) b.outside[node] = border ? 0u : mix(node);
-            if (tile == 0) b.outside[0] = 0u;
+    with_memory<ALONE>(count_runs(exists(d, p, 2 * lane) & ~f.x, exists(d, p, 2 * lane + 1) & ~f.y), [&](const Mem<ALONE> &mem) {
+        if (!mine) return;
+        if (!__any_sync(0xffffffffu, (f.x | f.y) != 0ull)) {   // nothing but background (no words): one component
+            const bool border = p.ty == 0 || p.tx == 0 || p.r0 + kRunSide >= d.H || p.c0 + kRunSide >= d.W;
+            const bool rim = p.open[0] || p.open[1] || p.open[2] || p.open[3];
+            uint16_t *s = reinterpret_cast<uint16_t *>(b.sides + (int64_t)tile * kRunSides) + lane;
+            const int nr = min(kRunSide, d.H - p.r0), nc = min(kRunSide, d.W - p.c0);
+            auto pair = [&](int n) { return (uint16_t)((2 * lane < n ? 0u : 255u) | (2 * lane + 1 < n ? 0u : 255u) << 8); };
+            if (p.open[0]) s[0] = pair(nc);
+            if (p.open[1]) s[kRunSide / 2] = pair(nc);
+            if (p.open[2]) s[2 * kRunSide / 2] = pair(nr);
+            if (p.open[3]) s[3 * kRunSide / 2] = pair(nr);
+            if (lane == 0) {
+                b.cnt[tile] = rim ? 1u : 0u;
+                if (rim) b.outside[node] = border ? 0u : mix(node);
+                if (tile == 0) b.outside[0] = 0u;
+            }
+            return;
         }
-        return;
-    }
-    int cnt = 0;
-    const Runs r = background<CONN>(d, p, f.x, f.y, P, lane, cnt, [&](int i, int k) {
-        b.outside[node + k] = P[i] & kBorder ? 0u : mix(node + k);
+        int cnt = 0;
+        volatile uint32_t *P = mem.runs();
+        const Runs r = background<CONN>(d, p, f.x, f.y, mem, lane, cnt, [&](int i, int k) {
+            b.outside[node + k] = P[i] & kBorder ? 0u : mix(node + k);
     });
     uint32_t *words = b.words + (int64_t)tile * kRunWords;
     for (int i = lane; i < r.total; i += 32) words[i] = P[i];
@@ -439,6 +475,7 @@ __global__ void __launch_bounds__(kWarps * 32) run_fill_local_kernel(const __gri
         b.cnt[tile] = (uint8_t)cnt;
         if (tile == 0) b.outside[0] = 0u;
     }
+    });
 }
 
 // Warp per tile: joins the slots across its right and lower seams (and, for
@@ -505,114 +542,123 @@ __global__ void __launch_bounds__(kWarps * 32) run_seam_kernel(const __grid_cons
 
 // Warp per tile. FILL: slots that did not reach the outside are filled, F is
 // written. LABEL: then the foreground's components become slots.
-template <bool FILL, int LABEL>
-__global__ void __launch_bounds__(kWarps * 32) run_local_kernel(const __grid_constant__ RunBatch b)
+template <bool FILL, int LABEL, bool ALONE>
+__global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_local_kernel(const __grid_constant__ RunBatch b)
 {
-    extern __shared__ uint32_t run_smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int tile = blockIdx.x * kWarps + warp;
-    if (tile >= b.ntiles) return;
-    volatile uint32_t *P = run_smem + warp * kWarpWords;
+    const int lane = threadIdx.x & 31, at = blockIdx.x * (ALONE ? 1 : kWarps) + (threadIdx.x >> 5);
+    const bool mine = at < b.ntiles;
+    const int tile = mine ? at : 0;
     const RunImage &d = run_image(b, tile);
     const Place p = place_of(d, tile);
     ulonglong2 *row = reinterpret_cast<ulonglong2 *>(b.bits + (int64_t)tile * kRunSide) + lane;
     ulonglong2 f = *row;
-    if (FILL) {
-        // holes: components that neither touch the image border nor reach it
-        // through their slot
-        const uint32_t node = 1u + (uint32_t)tile * kRunSlots;
-        u64 add[2] = {0ull, 0ull};
-        if (!__any_sync(0xffffffffu, (f.x | f.y) != 0ull)) {
-            if (b.cnt[tile] && node_find(b.outside, mix(node)) != 0u) {
-                add[0] = exists(d, p, 2 * lane);
-                add[1] = exists(d, p, 2 * lane + 1);
-            }
-        } else {
-            const Runs r = runs_of(exists(d, p, 2 * lane) & ~f.x, exists(d, p, 2 * lane + 1) & ~f.y, lane);
-            const uint32_t *words = b.words + (int64_t)tile * kRunWords;
-            for (int i = lane; i < r.total; i += 32) {
-                uint32_t v = words[i];
-                if ((v & kParent) == (uint32_t)i) {   // roots: kBorder if outside
-                    if ((v & kRim) && node_find(b.outside, mix(node + ((v >> kSlotShift) & kSlotMask))) == 0u) v |= kBorder;
-                    v = (v & kBorder) | (uint32_t)i;
+    // the background's runs and the foreground's after filling: a row's filled runs join what they touch, or are the
+    // row's only one
+    auto starts = [](u64 m) { return __popcll(m & ~(m << 1)); };
+    int runs = starts(f.x) + starts(f.y);
+    if (FILL)
+        runs = max(starts(f.x), starts(exists(d, p, 2 * lane) & ~f.x)) +
+               max(starts(f.y), starts(exists(d, p, 2 * lane + 1) & ~f.y));
+    with_memory<ALONE>((int)__reduce_add_sync(0xffffffffu, (uint32_t)runs), [&](const Mem<ALONE> &mem) {
+        if (!mine) return;
+        volatile uint32_t *P = mem.runs();
+        if (FILL) {
+            // holes: components that neither touch the image border nor reach it
+            // through their slot
+            const uint32_t node = 1u + (uint32_t)tile * kRunSlots;
+            u64 add[2] = {0ull, 0ull};
+            if (!__any_sync(0xffffffffu, (f.x | f.y) != 0ull)) {
+                if (b.cnt[tile] && node_find(b.outside, mix(node)) != 0u) {
+                    add[0] = exists(d, p, 2 * lane);
+                    add[1] = exists(d, p, 2 * lane + 1);
                 }
-                P[i] = v;
+            } else {
+                const Runs r = runs_of(exists(d, p, 2 * lane) & ~f.x, exists(d, p, 2 * lane + 1) & ~f.y, lane);
+                const uint32_t *words = b.words + (int64_t)tile * kRunWords;
+                for (int i = lane; i < r.total; i += 32) {
+                    uint32_t v = words[i];
+                    if ((v & kParent) == (uint32_t)i) {   // roots: kBorder if outside
+                        if ((v & kRim) && node_find(b.outside, mix(node + ((v >> kSlotShift) & kSlotMask))) == 0u) v |= kBorder;
+                        v = (v & kBorder) | (uint32_t)i;
+                    }
+                    P[i] = v;
+                }
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    u64 s = r.st[j];
+                    for (int k = 0; s; ++k, s &= s - 1)
+                        if (!(P[P[r.base[j] + k] & kParent] & kBorder)) add[j] |= run_bits(r.m[j], __ffsll((long long)s) - 1);
+                }
+                __syncwarp();
             }
+            if (__any_sync(0xffffffffu, (add[0] | add[1]) != 0ull)) {
+                f = make_ulonglong2(f.x | add[0], f.y | add[1]);
+                *row = f;
+            }
+            if (d.filled) {
+                // lane: 16 columns (lane & 3) of row 8 q + lane / 4
+#pragma unroll 2
+                for (int q = 0; q < 8; ++q) {
+                    const int i = 8 * q + (lane >> 2), r = p.r0 + i, c = p.c0 + (lane & 3) * 16;
+                    const u64 w0 = shfl64(f.x, i >> 1), w1 = shfl64(f.y, i >> 1);
+                    const uint32_t m = (uint32_t)((i & 1 ? w1 : w0) >> ((lane & 3) * 16)) & 0xffffu;
+                    const int n = r < d.H ? min(16, d.W - c) : 0;
+                    if (n <= 0) continue;
+                    uint8_t *o = d.filled + (int64_t)r * d.ld_filled + c;
+                    if (n == 16 && ((uintptr_t)o & 15u) == 0) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) w[k] = (((m >> (4 * k)) & 0xfu) * 0x00204081u) & 0x01010101u;
+                        *reinterpret_cast<uint4 *>(o) = make_uint4(w[0], w[1], w[2], w[3]);
+                    } else {
+                        for (int k = 0; k < n; ++k) o[k] = (uint8_t)((m >> k) & 1u);
+                    }
+                }
+            }
+        }
+        if (LABEL) {
+            if (tile == d.tile_base && lane == 0 && d.n_kept) *d.n_kept = 0;
+            const uint32_t node = 1u + (uint32_t)tile * kRunSlots;
+            if (!__any_sync(0xffffffffu, (f.x | f.y) != 0ull)) {
+                uint16_t *s = reinterpret_cast<uint16_t *>(b.sides + (int64_t)tile * kRunSides) + lane;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (p.open[k]) s[k * kRunSide / 2] = 0xffffu;
+                if (lane == 0) b.lcnt[tile] = 0u;
+                return;
+            }
+            const Runs r = components<LABEL ? LABEL : 8>(f.x, f.y, mem, lane);
+            flag_rim(r, p, P, lane);
+            const int cnt = number_slots(r, P, lane, [&](int, int k) {
+                b.U[node + k] = mix(node + k);
+                b.A[node + k] = 0u;
+            });
+            write_sides(b, r, p, P, lane);
             __syncwarp();
+            // areas: a slot's to its node, with its first pixel (a root run is its
+            // component's first), another component's to its root's upper bits
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 u64 s = r.st[j];
-                for (int k = 0; s; ++k, s &= s - 1)
-                    if (!(P[P[r.base[j] + k] & kParent] & kBorder)) add[j] |= run_bits(r.m[j], __ffsll((long long)s) - 1);
+                for (int k = 0; s; ++k, s &= s - 1) {
+                    const int run = r.base[j] + k, pos = __ffsll((long long)s) - 1;
+                    const uint32_t root = P[run] & kParent, v = P[root], area = (uint32_t)__popcll(run_bits(r.m[j], pos));
+                    if (v & kRim) {
+                        const uint32_t slot = node + ((v >> kSlotShift) & kSlotMask);
+                        atomicAdd(b.A + slot, area);
+                        if (root == (uint32_t)run) b.M[slot] = (uint32_t)((int64_t)(p.r0 + 2 * lane + j) * d.W + p.c0 + pos);
+                    } else {
+                        atomicAdd(const_cast<uint32_t *>(P + root), area << kSlotShift);
+                    }
+                }
             }
             __syncwarp();
+            uint32_t *words = b.words + (int64_t)tile * kRunWords;
+            for (int i = lane; i < r.total; i += 32) words[i] = P[i];
+            if (lane == 0) b.lcnt[tile] = (uint8_t)cnt;
         }
-        if (__any_sync(0xffffffffu, (add[0] | add[1]) != 0ull)) {
-            f = make_ulonglong2(f.x | add[0], f.y | add[1]);
-            *row = f;
-        }
-        if (d.filled) {
-            // lane: 16 columns (lane & 3) of row 8 q + lane / 4
-#pragma unroll 2
-            for (int q = 0; q < 8; ++q) {
-                const int i = 8 * q + (lane >> 2), r = p.r0 + i, c = p.c0 + (lane & 3) * 16;
-                const u64 w0 = shfl64(f.x, i >> 1), w1 = shfl64(f.y, i >> 1);
-                const uint32_t m = (uint32_t)((i & 1 ? w1 : w0) >> ((lane & 3) * 16)) & 0xffffu;
-                const int n = r < d.H ? min(16, d.W - c) : 0;
-                if (n <= 0) continue;
-                uint8_t *o = d.filled + (int64_t)r * d.ld_filled + c;
-                if (n == 16 && ((uintptr_t)o & 15u) == 0) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) w[k] = (((m >> (4 * k)) & 0xfu) * 0x00204081u) & 0x01010101u;
-                    *reinterpret_cast<uint4 *>(o) = make_uint4(w[0], w[1], w[2], w[3]);
-                } else {
-                    for (int k = 0; k < n; ++k) o[k] = (uint8_t)((m >> k) & 1u);
-                }
-            }
-        }
-    }
-    if (LABEL) {
-        if (tile == d.tile_base && lane == 0 && d.n_kept) *d.n_kept = 0;
-        const uint32_t node = 1u + (uint32_t)tile * kRunSlots;
-        if (!__any_sync(0xffffffffu, (f.x | f.y) != 0ull)) {
-            uint16_t *s = reinterpret_cast<uint16_t *>(b.sides + (int64_t)tile * kRunSides) + lane;
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (p.open[k]) s[k * kRunSide / 2] = 0xffffu;
-            if (lane == 0) b.lcnt[tile] = 0u;
-            return;
-        }
-        const Runs r = components<LABEL ? LABEL : 8>(f.x, f.y, P, P + kMaxRuns, lane);
-        flag_rim(r, p, P, lane);
-        const int cnt = number_slots(r, P, lane, [&](int, int k) {
-            b.U[node + k] = mix(node + k);
-            b.A[node + k] = 0u;
-        });
-        write_sides(b, r, p, P, lane);
-        __syncwarp();
-        // areas: a slot's to its node, with its first pixel (a root run is its
-        // component's first), another component's to its root's upper bits
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            u64 s = r.st[j];
-            for (int k = 0; s; ++k, s &= s - 1) {
-                const int run = r.base[j] + k, pos = __ffsll((long long)s) - 1;
-                const uint32_t root = P[run] & kParent, v = P[root], area = (uint32_t)__popcll(run_bits(r.m[j], pos));
-                if (v & kRim) {
-                    const uint32_t slot = node + ((v >> kSlotShift) & kSlotMask);
-                    atomicAdd(b.A + slot, area);
-                    if (root == (uint32_t)run) b.M[slot] = (uint32_t)((int64_t)(p.r0 + 2 * lane + j) * d.W + p.c0 + pos);
-                } else {
-                    atomicAdd(const_cast<uint32_t *>(P + root), area << kSlotShift);
-                }
-            }
-        }
-        __syncwarp();
-        uint32_t *words = b.words + (int64_t)tile * kRunWords;
-        for (int i = lane; i < r.total; i += 32) words[i] = P[i];
-        if (lane == 0) b.lcnt[tile] = (uint8_t)cnt;
-    }
+    });
 }
 
 // ------------------------------------------------------------------- labels
@@ -632,118 +678,125 @@ __global__ void __launch_bounds__(256) run_roots_kernel(const __grid_constant__ 
 }
 
 // Warp per tile: labels with the area filter, kept bits and count, from the
-// run words of the local stage.
-__global__ void __launch_bounds__(kWarps * 32) run_label_kernel(const __grid_constant__ RunBatch b)
+// run words of the local stage, in shared memory or, where they do not fit in
+// a warp's share (!ALONE), in place: a block then never waits for one of its
+// warps (waiting for the block's memory as above: 122 us for eight 4096 x 4096
+// tiles instead of 102).
+template <bool ALONE>
+__global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_label_kernel(const __grid_constant__ RunBatch b)
 {
-    extern __shared__ uint32_t run_smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int tile = blockIdx.x * kWarps + warp;
+    const int lane = threadIdx.x & 31, at = blockIdx.x * (ALONE ? 1 : kWarps) + (threadIdx.x >> 5);
+    const int tile = at;
     if (tile >= b.ntiles) return;
-    volatile uint32_t *P = run_smem + warp * kWarpWords;
     const RunImage &d = run_image(b, tile);
     const Place p = place_of(d, tile);
     const ulonglong2 f = *(reinterpret_cast<const ulonglong2 *>(b.bits + (int64_t)tile * kRunSide) + lane);
-    // rows [i0, nr) of the tile: its share when several warps take a tile
-    const int share = kRunSide / (int)gridDim.y, i0 = (int)blockIdx.y * share;
-    const int nr = min(i0 + share, d.H - p.r0), c = p.c0 + 2 * lane;
-    int32_t *out = d.labels + (int64_t)p.r0 * d.ld_lab + c;
-    const bool both = c + 1 < d.W, one = c < d.W;
-    const bool wide = both && (((uintptr_t)d.labels | (uintptr_t)d.ld_lab * 4u) & 7u) == 0;
-    auto store = [&](int i, int32_t x, int32_t y) {
-        int32_t *o = out + (int64_t)i * d.ld_lab;
-        if (wide) {
-            *reinterpret_cast<int2 *>(o) = make_int2(x, y);
-        } else {
-            if (one) o[0] = x;
-            if (both) o[1] = y;
-        }
-    };
-    u64 keep[2] = {0ull, 0ull};
-    const uint32_t rows = __ballot_sync(0xffffffffu, f.x != 0ull), rows1 = __ballot_sync(0xffffffffu, f.y != 0ull);
-    if (!(rows | rows1)) {
+    auto label = [&](volatile uint32_t *P, bool in_place) {
+        // rows [i0, nr) of the tile: its share when several warps take a tile (one alone works in place)
+        const int share = in_place ? kRunSide : kRunSide / (int)gridDim.y, i0 = (int)blockIdx.y * share;
+        if (i0 >= kRunSide) return;
+        const int nr = min(i0 + share, d.H - p.r0), c = p.c0 + 2 * lane;
+        int32_t *out = d.labels + (int64_t)p.r0 * d.ld_lab + c;
+        const bool both = c + 1 < d.W, one = c < d.W;
+        const bool wide = both && (((uintptr_t)d.labels | (uintptr_t)d.ld_lab * 4u) & 7u) == 0;
+        auto store = [&](int i, int32_t x, int32_t y) {
+            int32_t *o = out + (int64_t)i * d.ld_lab;
+            if (wide) {
+                *reinterpret_cast<int2 *>(o) = make_int2(x, y);
+            } else {
+                if (one) o[0] = x;
+                if (both) o[1] = y;
+            }
+        };
+        u64 keep[2] = {0ull, 0ull};
+        const uint32_t rows = __ballot_sync(0xffffffffu, f.x != 0ull), rows1 = __ballot_sync(0xffffffffu, f.y != 0ull);
+        if (!(rows | rows1)) {
 #pragma unroll 4
-        for (int i = i0; i < nr; ++i) store(i, -1, -1);
-    } else {
-        const Runs r = runs_of(f.x, f.y, lane);
-        const uint32_t *words = b.words + (int64_t)tile * kRunWords;
-        for (int i = lane; i < r.total; i += 32) P[i] = words[i];
-        __syncwarp();
-        // roots' labels (in their lane's order), then every run's
-        int kept = 0;
-        const uint32_t node = 1u + (uint32_t)tile * kRunSlots;
+            for (int i = i0; i < nr; ++i) store(i, -1, -1);
+        } else {
+            const Runs r = runs_of(f.x, f.y, lane);
+            const uint32_t *words = b.words + (int64_t)tile * kRunWords;
+            for (int i = lane; i < r.total && !in_place; i += 32) P[i] = words[i];
+            __syncwarp();
+            // roots' labels (in their lane's order), then every run's
+            int kept = 0;
+            const uint32_t node = 1u + (uint32_t)tile * kRunSlots;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            u64 s = r.st[j];
-            for (int k = 0; s; ++k, s &= s - 1) {
-                const int run = r.base[j] + k;
-                const uint32_t v = P[run];
-                if ((v & kParent) != (uint32_t)run) continue;
-                int32_t area, label;
-                bool first = true;
-                if (v & kRim) {
-                    const uint32_t x = node + ((v >> kSlotShift) & kSlotMask), root = b.U[x] * kUnmix;
-                    area = (int32_t)b.A[root];
-                    label = (int32_t)b.M[root];
-                    first = root == x;
-                } else {
-                    area = (int32_t)(v >> kSlotShift);
-                    label = (int32_t)((int64_t)(p.r0 + 2 * lane + j) * d.W + p.c0 + __ffsll((long long)s) - 1);
+            for (int j = 0; j < 2; ++j) {
+                u64 s = r.st[j];
+                for (int k = 0; s; ++k, s &= s - 1) {
+                    const int run = r.base[j] + k;
+                    const uint32_t v = P[run];
+                    if ((v & kParent) != (uint32_t)run) continue;
+                    int32_t area, label;
+                    bool first = true;
+                    if (v & kRim) {
+                        const uint32_t x = node + ((v >> kSlotShift) & kSlotMask), root = b.U[x] * kUnmix;
+                        area = (int32_t)b.A[root];
+                        label = (int32_t)b.M[root];
+                        first = root == x;
+                    } else {
+                        area = (int32_t)(v >> kSlotShift);
+                        label = (int32_t)((int64_t)(p.r0 + 2 * lane + j) * d.W + p.c0 + __ffsll((long long)s) - 1);
+                    }
+                    const bool in = area >= b.amin && area <= b.amax;
+                    kept += in && first;
+                    P[run] = in ? (uint32_t)label | kRim : kBorder;   // a root's final word: kRim | label, or kBorder: dropped
                 }
-                const bool in = area >= b.amin && area <= b.amax;
-                kept += in && first;
-                P[run] = in ? (uint32_t)label | kRim : kBorder;   // a root's final word: kRim | label, or kBorder: dropped
             }
-        }
-        __syncwarp();
-        // every run takes its root's word; a root keeps its own (bit 31 or 30
-        // set marks final words, which others read through their parent)
+            __syncwarp();
+            // every run takes its root's word; a root keeps its own (bit 31 or 30
+            // set marks final words, which others read through their parent)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            u64 s = r.st[j];
-            for (int k = 0; s; ++k, s &= s - 1) {
-                const int run = r.base[j] + k;
-                const uint32_t v = P[run];
-                const uint32_t w = v & (kRim | kBorder) ? v : P[v];
-                if (w & kRim) keep[j] |= run_bits(r.m[j], __ffsll((long long)s) - 1);
+            for (int j = 0; j < 2; ++j) {
+                u64 s = r.st[j];
+                for (int k = 0; s; ++k, s &= s - 1) {
+                    const int run = r.base[j] + k;
+                    const uint32_t v = P[run];
+                    const uint32_t w = v & (kRim | kBorder) ? v : P[v];
+                    if (w & kRim) keep[j] |= run_bits(r.m[j], __ffsll((long long)s) - 1);
+                }
             }
-        }
-        __syncwarp();
-        kept = __reduce_add_sync(0xffffffffu, kept);
-        if (lane == 0 && kept && d.n_kept && i0 == 0) atomicAdd(d.n_kept, kept);
+            __syncwarp();
+            kept = __reduce_add_sync(0xffffffffu, kept);
+            if (lane == 0 && kept && d.n_kept && i0 == 0) atomicAdd(d.n_kept, kept);
 #pragma unroll 2
-        for (int i = i0; i < nr; ++i) {
-            int32_t v[2] = {-1, -1};
-            if (((i & 1 ? rows1 : rows) >> (i >> 1)) & 1u) {   // whole warp
-                const u64 m = shfl64(i & 1 ? f.y : f.x, i >> 1), st = m & ~(m << 1);
-                const int base = __shfl_sync(0xffffffffu, i & 1 ? r.base[1] : r.base[0], i >> 1);
+            for (int i = i0; i < nr; ++i) {
+                int32_t v[2] = {-1, -1};
+                if (((i & 1 ? rows1 : rows) >> (i >> 1)) & 1u) {   // whole warp
+                    const u64 m = shfl64(i & 1 ? f.y : f.x, i >> 1), st = m & ~(m << 1);
+                    const int base = __shfl_sync(0xffffffffu, i & 1 ? r.base[1] : r.base[0], i >> 1);
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int x = 2 * lane + q;
-                    if ((m >> x) & 1ull) {
-                        uint32_t w = P[base + __popcll(st & (~0ull >> (63 - x))) - 1];
-                        if (!(w & (kRim | kBorder))) w = P[w];
-                        if (w & kRim) v[q] = (int32_t)(w & ~kRim);
+                    for (int q = 0; q < 2; ++q) {
+                        const int x = 2 * lane + q;
+                        if ((m >> x) & 1ull) {
+                            uint32_t w = P[base + __popcll(st & (~0ull >> (63 - x))) - 1];
+                            if (!(w & (kRim | kBorder))) w = P[w];
+                            if (w & kRim) v[q] = (int32_t)(w & ~kRim);
+                        }
                     }
                 }
+                store(i, v[0], v[1]);
             }
-            store(i, v[0], v[1]);
         }
-    }
-    if (b.kept && i0 == 0)
-        *(reinterpret_cast<ulonglong2 *>(b.kept + (int64_t)tile * kRunSide) + lane) = make_ulonglong2(keep[0], keep[1]);
+        if (b.kept && i0 == 0)
+            *(reinterpret_cast<ulonglong2 *>(b.kept + (int64_t)tile * kRunSide) + lane) = make_ulonglong2(keep[0], keep[1]);
+    };
+    extern __shared__ uint32_t run_smem[];
+    if (ALONE || count_runs(f.x, f.y) <= kWarpWords) label(run_smem + (ALONE ? 0 : (threadIdx.x >> 5) * kWarpWords), false);
+    else label(b.words + (int64_t)tile * kRunWords, true);
 }
 
 // --------------------------------------------------------------------- host
 namespace {
 
-template <class K>
-cudaError_t warp_per_tile(K kernel, const RunBatch &b, size_t smem, cudaStream_t s)
+// `alone` while there are few tiles, else `four`; y: CTAs that share a tile.
+using RunKernel = void (*)(RunBatch);
+cudaError_t warp_per_tile(RunKernel alone, RunKernel four, const RunBatch &b, cudaStream_t s, int y = 1)
 {
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    kernel<<<(unsigned)ceil_div(b.ntiles, kWarps), kWarps * 32, smem, s>>>(b);
+    const bool few = b.ntiles <= kFewTiles;
+    const int w = few ? 1 : kWarps;
+    (few ? alone : four)<<<dim3((unsigned)ceil_div(b.ntiles, w), y), w * 32, kRunSmem, s>>>(b);
     return cudaGetLastError();
 }
 
@@ -781,19 +834,20 @@ cudaError_t launch_run_pack(const RunBatch &b, cudaStream_t s)
 cudaError_t launch_run_fill(const RunBatch &b, int conn, int label_conn, cudaStream_t s)
 {
     if ((conn != 4 && conn != 8) || (label_conn != 0 && label_conn != 8)) return cudaErrorInvalidValue;
-    cudaError_t e = conn == 8 ? warp_per_tile(run_fill_local_kernel<8>, b, kRunSmem, s)
-                              : warp_per_tile(run_fill_local_kernel<4>, b, kRunSmem, s);
+    cudaError_t e = conn == 8
+                        ? warp_per_tile(run_fill_local_kernel<8, true>, run_fill_local_kernel<8, false>, b, s)
+                        : warp_per_tile(run_fill_local_kernel<4, true>, run_fill_local_kernel<4, false>, b, s);
     if (e != cudaSuccess) return e;
     if ((e = launch_seam(b, conn, b.outside, s)) != cudaSuccess) return e;
-    return label_conn ? warp_per_tile(run_local_kernel<true, 8>, b, kRunSmem, s)
-                      : warp_per_tile(run_local_kernel<true, 0>, b, kRunSmem, s);
+    return label_conn ? warp_per_tile(run_local_kernel<true, 8, true>, run_local_kernel<true, 8, false>, b, s)
+                      : warp_per_tile(run_local_kernel<true, 0, true>, run_local_kernel<true, 0, false>, b, s);
 }
 
 cudaError_t launch_run_local(const RunBatch &b, int conn, cudaStream_t s)
 {
     if (conn != 4 && conn != 8) return cudaErrorInvalidValue;
-    return conn == 8 ? warp_per_tile(run_local_kernel<false, 8>, b, kRunSmem, s)
-                     : warp_per_tile(run_local_kernel<false, 4>, b, kRunSmem, s);
+    return conn == 8 ? warp_per_tile(run_local_kernel<false, 8, true>, run_local_kernel<false, 8, false>, b, s)
+                     : warp_per_tile(run_local_kernel<false, 4, true>, run_local_kernel<false, 4, false>, b, s);
 }
 
 cudaError_t launch_run_label(const RunBatch &b, int conn, cudaStream_t s)
@@ -804,10 +858,7 @@ cudaError_t launch_run_label(const RunBatch &b, int conn, cudaStream_t s)
     run_roots_kernel<<<(unsigned)ceil_div(b.ntiles, 8), 256, 0, s>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // few tiles: four warps write a tile's labels (a warp's 64 rows are 10 us of latency)
-    e = cudaFuncSetAttribute(run_label_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRunSmem);
-    if (e != cudaSuccess) return e;
-    run_label_kernel<<<dim3((unsigned)ceil_div(b.ntiles, kWarps), b.ntiles <= kFewTiles ? 4 : 1), kWarps * 32, kRunSmem, s>>>(b);
-    return cudaGetLastError();
+    return warp_per_tile(run_label_kernel<true>, run_label_kernel<false>, b, s, b.ntiles <= kFewTiles ? 4 : 1);
 }
 
 }  // namespace rtk

@@ -97,3 +97,17 @@ def test_many_tiles(rt):
         for conn in (4, 8):   # large enough for the union-find over runs
             got = host(rt.label_area(dev(m), 2, 2 ** 31 - 1, conn=conn))
             assert np.array_equal(got, oracle.label_area(m, 2, 2 ** 31 - 1, conn)), conn
+
+
+def test_tiles_around_a_warps_share_of_memory(rt):
+    """Tiles of 100 to 1000 runs side by side in an image large enough for
+    several tiles per block: 384 runs (local stages) and 640 (labels) fit a
+    warp's share, the others take another way."""
+    rng = np.random.default_rng(5)
+    p = np.kron(rng.uniform(0.03, 0.5, (47, 48)), np.ones((64, 64)))[:3000, :3070]
+    m = (rng.random(p.shape) < p).astype(np.uint8)
+    for conn in (4, 8):
+        assert np.array_equal(host(rt.fill_holes(dev(m), conn=conn)), oracle.fill_holes(m, conn)), conn
+        assert np.array_equal(host(rt.fill_holes(dev(1 - m), conn=conn)), oracle.fill_holes(1 - m, conn)), conn
+        got = host(rt.label_area(dev(m), 2, 400, conn=conn))
+        assert np.array_equal(got, oracle.label_area(m, 2, 400, conn)), conn
