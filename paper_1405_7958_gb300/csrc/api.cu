@@ -408,6 +408,16 @@ rt_status run_contract(rt_ctx *ctx, CtBatch &b, int32_t *err, cudaStream_t s, co
     return RT_OK;
 }
 
+// Enqueue what a call that does not return R needs of it.
+rt_status run_reach(rt_ctx *ctx, const RunBatch &b, cudaStream_t s)
+{
+    ctx->visits_dev = nullptr;   // no tile visits
+    Phase ph(ctx, RT_PHASE_RECON_SWEEP, s);
+    ctx->launches += 3;
+    RT_CUDA_TRY(launch_run_reach(b, s));
+    return RT_OK;
+}
+
 // Workspace of the hole filling and labeling stages: the bits first, then
 // what no stage before them uses (carve_runs_late).
 void carve_bits(Carve &cv, RunBatch &b) { b.bits = cv.take<unsigned long long>((size_t)b.ntiles * kRunSide); }
@@ -504,6 +514,7 @@ int32_t *take_edt_ctl(Carve &cv, EdtBitsBatch &b, size_t bands, int &words)
 constexpr size_t kWsBytesPerPx = 13;
 struct Chunk {
     bool contract = false;   // reconstruction by contraction (cb), else by propagation (b, w)
+    bool reach = false;      // with contract: no tile asks for R, so only where it is below the threshold is found
     CtBatch cb;
     ReconBatch b;
     ReconWs w;
@@ -575,6 +586,8 @@ void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, con
         if (c.contract) {   // B = (R < threshold) goes straight to the bits
             c.cb.img[i].out = t.recon;
             c.cb.img[i].ld_out = t.ld_recon;
+            u.in = t.img;
+            u.ld_in = t.ld_img;
         } else {
             uint8_t *B = cv.take<uint8_t>((size_t)t.H * t.W);
             ReconImage &d = c.b.img[i];
@@ -600,6 +613,13 @@ void layout_chunk(Carve &cv, Chunk &c, const rt_tile *tiles, int c0, int cn, con
     carve_runs_late(cv, c.rb, true, true);
     c.rb.kept = cv.take<unsigned long long>((size_t)c.rb.ntiles * kRunSide);
     c.eb.bits = c.rb.kept;
+    // R(p) >= t exactly where a path from a pixel q with J(q) >= t leads to p through pixels with I >= t. The seeds lie
+    // where the kept pixels will be.
+    c.reach = c.contract && real;
+    for (int i = 0; real && i < cn; ++i) c.reach = c.reach && !tiles[c0 + i].recon;
+    c.rb.seeds = c.rb.kept;
+    c.rb.lo = P.threshold;
+    c.rb.hi = P.threshold > 0 ? P.threshold + P.h_offset : 0;
     for (int i = 0; i < cn; ++i) {
         const rt_tile &t = tiles[c0 + i];
         char *ews = cv.take<char>(edt_bits_workspace_bytes(t.H, t.W));
@@ -1296,7 +1316,7 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
         RT_CUDA_TRY(zero_words(c.err, c.ctl_words, s));
         ctx->launches += 1;
         auto reconstruct = [&](const int32_t *pick) {
-            return c.contract ? run_contract(ctx, c.cb, c.err, s, lim)
+            return c.reach ? run_reach(ctx, c.rb, s) : c.contract ? run_contract(ctx, c.cb, c.err, s, lim)
                               : run_recon(ctx, c.b, c.w, P.conn_recon, P.variant, P.max_local, c.err, s, lim, pick);
         };
         bool aside = false;
@@ -1326,7 +1346,7 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
                 if (st != RT_OK) return st;
             }
         }
-        {
+        if (!c.reach) {
             Phase ph(ctx, RT_PHASE_RECON_OUT, s);
             ctx->launches += 1;
             RT_CUDA_TRY(c.contract ? launch_contract_out(c.cb, P.threshold, s) : launch_recon_out(c.b, P.threshold, s));
@@ -1334,7 +1354,7 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
         {
             Phase ph(ctx, RT_PHASE_FILL, s);
             if (!c.contract) RT_CUDA_TRY(launch_run_pack(c.rb, s));
-            RT_CUDA_TRY(launch_run_fill(c.rb, P.conn_fill, 8, s));
+            RT_CUDA_TRY(launch_run_fill(c.rb, P.conn_fill, 8, s, c.reach));
             ctx->launches += c.contract ? 3 : 4;
         }
         {

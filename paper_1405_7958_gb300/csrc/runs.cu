@@ -377,31 +377,116 @@ __device__ __forceinline__ void write_sides(const RunBatch &b, const Runs &r, co
 // The bits of the run that starts at pos (a first bit of m).
 __device__ __forceinline__ u64 run_bits(u64 m, int pos) { return m & ~(m + (1ull << pos)); }
 
-// Background components of a tile (foreground f0, f1), marked kRim and
-// kBorder (on the image border), the rim ones numbered.
-template <int CONN, bool ALONE, class F>
-__device__ __forceinline__ Runs background(const RunImage &d, const Place &p, u64 f0, u64 f1, const Mem<ALONE> &mem, int lane,
-                                           int &cnt, F &&f)
+// Background components of a tile (foreground f), marked kRim and kBorder
+// (on the image border, or SEEDS: with a pixel of seed), the rim ones
+// numbered.
+template <int CONN, bool SEEDS, bool ALONE, class F>
+__device__ __forceinline__ Runs background(const RunImage &d, const Place &p, ulonglong2 f, ulonglong2 seed,
+                                           const Mem<ALONE> &mem, int lane, int &cnt, F &&fn)
 {
     volatile uint32_t *P = mem.runs();
-    const Runs r = components<CONN>(exists(d, p, 2 * lane) & ~f0, exists(d, p, 2 * lane + 1) & ~f1, mem, lane);
-    if (p.ty == 0) flag_runs(P, 0, __shfl_sync(0xffffffffu, r.n[0], 0), kBorder, lane);
-    const int last = d.H - 1 - p.r0;
-    if (last < kRunSide) {   // whole warp
-        const int first = __shfl_sync(0xffffffffu, last & 1 ? r.base[1] : r.base[0], last >> 1);
-        const int n = __shfl_sync(0xffffffffu, last & 1 ? r.n[1] : r.n[0], last >> 1);
-        flag_runs(P, first, n, kBorder, lane);
-    }
-    const int right = d.W - 1 - p.c0;
+    const Runs r = components<CONN>(exists(d, p, 2 * lane) & ~f.x, exists(d, p, 2 * lane + 1) & ~f.y, mem, lane);
+    if (SEEDS) {
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        if (p.tx == 0 && (r.m[j] & 1ull)) atomicOr(const_cast<uint32_t *>(P + (P[r.base[j]] & kParent)), kBorder);
-        if (right < kRunSide && ((r.m[j] >> right) & 1ull))
-            atomicOr(const_cast<uint32_t *>(P + (P[r.id(j, right)] & kParent)), kBorder);
+        for (int j = 0; j < 2; ++j) {
+            u64 s = r.st[j];
+            for (int k = 0; s; ++k, s &= s - 1)
+                if (run_bits(r.m[j], __ffsll((long long)s) - 1) & (j ? seed.y : seed.x))
+                    atomicOr(const_cast<uint32_t *>(P + (P[r.base[j] + k] & kParent)), kBorder);
+        }
+    } else {
+        if (p.ty == 0) flag_runs(P, 0, __shfl_sync(0xffffffffu, r.n[0], 0), kBorder, lane);
+        const int last = d.H - 1 - p.r0;
+        if (last < kRunSide) {   // whole warp
+            const int first = __shfl_sync(0xffffffffu, last & 1 ? r.base[1] : r.base[0], last >> 1);
+            const int n = __shfl_sync(0xffffffffu, last & 1 ? r.n[1] : r.n[0], last >> 1);
+            flag_runs(P, first, n, kBorder, lane);
+        }
+        const int right = d.W - 1 - p.c0;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            if (p.tx == 0 && (r.m[j] & 1ull)) atomicOr(const_cast<uint32_t *>(P + (P[r.base[j]] & kParent)), kBorder);
+            if (right < kRunSide && ((r.m[j] >> right) & 1ull))
+                atomicOr(const_cast<uint32_t *>(P + (P[r.id(j, right)] & kParent)), kBorder);
+        }
     }
     flag_rim(r, p, P, lane);
-    cnt = number_slots(r, P, lane, f);
+    cnt = number_slots(r, P, lane, fn);
     return r;
+}
+
+// The local stage of a fill in forest U: holes inside the tile are known
+// afterwards (words), the other background components become slots.
+template <int CONN, bool SEEDS, bool ALONE>
+__device__ __forceinline__ void fill_tile(const RunBatch &b, uint32_t *U, const RunImage &d, const Place &p, ulonglong2 f,
+                                          ulonglong2 seed, const Mem<ALONE> &mem, int lane)
+{
+    const uint32_t node = 1u + (uint32_t)p.tile * kRunSlots;
+    if (p.tile == 0 && lane == 0) U[0] = 0u;
+    if (!__any_sync(0xffffffffu, (f.x | f.y) != 0ull)) {   // nothing but background (no words): one component
+        const bool border = SEEDS ? __any_sync(0xffffffffu, (seed.x | seed.y) != 0ull)
+                                  : p.ty == 0 || p.tx == 0 || p.r0 + kRunSide >= d.H || p.c0 + kRunSide >= d.W;
+        const bool rim = p.open[0] || p.open[1] || p.open[2] || p.open[3];
+        uint16_t *s = reinterpret_cast<uint16_t *>(b.sides + (int64_t)p.tile * kRunSides) + lane;
+        const int nr = min(kRunSide, d.H - p.r0), nc = min(kRunSide, d.W - p.c0);
+        auto pair = [&](int n) { return (uint16_t)((2 * lane < n ? 0u : 255u) | (2 * lane + 1 < n ? 0u : 255u) << 8); };
+        if (p.open[0]) s[0] = pair(nc);
+        if (p.open[1]) s[kRunSide / 2] = pair(nc);
+        if (p.open[2]) s[2 * kRunSide / 2] = pair(nr);
+        if (p.open[3]) s[3 * kRunSide / 2] = pair(nr);
+        if (lane == 0) {
+            b.cnt[p.tile] = rim ? 1u : 0u;   // no neighbour: the whole image, whose border is outside
+            if (rim) U[node] = border ? 0u : mix(node);
+        }
+        return;
+    }
+    volatile uint32_t *P = mem.runs();
+    int cnt = 0;
+    const Runs r = background<CONN, SEEDS>(d, p, f, seed, mem, lane, cnt, [&](int i, int k) {
+        U[node + k] = P[i] & kBorder ? 0u : mix(node + k);
+    });
+    uint32_t *words = b.words + (int64_t)p.tile * kRunWords;
+    for (int i = lane; i < r.total; i += 32) words[i] = P[i];
+    write_sides(b, r, p, P, lane);
+    if (lane == 0) b.cnt[p.tile] = (uint8_t)cnt;
+}
+
+// The holes of the fill in U: components that neither are outside in the tile
+// nor reach it through their slot. From fill_tile's words.
+template <bool ALONE>
+__device__ __forceinline__ ulonglong2 holes_of(const RunBatch &b, uint32_t *U, const RunImage &d, const Place &p,
+                                               ulonglong2 f, const Mem<ALONE> &mem, int lane)
+{
+    const uint32_t node = 1u + (uint32_t)p.tile * kRunSlots;
+    u64 add[2] = {0ull, 0ull};
+    if (!__any_sync(0xffffffffu, (f.x | f.y) != 0ull)) {
+        if (b.cnt[p.tile] && node_find(U, mix(node)) != 0u) {
+            add[0] = exists(d, p, 2 * lane);
+            add[1] = exists(d, p, 2 * lane + 1);
+        }
+    } else {
+        volatile uint32_t *P = mem.runs();
+        const Runs r = runs_of(exists(d, p, 2 * lane) & ~f.x, exists(d, p, 2 * lane + 1) & ~f.y, lane);
+        const uint32_t *words = b.words + (int64_t)p.tile * kRunWords;
+        for (int i = lane; i < r.total; i += 32) {
+            uint32_t v = words[i];
+            if ((v & kParent) == (uint32_t)i) {   // roots: kBorder if outside
+                if ((v & kRim) && node_find(U, mix(node + ((v >> kSlotShift) & kSlotMask))) == 0u) v |= kBorder;
+                v = (v & kBorder) | (uint32_t)i;
+            }
+            P[i] = v;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            u64 s = r.st[j];
+            for (int k = 0; s; ++k, s &= s - 1)
+                if (!(P[P[r.base[j] + k] & kParent] & kBorder))
+                    add[j] |= run_bits(r.m[j], __ffsll((long long)s) - 1);
+        }
+        __syncwarp();
+    }
+    return make_ulonglong2(add[0], add[1]);
 }
 
 }  // namespace
@@ -431,10 +516,57 @@ __global__ void __launch_bounds__(256) run_pack_kernel(const __grid_constant__ R
     reinterpret_cast<uint16_t *>(b.bits + (int64_t)tile * kRunSide)[t] = (uint16_t)m;
 }
 
+// Bit 8 k + 7: byte k of v is at least t (0 <= t <= 255).
+__device__ __forceinline__ uint32_t at_least(uint32_t v, uint32_t t)
+{
+    const uint32_t low = ((v & 0x7f7f7f7fu) | 0x80808080u) - (t & 0x7fu) * 0x01010101u;
+    return (t < 128u ? v | low : v & low) & 0x80808080u;
+}
+
+// CTA per tile, thread = 16 columns of a row: bits = (I < lo) and seeds = (J
+// >= lo), J the chain's marker: I >= hi, or I >= lo on the image border.
+__global__ void __launch_bounds__(256) run_threshold_kernel(const __grid_constant__ RunBatch b)
+{
+    const int tile = blockIdx.x, t = threadIdx.x;
+    const RunImage &d = run_image(b, tile);
+    const int lt = tile - d.tile_base;
+    const int ty = lt / d.nx, tx = lt - ty * d.nx;
+    const int r = ty * kRunSide + (t >> 2), c = tx * kRunSide + (t & 3) * 16;
+    const int n = r < d.H ? min(16, d.W - c) : 0;   // may be negative: none
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+    const uint8_t *p = d.in + (int64_t)r * d.ld_in + c;
+    if (n == 16 && ((uintptr_t)p & 15u) == 0) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+        w[0] = v.x;
+        w[1] = v.y;
+        w[2] = v.z;
+        w[3] = v.w;
+    } else {
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (k < n) w[k >> 2] |= (uint32_t)__ldg(p + k) << (8 * (k & 3));
+    }
+    uint32_t m = 0, sd = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {   // four flags of a word to a nibble: no two products of the multiplication meet
+        m |= ((at_least(w[q], (uint32_t)min(b.lo, 255)) >> 7) * 0x10204080u >> 28) << (4 * q);
+        sd |= ((at_least(w[q], (uint32_t)min(b.hi, 255)) >> 7) * 0x10204080u >> 28) << (4 * q);
+    }
+    const uint32_t in = n >= 16 ? 0xffffu : n > 0 ? (1u << n) - 1u : 0u;
+    m = b.lo > 255 ? 0u : m & in;
+    sd = b.hi > 255 ? 0u : sd & in;
+    uint32_t border = r == 0 || r == d.H - 1 ? 0xffffu : 0u;
+    if (c == 0) border |= 1u;
+    if (d.W - 1 - c < 16 && d.W - 1 >= c) border |= 1u << (d.W - 1 - c);
+    sd |= border & m;
+    reinterpret_cast<uint16_t *>(b.bits + (int64_t)tile * kRunSide)[t] = (uint16_t)(in & ~m);
+    reinterpret_cast<uint16_t *>(b.seeds + (int64_t)tile * kRunSide)[t] = (uint16_t)sd;
+}
+
 // --------------------------------------------------------------------- fill
-// Warp per tile: holes inside the tile are filled; the other background
-// components become slots.
-template <int CONN, bool ALONE>
+// Warp per tile: the local stage of a fill. AGAIN: after the fill of the
+// unreached parts (b.U), whose holes join the foreground first.
+template <int CONN, bool SEEDS, bool AGAIN, bool ALONE>
 __global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_fill_local_kernel(const __grid_constant__ RunBatch b)
 {
     const int lane = threadIdx.x & 31, at = blockIdx.x * (ALONE ? 1 : kWarps) + (threadIdx.x >> 5);
@@ -442,39 +574,21 @@ __global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_fill_local_kerne
     const int tile = mine ? at : 0;
     const RunImage &d = run_image(b, tile);
     const Place p = place_of(d, tile);
-    const uint32_t node = 1u + (uint32_t)tile * kRunSlots;
-    const ulonglong2 f = *(reinterpret_cast<const ulonglong2 *>(b.bits + (int64_t)tile * kRunSide) + lane);
-    with_memory<ALONE>(count_runs(exists(d, p, 2 * lane) & ~f.x, exists(d, p, 2 * lane + 1) & ~f.y), [&](const Mem<ALONE> &mem) {
+    ulonglong2 *row = reinterpret_cast<ulonglong2 *>(b.bits + (int64_t)tile * kRunSide) + lane;
+    const ulonglong2 f = *row;
+    ulonglong2 seed = make_ulonglong2(0ull, 0ull);
+    if (SEEDS) seed = *(reinterpret_cast<const ulonglong2 *>(b.seeds + (int64_t)tile * kRunSide) + lane);
+    // (AGAIN: what stays of the background is some of its runs)
+    with_memory<ALONE>(count_runs(exists(d, p, 2 * lane) & ~f.x, exists(d, p, 2 * lane + 1) & ~f.y),
+                       [&](const Mem<ALONE> &mem) {
         if (!mine) return;
-        if (!__any_sync(0xffffffffu, (f.x | f.y) != 0ull)) {   // nothing but background (no words): one component
-            const bool border = p.ty == 0 || p.tx == 0 || p.r0 + kRunSide >= d.H || p.c0 + kRunSide >= d.W;
-            const bool rim = p.open[0] || p.open[1] || p.open[2] || p.open[3];
-            uint16_t *s = reinterpret_cast<uint16_t *>(b.sides + (int64_t)tile * kRunSides) + lane;
-            const int nr = min(kRunSide, d.H - p.r0), nc = min(kRunSide, d.W - p.c0);
-            auto pair = [&](int n) { return (uint16_t)((2 * lane < n ? 0u : 255u) | (2 * lane + 1 < n ? 0u : 255u) << 8); };
-            if (p.open[0]) s[0] = pair(nc);
-            if (p.open[1]) s[kRunSide / 2] = pair(nc);
-            if (p.open[2]) s[2 * kRunSide / 2] = pair(nr);
-            if (p.open[3]) s[3 * kRunSide / 2] = pair(nr);
-            if (lane == 0) {
-                b.cnt[tile] = rim ? 1u : 0u;
-                if (rim) b.outside[node] = border ? 0u : mix(node);
-                if (tile == 0) b.outside[0] = 0u;
-            }
-            return;
+        ulonglong2 g = f;
+        if (AGAIN) {
+            const ulonglong2 add = holes_of(b, b.U, d, p, f, mem, lane);
+            g = make_ulonglong2(f.x | add.x, f.y | add.y);
+            if (__any_sync(0xffffffffu, (add.x | add.y) != 0ull)) *row = g;
         }
-        int cnt = 0;
-        volatile uint32_t *P = mem.runs();
-        const Runs r = background<CONN>(d, p, f.x, f.y, mem, lane, cnt, [&](int i, int k) {
-            b.outside[node + k] = P[i] & kBorder ? 0u : mix(node + k);
-    });
-    uint32_t *words = b.words + (int64_t)tile * kRunWords;
-    for (int i = lane; i < r.total; i += 32) words[i] = P[i];
-    write_sides(b, r, p, P, lane);
-    if (lane == 0) {
-        b.cnt[tile] = (uint8_t)cnt;
-        if (tile == 0) b.outside[0] = 0u;
-    }
+        fill_tile<CONN, SEEDS>(b, SEEDS ? b.U : b.outside, d, p, g, seed, mem, lane);
     });
 }
 
@@ -563,37 +677,9 @@ __global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_local_kernel(con
         if (!mine) return;
         volatile uint32_t *P = mem.runs();
         if (FILL) {
-            // holes: components that neither touch the image border nor reach it
-            // through their slot
-            const uint32_t node = 1u + (uint32_t)tile * kRunSlots;
-            u64 add[2] = {0ull, 0ull};
-            if (!__any_sync(0xffffffffu, (f.x | f.y) != 0ull)) {
-                if (b.cnt[tile] && node_find(b.outside, mix(node)) != 0u) {
-                    add[0] = exists(d, p, 2 * lane);
-                    add[1] = exists(d, p, 2 * lane + 1);
-                }
-            } else {
-                const Runs r = runs_of(exists(d, p, 2 * lane) & ~f.x, exists(d, p, 2 * lane + 1) & ~f.y, lane);
-                const uint32_t *words = b.words + (int64_t)tile * kRunWords;
-                for (int i = lane; i < r.total; i += 32) {
-                    uint32_t v = words[i];
-                    if ((v & kParent) == (uint32_t)i) {   // roots: kBorder if outside
-                        if ((v & kRim) && node_find(b.outside, mix(node + ((v >> kSlotShift) & kSlotMask))) == 0u) v |= kBorder;
-                        v = (v & kBorder) | (uint32_t)i;
-                    }
-                    P[i] = v;
-                }
-                __syncwarp();
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    u64 s = r.st[j];
-                    for (int k = 0; s; ++k, s &= s - 1)
-                        if (!(P[P[r.base[j] + k] & kParent] & kBorder)) add[j] |= run_bits(r.m[j], __ffsll((long long)s) - 1);
-                }
-                __syncwarp();
-            }
-            if (__any_sync(0xffffffffu, (add[0] | add[1]) != 0ull)) {
-                f = make_ulonglong2(f.x | add[0], f.y | add[1]);
+            const ulonglong2 add = holes_of(b, b.outside, d, p, f, mem, lane);
+            if (__any_sync(0xffffffffu, (add.x | add.y) != 0ull)) {
+                f = make_ulonglong2(f.x | add.x, f.y | add.y);
                 *row = f;
             }
             if (d.filled) {
@@ -831,12 +917,25 @@ cudaError_t launch_run_pack(const RunBatch &b, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_run_fill(const RunBatch &b, int conn, int label_conn, cudaStream_t s)
+cudaError_t launch_run_reach(const RunBatch &b, cudaStream_t s)
+{
+    run_threshold_kernel<<<(unsigned)b.ntiles, 256, 0, s>>>(b);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    e = warp_per_tile(run_fill_local_kernel<8, true, false, true>, run_fill_local_kernel<8, true, false, false>, b, s);
+    return e != cudaSuccess ? e : launch_seam(b, 8, b.U, s);
+}
+
+cudaError_t launch_run_fill(const RunBatch &b, int conn, int label_conn, cudaStream_t s, bool again)
 {
     if ((conn != 4 && conn != 8) || (label_conn != 0 && label_conn != 8)) return cudaErrorInvalidValue;
-    cudaError_t e = conn == 8
-                        ? warp_per_tile(run_fill_local_kernel<8, true>, run_fill_local_kernel<8, false>, b, s)
-                        : warp_per_tile(run_fill_local_kernel<4, true>, run_fill_local_kernel<4, false>, b, s);
+    cudaError_t e;
+    if (conn == 8)
+        e = again ? warp_per_tile(run_fill_local_kernel<8, false, true, true>, run_fill_local_kernel<8, false, true, false>, b, s)
+                  : warp_per_tile(run_fill_local_kernel<8, false, false, true>, run_fill_local_kernel<8, false, false, false>, b, s);
+    else
+        e = again ? warp_per_tile(run_fill_local_kernel<4, false, true, true>, run_fill_local_kernel<4, false, true, false>, b, s)
+                  : warp_per_tile(run_fill_local_kernel<4, false, false, true>, run_fill_local_kernel<4, false, false, false>, b, s);
     if (e != cudaSuccess) return e;
     if ((e = launch_seam(b, conn, b.outside, s)) != cudaSuccess) return e;
     return label_conn ? warp_per_tile(run_local_kernel<true, 8, true>, run_local_kernel<true, 8, false>, b, s)

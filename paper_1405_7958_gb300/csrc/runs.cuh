@@ -17,7 +17,7 @@ constexpr int kRunMaxImgs = 32;
 // One image. Tiles are numbered row by row from tile_base.
 struct RunImage {
     int H, W, nx, ny, tile_base;
-    const uint8_t *in;     // byte image to pack (nonzero = foreground), stride ld_in; NULL: bits are given
+    const uint8_t *in;     // byte image to pack (nonzero = foreground) or to threshold, stride ld_in; NULL: bits are given
     int64_t ld_in;
     uint8_t *filled;       // nullable: F as bytes 0/1, stride ld_filled
     int64_t ld_filled;
@@ -31,6 +31,8 @@ struct RunBatch {
     int n, ntiles;
     int32_t amin, amax;              // area range kept, inclusive
     unsigned long long *bits;        // per tile: 64 rows, bit = column; foreground
+    unsigned long long *seeds;       // the same layout, launch_run_reach: pixels the marker reaches by itself
+    int lo, hi;                      // launch_run_reach: threshold, and threshold + marker offset (>= 0)
     unsigned long long *kept;        // nullable: the kept pixels, in the same layout
     uint8_t *sides;                  // per tile: slot (255: none) of the top, bottom, left, right pixels
     uint8_t *cnt;                    // per tile: slots of the fill's background components
@@ -46,10 +48,14 @@ size_t run_tiles(int H, int W);
 RunImage &run_add(RunBatch &b, int H, int W);
 // byte images -> bits
 cudaError_t launch_run_pack(const RunBatch &b, cudaStream_t s);
+// bits = (R < lo) for the reconstruction R by dilation of the chain's marker
+// under the images, 8-connected, but for the last step, which launch_run_fill
+// takes with again = true: the part of bits that its fill adds first
+cudaError_t launch_run_reach(const RunBatch &b, cudaStream_t s);
 // Holes filled in bits (and filled written); conn 4 or 8 is the background's
 // connectivity. With label_conn (4, 8; 0: none) the last launch also makes
 // the local components that launch_run_label needs.
-cudaError_t launch_run_fill(const RunBatch &b, int conn, int label_conn, cudaStream_t s);
+cudaError_t launch_run_fill(const RunBatch &b, int conn, int label_conn, cudaStream_t s, bool again = false);
 // local components of bits, where launch_run_fill has not made them
 cudaError_t launch_run_local(const RunBatch &b, int conn, cudaStream_t s);
 // labels with the area filter, counts and kept bits
