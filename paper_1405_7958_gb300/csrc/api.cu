@@ -170,11 +170,12 @@ rt_status cuda_status(cudaError_t e)
 // behind the caller's copies on a copy engine.
 __global__ void zero_words_kernel(uint32_t *p, int n)
 {
+    start_early();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0u;
 }
 cudaError_t zero_words(void *p, int n, cudaStream_t s)
 {
-    zero_words_kernel<<<(n + 255) / 256 < 16 ? (n + 255) / 256 : 16, 256, 0, s>>>(static_cast<uint32_t *>(p), n);
+    launch_early(zero_words_kernel, (n + 255) / 256 < 16 ? (n + 255) / 256 : 16, 256, 0, s, static_cast<uint32_t *>(p), n);
     return cudaGetLastError();
 }
 
@@ -459,6 +460,7 @@ struct StatusOut {
 };
 __global__ void copy_status_kernel(const int32_t *src, StatusOut o, int n)
 {
+    start_early();
     if ((int)threadIdx.x < n && o.dst[threadIdx.x]) *o.dst[threadIdx.x] = *src;
 }
 
@@ -1382,7 +1384,7 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
             any_status |= so.dst[i] != nullptr;
         }
         if (any_status) {
-            copy_status_kernel<<<1, 32, 0, s>>>(c.err, so, cn);
+            launch_early(copy_status_kernel, 1, 32, 0, s, c.err, so, cn);
             ctx->launches += 1;
             RT_CUDA_TRY(cudaGetLastError());
         }

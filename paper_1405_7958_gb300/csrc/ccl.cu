@@ -277,6 +277,7 @@ __device__ __forceinline__ int32_t global_index(const UfImage &d, int bx, int by
 template <int CONN>
 __global__ void __launch_bounds__(kThreads) uf_local_kernel(UfBatch b)
 {
+    start_early();
     __shared__ int P[kB * kB];
     __shared__ int cnt[kB * kB];
     __shared__ uint32_t M[kB];
@@ -354,6 +355,7 @@ __global__ void __launch_bounds__(kThreads) uf_local_kernel(UfBatch b)
 template <int CONN>
 __global__ void __launch_bounds__(96) uf_border_kernel(UfBatch b)
 {
+    start_early();
     const BlockRef br = find_block(b, blockIdx.x);
     const UfImage &d = *br.d;
     const int bx = br.bx, by = br.by, nbx = d.nbx;
@@ -399,6 +401,7 @@ __global__ void __launch_bounds__(96) uf_border_kernel(UfBatch b)
 // over the block's listed roots (four blocks per CTA)
 __global__ void __launch_bounds__(128) uf_roots_kernel(UfBatch b)
 {
+    start_early();
     const int64_t g = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
     if (g >= b.nblk) return;
     const int lane = threadIdx.x & 31;
@@ -421,6 +424,7 @@ __global__ void __launch_bounds__(128) uf_roots_kernel(UfBatch b)
 // the labels leave in 16-byte stores where the row allows them.
 __global__ void __launch_bounds__(kThreads) uf_labels_kernel(UfBatch b)
 {
+    start_early();
     const BlockRef br = find_block(b, blockIdx.x);
     const UfImage &d = *br.d;
     const int q = threadIdx.x & 7, lr = threadIdx.x >> 3;
@@ -465,16 +469,16 @@ cudaError_t launch_label_batch(const UfBatch &b, int conn, cudaStream_t s)
 {
     if (b.n < 1 || b.n > kUfMaxImgs || (conn != 4 && conn != 8)) return cudaErrorInvalidValue;
     const unsigned nb = (unsigned)b.nblk;
-    if (conn == 8) uf_local_kernel<8><<<nb, kThreads, 0, s>>>(b);
-    else uf_local_kernel<4><<<nb, kThreads, 0, s>>>(b);
+    if (conn == 8) launch_early(uf_local_kernel<8>, nb, kThreads, 0, s, b);
+    else launch_early(uf_local_kernel<4>, nb, kThreads, 0, s, b);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (conn == 8) uf_border_kernel<8><<<nb, 96, 0, s>>>(b);
-    else uf_border_kernel<4><<<nb, 96, 0, s>>>(b);
+    if (conn == 8) launch_early(uf_border_kernel<8>, nb, 96, 0, s, b);
+    else launch_early(uf_border_kernel<4>, nb, 96, 0, s, b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    uf_roots_kernel<<<(unsigned)ceil_div(b.nblk, 4), 128, 0, s>>>(b);
+    launch_early(uf_roots_kernel, (unsigned)ceil_div(b.nblk, 4), 128, 0, s, b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    uf_labels_kernel<<<nb, kThreads, 0, s>>>(b);
+    launch_early(uf_labels_kernel, nb, kThreads, 0, s, b);
     return cudaGetLastError();
 }
 

@@ -80,6 +80,81 @@ __device__ __forceinline__ bool grid_barrier(uint32_t *bar, uint32_t nblocks, in
     return s_ok != 0;
 }
 
+// 16 bytes of a row of W bytes from column c, of which n exist (<= 0: none;
+// the others are 0). Rows that are not 16-byte aligned: the aligned words
+// around them, shifted, while these lie in the row; else byte by byte.
+__device__ __forceinline__ void load_row16(const uint8_t *row, int c, int n, int W, uint32_t (&w)[4])
+{
+    const uint8_t *p = row + c;
+    const uint32_t off = (uint32_t)(uintptr_t)p & 3u;
+    w[0] = w[1] = w[2] = w[3] = 0u;
+    if (n == 16 && ((uintptr_t)p & 15u) == 0) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+        w[0] = v.x;
+        w[1] = v.y;
+        w[2] = v.z;
+        w[3] = v.w;
+    } else if (n == 16 && (off == 0 || (c >= 4 && c + 20 <= W))) {
+        const uint32_t *q = reinterpret_cast<const uint32_t *>(p - off);
+        uint32_t v[5];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = __ldg(q + k);
+        v[4] = off ? __ldg(q + 4) : 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = __funnelshift_r(v[k], v[k + 1], 8u * off);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (k < n) w[k >> 2] |= (uint32_t)__ldg(p + k) << (8 * (k & 3));
+    }
+}
+
+// The first n of 4 N bytes (w) to o, in the widest stores its alignment allows.
+template <int N>
+__device__ __forceinline__ void store_bytes(uint8_t *o, int n, const uint32_t (&w)[N])
+{
+    if (n == 4 * N && ((uintptr_t)o & 15u) == 0) {
+#pragma unroll
+        for (int k = 0; k < N / 4; ++k)
+            reinterpret_cast<uint4 *>(o)[k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+    } else if (n == 4 * N && ((uintptr_t)o & 3u) == 0) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) reinterpret_cast<uint32_t *>(o)[k] = w[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4 * N; ++k)
+            if (k < n) o[k] = (uint8_t)(w[k >> 2] >> (8 * (k & 3)));
+    }
+}
+
+// First statement of a kernel launched by launch_early: lets the next such
+// kernel of the stream take its place on the SMs as soon as all blocks of
+// this one have theirs, and waits until the kernels before this one are
+// complete and their writes visible.
+__device__ __forceinline__ void start_early()
+{
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+
+// kernel<<<grid, block, smem, s>>>(args...) whose blocks may be placed before
+// the stream's previous kernel has ended (they wait in start_early), so that
+// the launch's latency lies behind it: XXPDL
+template <class... P, class... A>
+inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 __host__ __device__ __forceinline__ int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 __host__ __device__ __forceinline__ int64_t round_up(int64_t a, int64_t b) { return ceil_div(a, b) * b; }
 

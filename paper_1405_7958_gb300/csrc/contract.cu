@@ -149,6 +149,7 @@ __device__ __forceinline__ uint32_t max3(uint32_t a, uint32_t b, uint32_t c) { r
 template <bool MARKER, int NT>
 __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const __grid_constant__ CtBatch b)
 {
+    start_early();
     constexpr int kWarps = NT / 32, kRows = kCtSide / kWarps, kPer = kRoots / NT;
     extern __shared__ __align__(16) uint32_t ct_smem[];
     uint32_t *W = ct_smem;                      // pixel words
@@ -193,15 +194,17 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
     for (int i = t; i < kCodes * 256 / 8; i += NT)
         reinterpret_cast<uint4 *>(table)[i] = __ldg(reinterpret_cast<const uint4 *>(kGroupTable.v) + i);
     {
-        const bool wide = (((uintptr_t)d.mask | (uintptr_t)d.ld_mask) & 3u) == 0;
         const int c = c0 + 4 * (t & 15);
 #pragma unroll
         for (int rr = t >> 4; rr < kCtSide; rr += NT / 16) {
             const int r = r0 + rr, n = r < d.H ? min(4, d.W - c) : 0;   // may be negative: none
             uint32_t v = 0;
             const uint8_t *p = d.mask + (int64_t)r * d.ld_mask + c;
-            if (n == 4 && wide) {
-                v = __ldg(reinterpret_cast<const uint32_t *>(p));
+            const uint32_t off = (uint32_t)(uintptr_t)p & 3u;
+            if (n == 4 && (off == 0 || (c >= 4 && c + 8 <= d.W))) {   // the aligned words around them, in the row
+                const uint32_t *q = reinterpret_cast<const uint32_t *>(p - off);
+                v = __ldg(q);
+                if (off) v = __funnelshift_r(v, __ldg(q + 1), 8u * off);
             } else {
 #pragma unroll 1
                 for (int k = 0; k < n; ++k) v |= (uint32_t)__ldg(p + k) << (8 * k);
@@ -782,6 +785,7 @@ __device__ __forceinline__ unsigned long long edge_key(int round, uint32_t w, ui
 // 240 us of 505 for eight 4096 x 4096 tiles; this kernel takes 15 per tile.)
 __global__ void __launch_bounds__(kCtUnits * 32) ct_seam_kernel(const __grid_constant__ CtBatch b)
 {
+    start_early();
     __shared__ __align__(16) uint32_t bw[3 * kCtNodes], bg[3 * kCtNodes];
     const int tile = blockIdx.x, t = threadIdx.x, lane = t & 31, part = t >> 5;
     const uint32_t all = 0xffffffffu, below = (1u << lane) - 1u;
@@ -1160,6 +1164,7 @@ __global__ void __launch_bounds__(kGT, 1) ct_global_kernel(const __grid_constant
 constexpr int kOutThreads = 128;
 __global__ void __launch_bounds__(kOutThreads) ct_out_kernel(const __grid_constant__ CtBatch b, int threshold)
 {
+    start_early();
     __shared__ uint8_t val[kCtNodes];
     const int tile = blockIdx.x, t = threadIdx.x;
     const uint4 *src = reinterpret_cast<const uint4 *>(b.plane + (int64_t)tile * kCtPx + t * 32);
@@ -1197,15 +1202,24 @@ __global__ void __launch_bounds__(kOutThreads) ct_out_kernel(const __grid_consta
     }
     // nothing past the image
     if (b.bits) reinterpret_cast<uint32_t *>(b.bits + (int64_t)tile * kCtSide)[t] = n >= 32 ? B : n > 0 ? B & ((1u << n) - 1u) : 0u;
-    if (!d.out || n <= 0) return;
+    if (!d.out) return;
+    const uint32_t next = __shfl_down_sync(0xffffffffu, R[0], 1);   // half a row further
+    if (n <= 0) return;
     uint8_t *o = d.out + (int64_t)r * d.ld_out + c;
-    if (n == 32 && ((uintptr_t)o & 15u) == 0) {
-        reinterpret_cast<uint4 *>(o)[0] = make_uint4(R[0], R[1], R[2], R[3]);
-        reinterpret_cast<uint4 *>(o)[1] = make_uint4(R[4], R[5], R[6], R[7]);
-    } else {
+    const int head = (int)(-(uintptr_t)o & 3u);
+    if (head && d.W - tx * kCtSide >= kCtSide) {   // the row's aligned words, shifted together; its ends by bytes
+        const bool first = (t & 1) == 0;
 #pragma unroll
-        for (int k = 0; k < 32; ++k)
-            if (k < n) o[k] = (uint8_t)(R[k >> 2] >> (8 * (k & 3)));
+        for (int k = 0; k < 8; ++k)
+            if (k < 7 || first)
+                *reinterpret_cast<uint32_t *>(o + head + 4 * k) = __funnelshift_r(R[k], k < 7 ? R[k + 1 < 8 ? k + 1 : 7] : next, 8u * head);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (first && k < head) o[k] = (uint8_t)(R[0] >> (8 * k));
+            if (!first && k >= head) o[28 + k] = (uint8_t)(R[7] >> (8 * k));
+        }
+    } else {
+        store_bytes(o, n, R);
     }
 }
 
@@ -1240,9 +1254,9 @@ cudaError_t launch_contract(const CtBatch &b, int num_sms, uint64_t timeout_ns, 
                    : (given ? ct_local_kernel<true, 256> : ct_local_kernel<false, 256>);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLocalSmem);
     if (e != cudaSuccess) return e;
-    fn<<<(unsigned)b.ntiles, few ? 512 : 256, kLocalSmem, s>>>(b);
+    launch_early(fn, (unsigned)b.ntiles, few ? 512 : 256, kLocalSmem, s, b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    ct_seam_kernel<<<(unsigned)b.ntiles, kCtUnits * 32, 0, s>>>(b);
+    launch_early(ct_seam_kernel, (unsigned)b.ntiles, kCtUnits * 32, 0, s, b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int64_t units = (int64_t)b.ntiles * kCtUnits;
     const int need = (int)ceil_div(units, kGT / 32);
@@ -1270,7 +1284,7 @@ cudaError_t launch_contract(const CtBatch &b, int num_sms, uint64_t timeout_ns, 
 
 cudaError_t launch_contract_out(const CtBatch &b, int threshold, cudaStream_t s)
 {
-    ct_out_kernel<<<(unsigned)b.ntiles, kOutThreads, 0, s>>>(b, threshold);
+    launch_early(ct_out_kernel, (unsigned)b.ntiles, kOutThreads, 0, s, b, threshold);
     return cudaGetLastError();
 }
 

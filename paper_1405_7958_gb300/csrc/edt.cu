@@ -215,6 +215,7 @@ void edt_bits_add(EdtBitsBatch &b, int H, int W, int32_t *d2, int64_t ld_d2, cha
 // ------------------------------------------------------------------- near
 __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const __grid_constant__ EdtBitsBatch b)
 {
+    start_early();
     __shared__ uint32_t bg[kRowsIn][kRowWords + 1];   // background bits of rows and columns -32 .. 95
     __shared__ uint16_t list[kEdtSide * kEdtSide];
     __shared__ __align__(16) uint16_t dist[kEdtSide * kEdtSide];
@@ -446,7 +447,7 @@ __global__ void __launch_bounds__(kFarThreads) edt_far_kernel(const __grid_const
 cudaError_t launch_edt_bits_batch(const EdtBitsBatch &b, int num_sms, uint64_t timeout_ns, cudaStream_t s)
 {
     if (b.n < 1 || b.n > kEdtMaxImgs) return cudaErrorInvalidValue;
-    edt_near_kernel<<<(unsigned)b.ntiles, kNearThreads, 0, s>>>(b);
+    launch_early(edt_near_kernel, (unsigned)b.ntiles, kNearThreads, 0, s, b);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const size_t smem = 2 * (size_t)b.maxW * sizeof(uint16_t);

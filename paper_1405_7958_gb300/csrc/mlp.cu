@@ -161,6 +161,7 @@ __global__ void mlp_grad_kernel(const float *ws, const float *act, int B, float 
 __global__ void mlp_adamw_kernel(float *master, uint16_t *wb, const float *grad, float *m, float *v, int step,
                                  float lr, float b1, float b2, float eps, float wd)
 {
+    start_early();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= kMlpParams) return;
     const float g = grad[t];
@@ -246,8 +247,7 @@ cudaError_t launch_mlp_backward(const uint16_t *wb, const float *norm, const flo
 cudaError_t launch_mlp_adamw(float *master, uint16_t *wb, const float *grad, float *m, float *v, int step, float lr,
                              float b1, float b2, float eps, float wd, cudaStream_t s)
 {
-    mlp_adamw_kernel<<<(unsigned)ceil_div(kMlpParams, 256), 256, 0, s>>>(master, wb, grad, m, v, step, lr, b1, b2,
-                                                                         eps, wd);
+    launch_early(mlp_adamw_kernel, (unsigned)ceil_div(kMlpParams, 256), 256, 0, s, master, wb, grad, m, v, step, lr, b1, b2, eps, wd);
     return cudaGetLastError();
 }
 

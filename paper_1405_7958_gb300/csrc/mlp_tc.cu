@@ -197,6 +197,7 @@ __global__ void __launch_bounds__(kTcThreads) mlp_forward_tc_kernel(const uint16
                                                               int B, float *logits, float *act, int32_t *pick,
                                                               float min_prob, int fallback, int32_t *err)
 {
+    start_early();
     __shared__ __align__(1024) uint8_t sm[kTcSmem];
     __shared__ __align__(8) uint64_t mbar_store;
     __shared__ uint32_t tmem_base;
@@ -369,6 +370,7 @@ __global__ void __launch_bounds__(kTcThreads) mlp_backward_tc_kernel(const uint1
                                                                      float *part, float *dz_out, float *loss_out,
                                                                      int32_t *err)
 {
+    start_early();
     extern __shared__ __align__(1024) uint8_t smb[];
     __shared__ __align__(8) uint64_t mbar_store;
     __shared__ uint32_t tmem_base;
@@ -536,6 +538,7 @@ __global__ void __launch_bounds__(kTcThreads) mlp_backward_tc_kernel(const uint1
 __global__ void mlp_grad_tc_kernel(const float *part, int nblk, const float *dz, const float *act, const float *lossb,
                                    int B, float *grad, float *loss)
 {
+    start_early();
     const int p = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (p > kMlpParams) return;
     float s = 0.f;
@@ -583,10 +586,9 @@ cudaError_t launch_mlp_backward_tc(const uint16_t *wb, const float *norm, const 
                                                                         : mlp_backward_tc_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwSmem);
     if (e != cudaSuccess) return e;
-    kernel<<<nblk, kTcThreads, kBwSmem, s>>>(wb, norm, x, act, logits, label, B, part, dz, lossb, err);
+    launch_early(kernel, nblk, kTcThreads, kBwSmem, s, wb, norm, x, act, logits, label, B, part, dz, lossb, err);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    mlp_grad_tc_kernel<<<(unsigned)ceil_div((int64_t)(kMlpParams + 1) * 32, 256), 256, 0, s>>>(part, nblk, dz, act,
-                                                                                               lossb, B, grad, loss);
+    launch_early(mlp_grad_tc_kernel, (unsigned)ceil_div((int64_t)(kMlpParams + 1) * 32, 256), 256, 0, s, part, nblk, dz, act, lossb, B, grad, loss);
     return cudaGetLastError();
 }
 
@@ -597,8 +599,7 @@ cudaError_t launch_mlp_forward_tc(const uint16_t *wb, const float *norm, const f
     if (B <= 0) return cudaSuccess;
     const auto kernel = aligned16(wb) && aligned16(x) && aligned16(act) ? mlp_forward_tc_kernel<true>
                                                                         : mlp_forward_tc_kernel<false>;
-    kernel<<<(unsigned)ceil_div(B, kTcM), kTcThreads, 0, s>>>(wb, norm, x, B, logits, act, pick, min_prob, fallback,
-                                                              err);
+    launch_early(kernel, (unsigned)ceil_div(B, kTcM), kTcThreads, 0, s, wb, norm, x, B, logits, act, pick, min_prob, fallback, err);
     return cudaGetLastError();
 }
 

@@ -85,6 +85,7 @@ void obj_carve(ObjArgs &a, char *base, bool features, bool watershed)
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads) obj_scan_kernel(ObjArgs a)
 {
+    start_early();
     constexpr int kSteps = kObjChunk / 128;
     __shared__ uint32_t roots_of[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -220,6 +221,7 @@ __global__ void __launch_bounds__(kThreads) obj_scan_kernel(ObjArgs a)
 // RT_EINVAL in the status.
 __global__ void __launch_bounds__(kThreads) obj_grow_kernel(ObjArgs a, int nblk, int span)
 {
+    start_early();
     __shared__ uint32_t part[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t N = (int64_t)a.H * a.W, nch = ceil_div(N, kObjChunk);
@@ -278,13 +280,13 @@ cudaError_t launch_enumeration(const ObjArgs &a, int num_sms, cudaStream_t s, in
     const int nblk = (int)ceil_div(nch, kWarps);
     auto quads = [](const void *p, int64_t ld) { return ((uintptr_t)p & 15u) == 0 && ld % 4 == 0; };
     if (a.W % 4 == 0 && quads(a.L, a.ld_L) && (!a.basins || quads(a.basins, a.ld_B)))
-        obj_scan_kernel<true><<<nblk, kThreads, 0, s>>>(a);
+        launch_early(obj_scan_kernel<true>, nblk, kThreads, 0, s, a);
     else
-        obj_scan_kernel<false><<<nblk, kThreads, 0, s>>>(a);
+        launch_early(obj_scan_kernel<false>, nblk, kThreads, 0, s, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int span = (int)ceil_div(nblk, num_sms * 8);
-    obj_grow_kernel<<<(unsigned)ceil_div(nblk, span), kThreads, 0, s>>>(a, nblk, span);
+    launch_early(obj_grow_kernel, (unsigned)ceil_div(nblk, span), kThreads, 0, s, a, nblk, span);
     *launches += 2;
     return cudaGetLastError();
 }
@@ -512,6 +514,7 @@ __device__ __forceinline__ bool warp_box(int bh, int bw)
 // 10).
 __global__ void __launch_bounds__(kThreads) obj_inter_kernel(ObjArgs a)
 {
+    start_early();
     __shared__ __align__(16) uint32_t hist_of[kWarps][256];
     __shared__ __align__(16) uint32_t glcm_of[kWarps][64];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -608,6 +611,7 @@ __global__ void __launch_bounds__(kThreads) obj_inter_kernel(ObjArgs a)
 // intermediate results to the features; then four lanes per other object.
 __global__ void __launch_bounds__(kThreads) obj_feature_kernel(ObjArgs a)
 {
+    start_early();
     __shared__ uint32_t hist[256], glcm[64];
     __shared__ unsigned long long sums[9];
     __shared__ int slot;
@@ -692,9 +696,9 @@ cudaError_t launch_object_features(const ObjArgs &a, int num_sms, cudaStream_t s
     cudaError_t e = launch_enumeration(a, num_sms, s, launches);
     if (e != cudaSuccess) return e;
     if (a.cap < 1) return cudaSuccess;
-    obj_inter_kernel<<<(unsigned)persistent_grid((const void *)obj_inter_kernel, 0, num_sms), kThreads, 0, s>>>(a);
+    launch_early(obj_inter_kernel, (unsigned)persistent_grid((const void *)obj_inter_kernel, 0, num_sms), kThreads, 0, s, a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    obj_feature_kernel<<<(unsigned)(2 * num_sms), kThreads, 0, s>>>(a);
+    launch_early(obj_feature_kernel, (unsigned)(2 * num_sms), kThreads, 0, s, a);
     *launches += 2;
     return cudaGetLastError();
 }
@@ -1381,6 +1385,7 @@ __device__ __forceinline__ bool watershed_small(const ObjArgs &a, int4 b, int32_
 // size first.
 __global__ void __launch_bounds__(kThreads, 4) obj_watershed_small_kernel(ObjArgs a)
 {
+    start_early();
     extern __shared__ __align__(16) uint16_t slots[];
     __shared__ int sh[5];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1437,6 +1442,7 @@ constexpr int kWsBlockCells = (int)(kWsSmemBytes / kWsCellBytes) & ~1;
 
 __global__ void __launch_bounds__(kWsThreads) obj_watershed_kernel(ObjArgs a)
 {
+    start_early();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int slot, red, sh[4];
     const SmemView sv = smem_view(smem, kWsSmemPx);
@@ -1481,13 +1487,9 @@ cudaError_t launch_watershed(const ObjArgs &a, int num_sms, cudaStream_t s, int 
     const cudaFuncAttribute dyn = cudaFuncAttributeMaxDynamicSharedMemorySize;
     if ((e = cudaFuncSetAttribute(obj_watershed_small_kernel, dyn, (int)kWsWarpSmem)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(obj_watershed_kernel, dyn, (int)kWsSmemBytes)) != cudaSuccess) return e;
-    obj_watershed_small_kernel<<<(unsigned)persistent_grid((const void *)obj_watershed_small_kernel, kWsWarpSmem,
-                                                          num_sms),
-                                kThreads, kWsWarpSmem, s>>>(a);
+    launch_early(obj_watershed_small_kernel, (unsigned)persistent_grid((const void *)obj_watershed_small_kernel, kWsWarpSmem, num_sms), kThreads, kWsWarpSmem, s, a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    obj_watershed_kernel<<<(unsigned)persistent_grid((const void *)obj_watershed_kernel, kWsSmemBytes, num_sms,
-                                                     kWsThreads),
-                           kWsThreads, kWsSmemBytes, s>>>(a);
+    launch_early(obj_watershed_kernel, (unsigned)persistent_grid((const void *)obj_watershed_kernel, kWsSmemBytes, num_sms, kWsThreads), kWsThreads, kWsSmemBytes, s, a);
     *launches += 2;
     return cudaGetLastError();
 }

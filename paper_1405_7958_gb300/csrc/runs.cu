@@ -495,24 +495,19 @@ __device__ __forceinline__ ulonglong2 holes_of(const RunBatch &b, uint32_t *U, c
 // CTA per tile: thread = 16 columns of a row.
 __global__ void __launch_bounds__(256) run_pack_kernel(const __grid_constant__ RunBatch b)
 {
+    start_early();
     const int tile = blockIdx.x, t = threadIdx.x;
     const RunImage &d = run_image(b, tile);
     const int lt = tile - d.tile_base;
     const int ty = lt / d.nx, tx = lt - ty * d.nx;
     const int r = ty * kRunSide + (t >> 2), c = tx * kRunSide + (t & 3) * 16;
     const int n = r < d.H ? min(16, d.W - c) : 0;   // may be negative: none
-    uint32_t m = 0;
-    const uint8_t *p = d.in + (int64_t)r * d.ld_in + c;
-    if (n == 16 && ((uintptr_t)p & 15u) == 0) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t w[4], m = 0;
+    load_row16(d.in + (int64_t)r * d.ld_in, c, n, d.W, w);
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) m |= (uint32_t)(((w[q] >> (8 * k)) & 0xffu) != 0u) << (4 * q + k);
-    } else {
-        for (int k = 0; k < n; ++k) m |= (uint32_t)(p[k] != 0) << k;
-    }
+        for (int k = 0; k < 4; ++k) m |= (uint32_t)(((w[q] >> (8 * k)) & 0xffu) != 0u) << (4 * q + k);
     reinterpret_cast<uint16_t *>(b.bits + (int64_t)tile * kRunSide)[t] = (uint16_t)m;
 }
 
@@ -527,25 +522,15 @@ __device__ __forceinline__ uint32_t at_least(uint32_t v, uint32_t t)
 // >= lo), J the chain's marker: I >= hi, or I >= lo on the image border.
 __global__ void __launch_bounds__(256) run_threshold_kernel(const __grid_constant__ RunBatch b)
 {
+    start_early();
     const int tile = blockIdx.x, t = threadIdx.x;
     const RunImage &d = run_image(b, tile);
     const int lt = tile - d.tile_base;
     const int ty = lt / d.nx, tx = lt - ty * d.nx;
     const int r = ty * kRunSide + (t >> 2), c = tx * kRunSide + (t & 3) * 16;
     const int n = r < d.H ? min(16, d.W - c) : 0;   // may be negative: none
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-    const uint8_t *p = d.in + (int64_t)r * d.ld_in + c;
-    if (n == 16 && ((uintptr_t)p & 15u) == 0) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
-        w[0] = v.x;
-        w[1] = v.y;
-        w[2] = v.z;
-        w[3] = v.w;
-    } else {
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-            if (k < n) w[k >> 2] |= (uint32_t)__ldg(p + k) << (8 * (k & 3));
-    }
+    uint32_t w[4];
+    load_row16(d.in + (int64_t)r * d.ld_in, c, n, d.W, w);
     uint32_t m = 0, sd = 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {   // four flags of a word to a nibble: no two products of the multiplication meet
@@ -569,6 +554,7 @@ __global__ void __launch_bounds__(256) run_threshold_kernel(const __grid_constan
 template <int CONN, bool SEEDS, bool AGAIN, bool ALONE>
 __global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_fill_local_kernel(const __grid_constant__ RunBatch b)
 {
+    start_early();
     const int lane = threadIdx.x & 31, at = blockIdx.x * (ALONE ? 1 : kWarps) + (threadIdx.x >> 5);
     const bool mine = at < b.ntiles;
     const int tile = mine ? at : 0;
@@ -597,6 +583,7 @@ __global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_fill_local_kerne
 template <int CONN>
 __global__ void __launch_bounds__(kWarps * 32) run_seam_kernel(const __grid_constant__ RunBatch b, uint32_t *U)
 {
+    start_early();
     __shared__ uint32_t s_pairs[kWarps][2 * kRunSide * 3];
     const int lane = threadIdx.x & 31;
     const int tile = blockIdx.x * kWarps + (threadIdx.x >> 5);
@@ -659,6 +646,7 @@ __global__ void __launch_bounds__(kWarps * 32) run_seam_kernel(const __grid_cons
 template <bool FILL, int LABEL, bool ALONE>
 __global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_local_kernel(const __grid_constant__ RunBatch b)
 {
+    start_early();
     const int lane = threadIdx.x & 31, at = blockIdx.x * (ALONE ? 1 : kWarps) + (threadIdx.x >> 5);
     const bool mine = at < b.ntiles;
     const int tile = mine ? at : 0;
@@ -687,18 +675,26 @@ __global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_local_kernel(con
 #pragma unroll 2
                 for (int q = 0; q < 8; ++q) {
                     const int i = 8 * q + (lane >> 2), r = p.r0 + i, c = p.c0 + (lane & 3) * 16;
-                    const u64 w0 = shfl64(f.x, i >> 1), w1 = shfl64(f.y, i >> 1);
-                    const uint32_t m = (uint32_t)((i & 1 ? w1 : w0) >> ((lane & 3) * 16)) & 0xffffu;
+                    const u64 w0 = shfl64(f.x, i >> 1), w1 = shfl64(f.y, i >> 1), bits = i & 1 ? w1 : w0;
+                    const uint32_t m = (uint32_t)(bits >> ((lane & 3) * 16)) & 0xffffu;
                     const int n = r < d.H ? min(16, d.W - c) : 0;
                     if (n <= 0) continue;
-                    uint8_t *o = d.filled + (int64_t)r * d.ld_filled + c;
-                    if (n == 16 && ((uintptr_t)o & 15u) == 0) {
+                    auto spread = [](uint32_t x) { return ((x & 0xfu) * 0x00204081u) & 0x01010101u; };
+                    uint8_t *o = d.filled + (int64_t)r * d.ld_filled + p.c0;
+                    const int head = (int)(-(uintptr_t)o & 3u);
+                    if (head && d.W - p.c0 >= kRunSide) {   // the row's aligned words, from its bits; its ends by bytes
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int at = head + 16 * (lane & 3) + 4 * k;
+                            if (at + 4 <= kRunSide) *reinterpret_cast<uint32_t *>(o + at) = spread((uint32_t)(bits >> at));
+                        }
+                        if ((lane & 3) < head) o[lane & 3] = (uint8_t)((bits >> (lane & 3)) & 1ull);
+                        else o[kRunSide - 4 + (lane & 3)] = (uint8_t)((bits >> (kRunSide - 4 + (lane & 3))) & 1ull);
+                    } else {
                         uint32_t w[4];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) w[k] = (((m >> (4 * k)) & 0xfu) * 0x00204081u) & 0x01010101u;
-                        *reinterpret_cast<uint4 *>(o) = make_uint4(w[0], w[1], w[2], w[3]);
-                    } else {
-                        for (int k = 0; k < n; ++k) o[k] = (uint8_t)((m >> k) & 1u);
+                        for (int k = 0; k < 4; ++k) w[k] = spread(m >> (4 * k));
+                        store_bytes(o + (lane & 3) * 16, n, w);
                     }
                 }
             }
@@ -751,6 +747,7 @@ __global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_local_kernel(con
 // Thread per slot: areas and first pixels of a tree meet at its root.
 __global__ void __launch_bounds__(256) run_roots_kernel(const __grid_constant__ RunBatch b)
 {
+    start_early();
     const int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int tile = (int)(g / 32), lane = (int)(g % 32);   // a warp per tile
     if (tile >= b.ntiles) return;
@@ -771,6 +768,7 @@ __global__ void __launch_bounds__(256) run_roots_kernel(const __grid_constant__ 
 template <bool ALONE>
 __global__ void __launch_bounds__(ALONE ? 32 : kWarps * 32) run_label_kernel(const __grid_constant__ RunBatch b)
 {
+    start_early();
     const int lane = threadIdx.x & 31, at = blockIdx.x * (ALONE ? 1 : kWarps) + (threadIdx.x >> 5);
     const int tile = at;
     if (tile >= b.ntiles) return;
@@ -882,15 +880,15 @@ cudaError_t warp_per_tile(RunKernel alone, RunKernel four, const RunBatch &b, cu
 {
     const bool few = b.ntiles <= kFewTiles;
     const int w = few ? 1 : kWarps;
-    (few ? alone : four)<<<dim3((unsigned)ceil_div(b.ntiles, w), y), w * 32, kRunSmem, s>>>(b);
+    launch_early((few ? alone : four), dim3((unsigned)ceil_div(b.ntiles, w), y), w * 32, kRunSmem, s, b);
     return cudaGetLastError();
 }
 
 cudaError_t launch_seam(const RunBatch &b, int conn, uint32_t *U, cudaStream_t s)
 {
     const unsigned grid = (unsigned)ceil_div(b.ntiles, kWarps);
-    if (conn == 8) run_seam_kernel<8><<<grid, kWarps * 32, 0, s>>>(b, U);
-    else run_seam_kernel<4><<<grid, kWarps * 32, 0, s>>>(b, U);
+    if (conn == 8) launch_early(run_seam_kernel<8>, grid, kWarps * 32, 0, s, b, U);
+    else launch_early(run_seam_kernel<4>, grid, kWarps * 32, 0, s, b, U);
     return cudaGetLastError();
 }
 
@@ -913,13 +911,13 @@ RunImage &run_add(RunBatch &b, int H, int W)
 
 cudaError_t launch_run_pack(const RunBatch &b, cudaStream_t s)
 {
-    run_pack_kernel<<<(unsigned)b.ntiles, 256, 0, s>>>(b);
+    launch_early(run_pack_kernel, (unsigned)b.ntiles, 256, 0, s, b);
     return cudaGetLastError();
 }
 
 cudaError_t launch_run_reach(const RunBatch &b, cudaStream_t s)
 {
-    run_threshold_kernel<<<(unsigned)b.ntiles, 256, 0, s>>>(b);
+    launch_early(run_threshold_kernel, (unsigned)b.ntiles, 256, 0, s, b);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = warp_per_tile(run_fill_local_kernel<8, true, false, true>, run_fill_local_kernel<8, true, false, false>, b, s);
@@ -954,7 +952,7 @@ cudaError_t launch_run_label(const RunBatch &b, int conn, cudaStream_t s)
     if (conn != 4 && conn != 8) return cudaErrorInvalidValue;
     cudaError_t e = launch_seam(b, conn, b.U, s);
     if (e != cudaSuccess) return e;
-    run_roots_kernel<<<(unsigned)ceil_div(b.ntiles, 8), 256, 0, s>>>(b);
+    launch_early(run_roots_kernel, (unsigned)ceil_div(b.ntiles, 8), 256, 0, s, b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // few tiles: four warps write a tile's labels (a warp's 64 rows are 10 us of latency)
     return warp_per_tile(run_label_kernel<true>, run_label_kernel<false>, b, s, b.ntiles <= kFewTiles ? 4 : 1);
