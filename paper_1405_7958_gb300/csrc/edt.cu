@@ -178,7 +178,11 @@ size_t piece(size_t bytes) { return (size_t)round_up((int64_t)bytes, 256); }
 
 typedef unsigned long long u64;
 
-constexpr int kNearThreads = 128;
+// Threads per tile of the near stage: 256 up to kFewTiles tiles, where a
+// tile's latency counts (900 x 900, dense nuclei: a call takes 20 us, with 128
+// threads 23; equal at 4096 x 4096), 128 above (eight of these: 116 us, with
+// 256 129).
+constexpr int kFewTiles = 4096;
 constexpr int kReach = 32;                       // rows and columns a tile looks beyond itself
 constexpr uint32_t kNearMax = kReach * kReach;   // distances below are exact
 constexpr int kFarThreads = 256;
@@ -213,7 +217,8 @@ void edt_bits_add(EdtBitsBatch &b, int H, int W, int32_t *d2, int64_t ld_d2, cha
 }
 
 // ------------------------------------------------------------------- near
-__global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const __grid_constant__ EdtBitsBatch b)
+template <int NT>
+__global__ void __launch_bounds__(NT) edt_near_kernel(const __grid_constant__ EdtBitsBatch b)
 {
     start_early();
     __shared__ uint32_t bg[kRowsIn][kRowWords + 1];   // background bits of rows and columns -32 .. 95
@@ -231,13 +236,13 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const __grid_con
     const int nr = min(kEdtSide, d.H - r0), nc = min(kEdtSide, d.W - c0);
     const bool wide = nc == kEdtSide && (((uintptr_t)d.d2 | (uintptr_t)d.ld_d2 * 4u) & 15u) == 0;
     // own bits: thread = half a row
-    uint32_t own = __ldg(reinterpret_cast<const uint32_t *>(b.bits + (int64_t)tile * kEdtSide) + t);
+    uint32_t own = t < 2 * kEdtSide ? __ldg(reinterpret_cast<const uint32_t *>(b.bits + (int64_t)tile * kEdtSide) + t) : 0u;
     if (!__syncthreads_or(own != 0u)) {
         if (wide) {
-            for (int i = t >> 4; i < nr; i += kNearThreads / 16)
+            for (int i = t >> 4; i < nr; i += NT / 16)
                 reinterpret_cast<int4 *>(d.d2 + (int64_t)(r0 + i) * d.ld_d2 + c0)[t & 15] = make_int4(0, 0, 0, 0);
         } else {
-            for (int i = t >> 6; i < nr; i += kNearThreads / 64)
+            for (int i = t >> 6; i < nr; i += NT / 64)
                 if ((t & 63) < nc) d.d2[(int64_t)(r0 + i) * d.ld_d2 + c0 + (t & 63)] = 0;
         }
         return;
@@ -245,7 +250,7 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const __grid_con
     if (t == 0) s_n = 0, s_far[0] = s_far[1] = 0u;
     uint32_t any = 0;
     // background of the neighbourhood: word w of a row = columns c0 - 32 + 32 w; only pixels inside the image count
-    for (int i = t; i < kRowsIn * kRowWords; i += kNearThreads) {
+    for (int i = t; i < kRowsIn * kRowWords; i += NT) {
         const int y = i / kRowWords, w = i - y * kRowWords;
         const int r = r0 - kReach + y, c = c0 - kReach + 32 * w;
         uint32_t v = 0;
@@ -257,7 +262,7 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const __grid_con
         bg[y][w] = v;
         any |= v;
     }
-    for (int i = t; i < kEdtSide * kEdtSide / 8; i += kNearThreads)
+    for (int i = t; i < kEdtSide * kEdtSide / 8; i += NT)
         reinterpret_cast<uint4 *>(dist)[i] = make_uint4(0u, 0u, 0u, 0u);
     const int some = __syncthreads_count(any != 0u);   // threads whose words hold background
     {
@@ -283,8 +288,8 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const __grid_con
     // left to the far stage, whose step costs half as much where distances are
     // long (2048 x 2048, one pixel in a thousand background: 178 us in this
     // stage against 24). Nuclei never fill three quarters of a tile.
-    const uint32_t reach = n > 3 * kEdtSide * kEdtSide / 4 && some < kNearThreads / 4 ? 0u : kNearMax;
-    for (int i = t; i < n; i += kNearThreads) {
+    const uint32_t reach = n > 3 * kEdtSide * kEdtSide / 4 && some < NT / 4 ? 0u : kNearMax;
+    for (int i = t; i < n; i += NT) {
         const int p = list[i], r = p / kEdtSide, c = p % kEdtSide;
         // window: columns c - 32 .. c + 31 of the row = bits c .. c + 63
         const int w = c >> 5, sh = c & 31;
@@ -307,13 +312,13 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const __grid_con
         *b.far_any = 1u;
     }
     if (wide) {
-        for (int i = t >> 4; i < nr; i += kNearThreads / 16) {
+        for (int i = t >> 4; i < nr; i += NT / 16) {
             const uint2 v = *reinterpret_cast<const uint2 *>(dist + i * kEdtSide + 4 * (t & 15));
             reinterpret_cast<int4 *>(d.d2 + (int64_t)(r0 + i) * d.ld_d2 + c0)[t & 15] =
                 make_int4((int)(v.x & 0xffffu), (int)(v.x >> 16), (int)(v.y & 0xffffu), (int)(v.y >> 16));
         }
     } else {
-        for (int i = t >> 6; i < nr; i += kNearThreads / 64)
+        for (int i = t >> 6; i < nr; i += NT / 64)
             if ((t & 63) < nc) d.d2[(int64_t)(r0 + i) * d.ld_d2 + c0 + (t & 63)] = dist[i * kEdtSide + (t & 63)];
     }
 }
@@ -447,7 +452,8 @@ __global__ void __launch_bounds__(kFarThreads) edt_far_kernel(const __grid_const
 cudaError_t launch_edt_bits_batch(const EdtBitsBatch &b, int num_sms, uint64_t timeout_ns, cudaStream_t s)
 {
     if (b.n < 1 || b.n > kEdtMaxImgs) return cudaErrorInvalidValue;
-    launch_early(edt_near_kernel, (unsigned)b.ntiles, kNearThreads, 0, s, b);
+    if (b.ntiles <= kFewTiles) launch_early(edt_near_kernel<256>, (unsigned)b.ntiles, 256, 0, s, b);
+    else launch_early(edt_near_kernel<128>, (unsigned)b.ntiles, 128, 0, s, b);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const size_t smem = 2 * (size_t)b.maxW * sizeof(uint16_t);
