@@ -903,6 +903,213 @@ __global__ void __launch_bounds__(kCtUnits * 32) ct_seam_kernel(const __grid_con
     }
 }
 
+// ------------------------------------------------------- few nodes: one CTA
+// The nodes and edges of up to kSmallTiles tiles, if they fit, are contracted
+// by one CTA in shared memory: the rounds of the global kernel below are L2
+// round trips and barriers, 5 to 6 us each however little they do (512 x 512,
+// 2600 nodes and 7300 edges: XXG).
+namespace {
+constexpr int kSmallTiles = 128, kSmallNodes = 4096, kSmallEdges = 16384;
+constexpr size_t kSmallSmem = sizeof(uint32_t) * (kSmallEdges + 2 * kSmallNodes) + 2 * sizeof(uint16_t) * kSmallNodes;
+// An edge is weight << 24 | node << 12 | node, a link word as in the local stage: kRootBit | kSmallDone | S, else
+// weight << 16 | parent. A best edge is weight << 14 | mixed position, + 1: ties in no geometric order.
+constexpr uint32_t kSmallDone = 0x40000000u, kMixPos = 0x19e5u, kUnmixPos = 0x3bedu;
+constexpr uint32_t kPosMask = kSmallEdges - 1;
+static_assert(((kMixPos * kUnmixPos) & kPosMask) == 1u, "inverse");
+
+struct SmallSums {
+    int node[kSmallTiles + 1], edge[kSmallTiles * kCtUnits + 1];   // exclusive prefix sums over tiles, over units
+};
+
+// Sums the batch's nodes and edges; whole CTA. True if they fit.
+__device__ __forceinline__ bool small_sums(const CtBatch &b, SmallSums &p)
+{
+    const int t = threadIdx.x;
+    if (b.ntiles > kSmallTiles) return false;   // all threads
+    if (t < 32) {
+        int nodes = 0, edges = 0;
+#pragma unroll
+        for (int k = 0; k < kSmallTiles; k += 32) {
+            const int i = k + t;
+            const int n = i < b.ntiles ? (int)(__ldcg(b.cnt + i) & 0xffffu) : 0;
+            const uint32_t e4 = i < b.ntiles ? __ldcg(reinterpret_cast<const uint32_t *>(b.ecnt) + i) : 0u;
+            int e[kCtUnits], sum = 0;
+#pragma unroll
+            for (int q = 0; q < kCtUnits; ++q) sum += e[q] = (int)((e4 >> (8 * q)) & 0xffu);
+            int ni = n, ei = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, ni, o), y = __shfl_up_sync(0xffffffffu, ei, o);
+                if (t >= o) ni += x, ei += y;
+            }
+            p.node[i] = nodes + ni - n;
+            int at = edges + ei - sum;
+#pragma unroll
+            for (int q = 0; q < kCtUnits; ++q) {
+                p.edge[i * kCtUnits + q] = at;
+                at += e[q];
+            }
+            nodes += __shfl_sync(0xffffffffu, ni, 31);
+            edges += __shfl_sync(0xffffffffu, ei, 31);
+        }
+        if (t == 0) p.node[kSmallTiles] = nodes, p.edge[kSmallTiles * kCtUnits] = edges;
+    }
+    __syncthreads();
+    return p.node[kSmallTiles] <= kSmallNodes && p.edge[kSmallTiles * kCtUnits] <= kSmallEdges;
+}
+
+__device__ __forceinline__ void small_contract(const CtBatch &b, const SmallSums &p)
+{
+    extern __shared__ __align__(16) uint32_t small_smem[];
+    uint32_t *E = small_smem;
+    volatile uint32_t *link = E + kSmallEdges, *best = link + kSmallNodes;
+    volatile uint16_t *act = reinterpret_cast<volatile uint16_t *>(best + kSmallNodes);   // two lists
+    __shared__ int s_open[2];
+    constexpr int kWarps = kGT / 32, kPer = kSmallNodes / kGT;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint32_t below = (1u << lane) - 1u;
+    const int nn = p.node[kSmallTiles], nedge = p.edge[kSmallTiles * kCtUnits];
+    if (t < 2) s_open[t] = 0;
+    auto key_of = [](uint32_t w, uint32_t pos) { return (w << 14 | ((pos * kMixPos) & kPosMask)) + 1u; };
+    // a warp takes whole tiles: their nodes, with round 0's best edges, and their units' edges
+#pragma unroll 1
+    for (int tile = warp; tile < b.ntiles; tile += kWarps) {
+        const int n0 = p.node[tile], n = p.node[tile + 1] - n0;
+        for (int i = lane; i < n; i += 32) {
+            const unsigned long long l = __ldcg(b.link + tile * kCtNodes + i), k = __ldcg(b.best + tile * kCtNodes + i);
+            const uint32_t g = (uint32_t)k * kUnmix;   // the edge's slot
+            link[n0 + i] = kRootBit | node_S(l);
+            best[n0 + i] = k ? key_of(((uint32_t)(k >> 32) & 0xffffu) - 1u,
+                                      (uint32_t)p.edge[g / kCtUnitEdges] + g % kCtUnitEdges) : 0u;
+            act[n0 + i] = (uint16_t)(n0 + i);
+        }
+#pragma unroll
+        for (int q = 0; q < kCtUnits; ++q) {
+            const int u = tile * kCtUnits + q, e0 = p.edge[u], ne = p.edge[u + 1] - e0;
+#pragma unroll 2
+            for (int i = lane; i < ne; i += 32) {
+                const unsigned long long e = __ldcg(b.edge + (int64_t)u * kCtUnitEdges + i);
+                const uint32_t a = (uint32_t)(e >> 28) & kNodeId, c = (uint32_t)e & kNodeId;
+                E[e0 + i] = (uint32_t)(e >> 56) << 24 | ((uint32_t)p.node[a >> 8] + (a & 0xffu)) << 12 |
+                            ((uint32_t)p.node[c >> 8] + (c & 0xffu));
+            }
+        }
+    }
+    __syncthreads();
+    // each warp keeps a range of the edges and compacts it in place
+    const int per = (((nedge + kWarps - 1) / kWarps) + 31) & ~31;
+    const int start = min(warp * per, nedge);
+    int cnt = min(per, nedge - start), nl = nn;
+#pragma unroll 1
+    for (int round = 0;; ++round) {
+        int kept = round ? 0 : cnt;
+#pragma unroll 1
+        for (int i = lane; round && i < cnt + lane; i += 32) {
+            bool keep = false, oa = false, oc = false;
+            uint32_t a = 0, c = 0, w = 0;
+            if (i < cnt) {
+                const uint32_t e = E[start + i];
+                w = e >> 24;
+                a = (e >> 12) & 0xfffu;
+                c = e & 0xfffu;
+                uint32_t la = link[a], lc = link[c];
+                if (!(la & kRootBit)) la = link[a = la & 0xffffu];   // links of the last round are compressed
+                if (!(lc & kRootBit)) lc = link[c = lc & 0xffffu];
+                oa = !(la & kSmallDone);
+                oc = !(lc & kSmallDone);
+                keep = a != c && (oa || oc);
+            }
+            const uint32_t m = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                const uint32_t pos = (uint32_t)(start + kept + __popc(m & below));
+                E[pos] = w << 24 | a << 12 | c;
+                const uint32_t key = key_of(w, pos);
+                if (oa && best[a] < key) atomicMax(const_cast<uint32_t *>(best + a), key);
+                if (oc && best[c] < key) atomicMax(const_cast<uint32_t *>(best + c), key);
+            }
+            kept += __popc(m);
+            __syncwarp();
+        }
+        cnt = kept;
+        __syncthreads();
+        // decisions: w << 16 | parent, or none
+        const volatile uint16_t *from = act + (round & 1) * kSmallNodes;
+        volatile uint16_t *to = act + (~round & 1) * kSmallNodes;
+        constexpr uint32_t kNo = ~0u, kStay = ~0u - 1u;
+        uint32_t dec[kPer], id[kPer];
+        uint32_t S[kPer];
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            dec[q] = kNo;
+            id[q] = S[q] = 0u;
+            if (t + q * kGT >= nl) continue;
+            const uint32_t k = from[t + q * kGT], key = best[k], w = (key - 1u) >> 14;
+            id[q] = k;
+            S[q] = link[k] & 0xffu;
+            if (!key || S[q] >= w) {
+                dec[q] = kNo;   // final
+                continue;
+            }
+            const uint32_t e = E[((key - 1u) * kUnmixPos) & kPosMask], a = (e >> 12) & 0xfffu, c = e & 0xfffu,
+                           o = a == k ? c : a;
+            // o joins k by the same edge: the smaller of the two stays
+            const bool mutual = k < o && best[o] == key && (link[o] & 0xffu) < w;
+            dec[q] = mutual ? kStay : w << 16 | o;
+        }
+        if (t == 0) s_open[~round & 1] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            if (t + q * kGT >= nl) continue;
+            if (dec[q] == kNo) link[id[q]] = link[id[q]] | kSmallDone;
+            else if (dec[q] != kStay) link[id[q]] = dec[q];
+            else best[id[q]] = 0u;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            if (warp * 32 + q * kGT >= nl) continue;   // whole warp
+            const bool in = t + q * kGT < nl;
+            if (in && dec[q] < kStay) {
+                uint32_t w = dec[q] >> 16, x = dec[q] & 0xffffu, v = link[x];
+#pragma unroll 1
+                for (int n = 0; n < kSmallNodes && !(v & kRootBit); ++n) {
+                    w = min(w, v >> 16);
+                    x = v & 0xffffu;
+                    v = link[x];
+                }
+                link[id[q]] = w << 16 | x;
+                if ((v & 0xffu) < S[q]) atomicMax(const_cast<uint32_t *>(link + x), kRootBit | S[q]);
+            }
+            const bool stays = in && dec[q] == kStay;
+            const uint32_t m = __ballot_sync(0xffffffffu, stays);
+            int base = 0;
+            if (lane == 0 && m) base = atomicAdd(&s_open[~round & 1], __popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (stays) to[base + __popc(m & below)] = (uint16_t)id[q];
+        }
+        __syncthreads();
+        nl = s_open[~round & 1];
+        if (nl == 0) break;
+    }
+    // every node's value, as a root
+#pragma unroll 1
+    for (int tile = warp; tile < b.ntiles; tile += kWarps) {
+        const int n0 = p.node[tile], n = p.node[tile + 1] - n0;
+        for (int i = lane; i < n; i += 32) {
+            uint32_t v = 255u, l = link[n0 + i];
+#pragma unroll 1
+            for (int k = 0; k < kSmallNodes && !(l & kRootBit); ++k) {
+                v = min(v, l >> 16);
+                l = link[l & 0xffffu];
+            }
+            const uint32_t g = (uint32_t)(tile * kCtNodes + i);
+            b.link[g] = kNodeRoot | (unsigned long long)min(v, l & 0xffu) << 40 | g;
+        }
+    }
+}
+}  // namespace
+
 // Contraction of the nodes of the batch. The work is cut into units, four a
 // tile; every warp owns the units [u0, u1) and keeps their nodes and, from
 // round 1 on, edges compacted at the start of their slots, so no list is
@@ -933,6 +1140,13 @@ __global__ void __launch_bounds__(kGT, 1) ct_global_kernel(const __grid_constant
     __shared__ uint32_t s_open[3];
     if (threadIdx.x < 3) s_open[threadIdx.x] = 0u;
     __syncthreads();
+    if (CLUSTER) {
+        __shared__ SmallSums sums;
+        if (small_sums(b, sums)) {   // the same answer in every CTA
+            if (blockIdx.x == 0) small_contract(b, sums);
+            return;
+        }
+    }
     if (CLUSTER)   // no CTA adds to another's before it is zero
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 
@@ -1264,9 +1478,12 @@ cudaError_t launch_contract(const CtBatch &b, int num_sms, uint64_t timeout_ns, 
     // most (512 x 512: 90 us against 110 for both stages; 768 x 768: equal).
     if (units <= kGClusterUnits) {
         auto *gfn = ct_global_kernel<true>;
+        e = cudaFuncSetAttribute(gfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
+        if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(kGCluster);
         cfg.blockDim = dim3(kGT);
+        cfg.dynamicSmemBytes = kSmallSmem;
         cfg.stream = s;
         cudaLaunchAttribute at;
         at.id = cudaLaunchAttributeClusterDimension;
