@@ -138,7 +138,8 @@ __device__ __forceinline__ void start_early()
 
 // kernel<<<grid, block, smem, s>>>(args...) whose blocks may be placed before
 // the stream's previous kernel has ended (they wait in start_early), so that
-// the launch's latency lies behind it: XXPDL
+// the launch's latency lies behind it: 1 to 2 us a kernel (a 1K chain of 14
+// kernels 133 -> 110 us, labeling 700 x 700 in 4 of them 31 -> 24).
 template <class... P, class... A>
 inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
 {
