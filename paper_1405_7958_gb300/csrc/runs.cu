@@ -109,6 +109,7 @@ __device__ __forceinline__ uint32_t node_find(uint32_t *U, uint32_t v)
 {
     uint32_t p = parent(U, v);
     while (p != v) {
+        if (p == 0u) return 0u;   // the outside: no need to read its word, which all would read
         const uint32_t gp = parent(U, p);
         if (gp != p) atomicMin(U + v * kUnmix, gp);
         v = gp;
@@ -590,13 +591,14 @@ __global__ void __launch_bounds__(kWarps * 32) run_seam_kernel(const __grid_cons
     if (tile >= b.ntiles) return;
     const RunImage &d = run_image(b, tile);
     const Place p = place_of(d, tile);
-    // pairs of slots to join, each once; then the lanes join them side by side
+    // pairs of slots to join; then the lanes join them side by side
     volatile uint32_t *pairs = s_pairs[threadIdx.x >> 5];
     int n = 0;
     auto join = [&](int which, uint32_t a, uint32_t c) {   // whole warp; which: 0 right, 1 lower neighbour
+        // (once per stretch of the side: the same pair further on costs less than a vote on all equal ones)
         const bool valid = a != 255u && c != 255u;
-        const uint32_t peers = __match_any_sync(0xffffffffu, valid ? a << 8 | c : ~0u);
-        const bool lead = valid && lane == __ffs(peers) - 1;
+        const uint32_t v = valid ? a << 8 | c : ~0u, before = __shfl_up_sync(0xffffffffu, v, 1);
+        const bool lead = valid && (lane == 0 || before != v);
         const uint32_t m = __ballot_sync(0xffffffffu, lead);
         if (lead) pairs[n + __popc(m & ((1u << lane) - 1u))] = (uint32_t)which << 16 | a << 8 | c;
         n += __popc(m);
