@@ -36,11 +36,11 @@ BYTES_RECON = 2          # reconstruction: read mask 1, write R 1
 BYTES_PASS = 3           # one directional raster pass over a pixel: read R and I, write R
 PASSES_PER_ITERATION = 3 # a dense tile iteration: down, up and row passes
 TILE_PX = 32 * 64        # pixels of one warp tile
-# ncu summary of the propagation kernel on the bench workload: its DRAM
-# traffic per launch is reported while the kernel sources still hash to the
+# ncu summary of the reconstruction's kernels on the bench workload: their
+# DRAM traffic per step is reported while the kernel sources still hash to the
 # value recorded there (else traffic is null: the counters are stale)
-TRAFFIC_PROFILE = os.path.join(ROOT, "profiles", "recon_persistent_8x4k.md")
-KERNEL_SOURCES = ("paper_1405_7958_gb300/csrc/recon.cu", "paper_1405_7958_gb300/csrc/recon.cuh")
+TRAFFIC_PROFILE = os.path.join(ROOT, "profiles", "contract_8x4k.md")
+KERNEL_SOURCES = ("paper_1405_7958_gb300/csrc/contract.cu", "paper_1405_7958_gb300/csrc/contract.cuh")
 
 
 def parse():
@@ -84,8 +84,8 @@ def kernel_hash() -> str:
 
 
 def profiled_traffic():
-    """DRAM bytes per launch of the propagation kernel from its committed ncu
-    summary, or None when the summary is missing or the kernel has changed."""
+    """DRAM bytes per step of the reconstruction's kernels from their committed
+    ncu summary, or None when the summary is missing or a kernel has changed."""
     try:
         with open(TRAFFIC_PROFILE) as fh:
             text = fh.read()
@@ -669,7 +669,7 @@ def run_native(a, rank, world, local_rank):
         serving = {"rate_tiles_s": 800, "seconds": a.serve_seconds, "tiles": "512..4096 px sides",
                    **serve.summarize(reqs, a.serve_seconds)}
 
-    # dominant kernel: the propagation sweeps (one launch per step)
+    # dominant stage: the reconstruction by contraction (three launches per step, the first 85 % of it)
     sweep_ms, sweep_n = phases["recon_sweep"]
     peak, peak_kind = load_peaks()
     roof = None
@@ -677,17 +677,18 @@ def run_native(a, rank, world, local_rank):
         per_launch_s = sweep_ms / sweep_n / 1000.0
         algo_bytes = BYTES_RECON * px * a.batch
         ach = algo_bytes / per_launch_s / 1e9
-        its = visits[1]       # dense tile iterations of one step (the last one)
-        pass_bytes = its * PASSES_PER_ITERATION * TILE_PX * BYTES_PASS
+        its = visits[1]       # dense tile iterations of one step (the last one; 0 by contraction)
         ms_alone, n_alone = phases_alone["recon_sweep"]
         alone_s = ms_alone / max(n_alone, 1) / 1000.0
-        roof = {"kernel": "recon_persistent_kernel<8,0>", "bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
+        roof = {"kernel": "ct_local_kernel + ct_seam_kernel + ct_global_kernel", "bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
                 "launch_ms_alone": alone_s * 1000, "achieved_alone": algo_bytes / alone_s / 1e9,
                 "frac_alone": algo_bytes / alone_s / 1e9 / peak,
                 "frac": ach / peak, "peak_source": peak_kind, "traffic": profiled_traffic(),
-                "algorithmic_bytes_per_launch": algo_bytes, "launch_ms": per_launch_s * 1000,
-                "pass_bytes_per_launch": pass_bytes, "pass_equivalent_gbs": pass_bytes / per_launch_s / 1e9,
-                "pass_equivalent_frac": pass_bytes / per_launch_s / 1e9 / peak}
+                "algorithmic_bytes_per_launch": algo_bytes, "launch_ms": per_launch_s * 1000}
+        if its:
+            pass_bytes = its * PASSES_PER_ITERATION * TILE_PX * BYTES_PASS
+            roof |= {"pass_bytes_per_launch": pass_bytes, "pass_equivalent_gbs": pass_bytes / per_launch_s / 1e9,
+                     "pass_equivalent_frac": pass_bytes / per_launch_s / 1e9 / peak}
 
     # end to end through the public API with host buffers: every step copies
     # its inputs from pinned host memory, runs the chain and copies labels and

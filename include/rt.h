@@ -102,9 +102,10 @@ typedef struct rt_ctx rt_ctx;
  * usable; RT_ENOMEM: the reservation failed). */
 RT_API rt_status rt_create(rt_ctx **ctx, int device, size_t workspace_bytes);
 
-/* Bounds of the iterative steps of the single-operation entry points
- * (rt_reconstruct, rt_fill_holes) on this context, and the defaults of
- * rt_segment_batch: max_iters > 0 lets one reconstruction propagation make
+/* Bounds of the propagations of rt_reconstruct on this context, and the
+ * defaults of rt_segment_batch (a call with such a bound runs the
+ * propagation, not the contraction; the other operations have nothing to
+ * bound): max_iters > 0 lets one reconstruction propagation make
  * at most max_iters tile visits per 32 x 64 tile of its images on average (0: no
  * bound; how many visits a propagation needs depends on the schedule, so a
  * bound close to the need may or may not be reached); timeout_ms > 0 bounds
@@ -507,8 +508,10 @@ RT_API void rt_seg_params_default(rt_seg_params *p);
  *   L' = label_area(F, 8, [min_area, max_area]); D = edt(L' >= 0).
  * `tiles` is a HOST array (copied before return); all outputs are device
  * buffers. The per-tile outputs are identical to running the single-tile
- * entry points one tile at a time. Tiles run in chunks of up to 32; every
- * stage of the chain is one launch for the whole chunk. A single tile may be
+ * entry points one tile at a time. R itself is computed where a tile of the
+ * chunk returns it; where none does, RT_AUTO finds only where it is below
+ * the threshold. Tiles run in chunks of up to 32; every stage of the chain
+ * is one to four launches for the whole chunk. A single tile may be
  * a whole slide (up to 32768 x 32768): the propagations cross the seams of
  * their internal tiles and the labels join across block edges, so the
  * result is that of the slide as one image.

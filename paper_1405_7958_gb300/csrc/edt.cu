@@ -34,12 +34,6 @@ namespace rtk {
 constexpr int kSeg = 32;
 constexpr uint16_t kInf = 0xFFFFu;
 
-size_t edt_workspace_bytes(int H, int W)
-{
-    const int64_t nseg = ceil_div(H, kSeg);
-    return (size_t)H * W * sizeof(uint16_t) + (size_t)3 * nseg * W * sizeof(int32_t) + 512;
-}
-
 __device__ __forceinline__ bool edt_is_bg(const EdtArgs &a, int r, int c)
 {
     return a.fg8[(int64_t)r * a.ld_in + c] == 0;

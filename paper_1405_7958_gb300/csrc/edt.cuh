@@ -17,7 +17,6 @@ struct EdtArgs {
     uint32_t *any_bg;       // workspace word
 };
 
-size_t edt_workspace_bytes(int H, int W);
 cudaError_t launch_edt(const EdtArgs &a, cudaStream_t s);
 
 // A batch of images given as bits of their foreground, per 64 x 64 tile 64
