@@ -127,6 +127,22 @@ __device__ __forceinline__ void store_bytes(uint8_t *o, int n, const uint32_t (&
     }
 }
 
+// 64 ints of a row, value(c) for column c, by 16 threads (q = 0 .. 15): the
+// aligned quads of the row, whatever its alignment, and its ends one by one.
+template <class V>
+__device__ __forceinline__ void store_row64(int32_t *row, int q, V &&value)
+{
+    const int head = (int)((0u - (uint32_t)(uintptr_t)row) >> 2) & 3, at = head + 4 * q;
+    if (at + 4 <= 64) {
+        *reinterpret_cast<int4 *>(row + at) = make_int4(value(at), value(at + 1), value(at + 2), value(at + 3));
+    } else {
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (at + k < 64) row[at + k] = value(at + k);
+    }
+    if (q < head) row[q] = value(q);
+}
+
 // First statement of a kernel launched by launch_early: lets the next such
 // kernel of the stream take its place on the SMs as soon as all blocks of
 // this one have theirs, and waits until the kernels before this one are

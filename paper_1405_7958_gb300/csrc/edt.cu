@@ -235,6 +235,9 @@ __global__ void __launch_bounds__(NT) edt_near_kernel(const __grid_constant__ Ed
         if (wide) {
             for (int i = t >> 4; i < nr; i += NT / 16)
                 reinterpret_cast<int4 *>(d.d2 + (int64_t)(r0 + i) * d.ld_d2 + c0)[t & 15] = make_int4(0, 0, 0, 0);
+        } else if (nc == kEdtSide) {
+            for (int i = t >> 4; i < nr; i += NT / 16)
+                store_row64(d.d2 + (int64_t)(r0 + i) * d.ld_d2 + c0, t & 15, [](int) { return 0; });
         } else {
             for (int i = t >> 6; i < nr; i += NT / 64)
                 if ((t & 63) < nc) d.d2[(int64_t)(r0 + i) * d.ld_d2 + c0 + (t & 63)] = 0;
@@ -311,6 +314,10 @@ __global__ void __launch_bounds__(NT) edt_near_kernel(const __grid_constant__ Ed
             reinterpret_cast<int4 *>(d.d2 + (int64_t)(r0 + i) * d.ld_d2 + c0)[t & 15] =
                 make_int4((int)(v.x & 0xffffu), (int)(v.x >> 16), (int)(v.y & 0xffffu), (int)(v.y >> 16));
         }
+    } else if (nc == kEdtSide) {
+        for (int i = t >> 4; i < nr; i += NT / 16)
+            store_row64(d.d2 + (int64_t)(r0 + i) * d.ld_d2 + c0, t & 15,
+                        [&](int c) { return (int)dist[i * kEdtSide + c]; });
     } else {
         for (int i = t >> 6; i < nr; i += NT / 64)
             if ((t & 63) < nc) d.d2[(int64_t)(r0 + i) * d.ld_d2 + c0 + (t & 63)] = dist[i * kEdtSide + (t & 63)];
