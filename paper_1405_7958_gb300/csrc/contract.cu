@@ -67,7 +67,7 @@ static_assert(sizeof(uint16_t) * kCtPx == sizeof(uint32_t) * kRoots + 2 * sizeof
 
 // For every set of larger neighbours (bit j: kNear[j]) and code of the
 // largest: one neighbour of each group that does not hold the largest, as up
-// to three nibbles code + 1.
+// to three nibbles code + 1, and their number in the fourth.
 struct alignas(16) GroupTable {
     uint16_t v[kCodes * 256];
 };
@@ -95,7 +95,7 @@ constexpr GroupTable group_table()
                 left &= ~grp;
                 bool own = false;
                 for (int j = 0; j < 8; ++j) own = own || (((grp >> j) & 1) && kNear[j] == c);
-                if (!own) out |= (kNear[rep] + 1) << shift, shift += 4;
+                if (!own) out += 0x1000 | (kNear[rep] + 1) << shift, shift += 4;
             }
             g.v[c * 256 + m] = (uint16_t)out;
         }
@@ -139,13 +139,14 @@ __device__ __forceinline__ uint32_t max3(uint32_t a, uint32_t b, uint32_t c) { r
 
 // ------------------------------------------------------------------ local
 // NT threads; a warp takes 64 / warps rows, a lane two adjacent columns.
-// Bound by instruction issue (77 % active, 49 k warp instructions a tile,
+// Bound by instruction issue (75 % active, 47 k warp instructions a tile,
 // 220 us per 4096 x 4096 image, DRAM idle). What it measured on that image:
 // edges from 2 x 2 windows with flags 377 us; cluster ids in the edges, lists
 // of open roots, parents apart from the pixel words 290; edges from groups of
 // larger neighbours by table 240; loops kept rolled (43 KB of code instead of
 // 88, which missed the instruction cache) and five CTAs an SM instead of four
-// 220. The first full version took 373 us.
+// 220; edges counted first and written at one position per warp, not per row,
+// 215. The first full version took 373 us.
 template <bool MARKER, int NT>
 __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const __grid_constant__ CtBatch b)
 {
@@ -350,24 +351,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
         uint32_t u[4], m[4], n[4];
         load(rs - 1, u);
         load(rs, m);
-        // a pixel's second and third edge (rare) wait in `more`, 16 bits each
-        unsigned long long more = 0;
-        auto put = [&](uint32_t e0, uint32_t e1) {   // whole warp
-            const uint32_t b0 = __ballot_sync(0xffffffffu, e0 != 0u), b1 = __ballot_sync(0xffffffffu, e1 != 0u);
-            const int n0 = __popc(b0);
-            int at = 0;
-            if (lane == 0) at = atomicAdd(&s_edges, n0 + __popc(b1));
-            at = __shfl_sync(0xffffffffu, at, 0);
-            const int p0 = at + __popc(b0 & below), p1 = at + n0 + __popc(b1 & below);
-            if (e0 && p0 < kList) list[p0] = e0;   // p < kList: always (see kList)
-            if (e1 && p1 < kList) list[p1] = e1;
-        };
-        auto flush = [&]() {
-            do {
-                put((uint32_t)more & 0xffffu, (uint32_t)(more >> 16) & 0xffffu);
-                more >>= 32;
-            } while (__any_sync(0xffffffffu, more != 0ull));
-        };
+        // the pixels' groups take the place of their parents and are counted; then every lane writes its own
+        int cnt = 0;
 #pragma unroll 1   // the loops over rows stay rolled: the kernel's time is lost to instruction fetch otherwise
         for (int j = 0; j < kRows; ++j) {
             const int r = rs + j;
@@ -384,22 +369,38 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
                 const uint32_t code = q ? pp >> 28 : (pp >> 12) & 0xfu;
                 g[q] = table[code * 256u + (set & 0xffu)];
                 if (m[q + 1] == 0u) g[q] = 0u;
+                cnt += (int)(g[q] >> 12);
             }
-            const uint32_t at0 = (uint32_t)(r * kCtSide + cl);
-            put(g[0] ? at0 | (g[0] & 0xfu) << 12 : 0u, g[1] ? (at0 + 1u) | (g[1] & 0xfu) << 12 : 0u);
-            if ((g[0] | g[1]) >> 4) {
-#pragma unroll
-                for (int q = 0; q < 2; ++q)
-#pragma unroll 1
-                    for (uint32_t f = g[q] >> 4; f; f >>= 4) more = more << 16 | (at0 + q) | (f & 0xfu) << 12;
-            }
-            // of two adjacent pixels one at most has four groups (its corners
-            // larger, its edge neighbours not): a row adds at most 2 + 1
-            if (__any_sync(0xffffffffu, more >> 16 != 0ull)) flush();
+            reinterpret_cast<volatile uint32_t *>(P)[(r * kCtSide + cl) / 2] = g[0] | g[1] << 16;
 #pragma unroll
             for (int q = 0; q < 4; ++q) u[q] = m[q], m[q] = n[q];
         }
-        if (__any_sync(0xffffffffu, more != 0ull)) flush();
+        int pos = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, pos, o);
+            if (lane >= o) pos += v;
+        }
+        int base = 0;
+        if (lane == 31) base = atomicAdd(&s_edges, pos);
+        pos += __shfl_sync(0xffffffffu, base, 31) - cnt;
+#pragma unroll 1
+        for (int j = 0; j < kRows && cnt; ++j) {
+            const uint32_t at0 = (uint32_t)((rs + j) * kCtSide + cl);
+            const uint32_t gg = reinterpret_cast<volatile uint32_t *>(P)[at0 / 2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uint32_t f = (q ? gg >> 16 : gg) & 0xfffu;
+                if (!f) continue;
+                if (pos < kList) list[pos] = (at0 + q) | (f & 0xfu) << 12;   // pos < kList: always (see kList)
+                ++pos;
+#pragma unroll 1
+                while (f >>= 4) {
+                    if (pos < kList) list[pos] = (at0 + q) | (f & 0xfu) << 12;
+                    ++pos;
+                }
+            }
+        }
     }
     __syncthreads();
 
