@@ -286,6 +286,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
     // of flat images.
     {
         bool bad = false;
+        const bool rim_tile = ty == 0 || tx == 0 || ty == d.ny - 1 || tx == d.nx - 1;   // holds pixels of the image's border
 #pragma unroll 2
         for (int j = 0; j < kRows; ++j) {
             const int at = (rs + j) * kCtSide + cl;
@@ -319,7 +320,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
                     bad |= J > I;
                     const uint32_t s = kRootBit | min(J, I);
                     if (nlink[k] < s) atomicMax(sk, s);
-                } else if (gr == 0 || gr == d.H - 1 || gc == 0 || gc == d.W - 1) {
+                } else if (rim_tile && (gr == 0 || gr == d.H - 1 || gc == 0 || gc == d.W - 1)) {
                     atomicMax(sk, kRootBit | I);
                 }
             }
@@ -366,9 +367,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
                 uint32_t set = 0;
 #pragma unroll
                 for (int j = 7; j >= 0; --j) set = __funnelshift_l(m[q + 1] - near[j], set, 1);
-                const uint32_t code = q ? pp >> 28 : (pp >> 12) & 0xfu;
-                g[q] = table[code * 256u + (set & 0xffu)];
-                if (m[q + 1] == 0u) g[q] = 0u;
+                // (code << 8 | set; code 4, a root or outside the image, has no groups)
+                g[q] = table[((q ? pp >> 20 : pp >> 4) & 0xf00u) | set];
                 cnt += (int)(g[q] >> 12);
             }
             reinterpret_cast<volatile uint32_t *>(P)[(r * kCtSide + cl) / 2] = g[0] | g[1] << 16;
