@@ -464,6 +464,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
         int any = 0;
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
+            if (q * NT >= nl) break;   // (q > 0: round 0 only, as a rule)
             dec[q] = 0xffffu;
             id[q] = 0u;
             if (t + q * NT >= nl) continue;
@@ -484,14 +485,16 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
         if (t == 0) s_live[~round & 1] = 0;
         if (!__syncthreads_or(any)) break;
 #pragma unroll
-        for (int q = 0; q < kPer; ++q)
+        for (int q = 0; q < kPer; ++q) {
+            if (q * NT >= nl) break;
             if ((dec[q] & 0xffffu) != 0xffffu) nlink[id[q] & 0xffffu] = dec[q] & 0xffffffu;
+        }
         __syncthreads();
         // joined: find the new root, with the smallest weight on the way, and
         // hand it the sources; the others make the next list
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
-            if (warp * 32 + q * NT >= nl) continue;   // whole warp
+            if (warp * 32 + q * NT >= nl) break;   // whole warp
             const bool in = t + q * NT < nl, joined = (dec[q] & 0xffffu) != 0xffffu;
             const uint32_t k = id[q] & 0xffffu;
             if (joined) {
