@@ -40,9 +40,8 @@
 //
 // Measured on one GB300 against the directional sweeps (rt_segment_batch or
 // rt_reconstruct, whole call; the chain's other stages are the same):
-// 512 x 512 reconstruction 78 us against 357; one 4096 x 4096 tile 0.47 ms
-// against 1.17; eight of them 2.6 ms against 4.7; a 16384 x 16384 slide 5.0
-// ms against 8.5. So the contraction runs wherever the call leaves the
+// 512 x 512 reconstruction 67 us against 357; one 4096 x 4096 tile 0.43 ms
+// against 1.13; eight of them 2.42 ms against 4.6. So the contraction runs wherever the call leaves the
 // schedule to the library.
 #include "contract.cuh"
 
@@ -139,14 +138,15 @@ __device__ __forceinline__ uint32_t max3(uint32_t a, uint32_t b, uint32_t c) { r
 
 // ------------------------------------------------------------------ local
 // NT threads; a warp takes 64 / warps rows, a lane two adjacent columns.
-// Bound by instruction issue (75 % active, 47 k warp instructions a tile,
-// 220 us per 4096 x 4096 image, DRAM idle). What it measured on that image:
+// Bound by instruction issue (74 % active, 45 k warp instructions a tile,
+// 205 us per 4096 x 4096 image, DRAM idle). What it measured on that image:
 // edges from 2 x 2 windows with flags 377 us; cluster ids in the edges, lists
 // of open roots, parents apart from the pixel words 290; edges from groups of
 // larger neighbours by table 240; loops kept rolled (43 KB of code instead of
 // 88, which missed the instruction cache) and five CTAs an SM instead of four
 // 220; edges counted first and written at one position per warp, not per row,
-// 215. The first full version took 373 us.
+// 215; no tests of the image's border in inner tiles and none of roots that
+// no warp has 205. The first full version took 373 us.
 template <bool MARKER, int NT>
 __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const __grid_constant__ CtBatch b)
 {
