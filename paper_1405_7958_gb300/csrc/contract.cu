@@ -1466,9 +1466,9 @@ cudaError_t launch_contract(const CtBatch &b, int num_sms, uint64_t timeout_ns, 
 {
     const bool given = b.img[0].marker != nullptr;   // all images of a batch, or none
     // With two tiles per SM or fewer little hides a tile's latency: then 512
-    // threads share it (512 x 512: 75 us against 87 for both stages, 1024 x
-    // 1024: 112 against 117; equal from 1536 x 1536 on, and above that the
-    // barriers of larger CTAs cost more: 247 us against 220 at 4096 x 4096).
+    // threads share it (512 x 512: 66 us against 75 for all stages, 1024 x
+    // 1024: 85 against 90; equal at 1280 x 1280, and above that the barriers
+    // of larger CTAs cost more: 108 against 102 at 1536 x 1536).
     const bool few = b.ntiles <= kFewTiles;
     auto *fn = few ? (given ? ct_local_kernel<true, 512> : ct_local_kernel<false, 512>)
                    : (given ? ct_local_kernel<true, 256> : ct_local_kernel<false, 256>);
@@ -1481,7 +1481,8 @@ cudaError_t launch_contract(const CtBatch &b, int num_sms, uint64_t timeout_ns, 
     const int64_t units = (int64_t)b.ntiles * kCtUnits;
     const int need = (int)ceil_div(units, kGT / 32);
     // One cluster of eight CTAs while its 256 warps hold two units each at
-    // most (512 x 512: 90 us against 110 for both stages; 768 x 768: equal).
+    // most (640 x 640: 71 us against 73 for all stages; 768 x 768: equal; 1024
+    // x 1024: 88 against 85); a smaller one may fit a single CTA.
     if (units <= kGClusterUnits) {
         auto *gfn = ct_global_kernel<true>;
         e = cudaFuncSetAttribute(gfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
