@@ -87,7 +87,10 @@ class Phase {
     PhaseRec rec_{0, nullptr, nullptr};
 };
 
-constexpr uint64_t kSweepTimeoutNs = 20000000000ull;   // default bound on one propagation (20 s)
+// Default bound on one propagation (20 s). The barriers of the other
+// cooperative kernels wait this long too, whatever the caller's bound on a
+// propagation: they have no partial result to stop at.
+constexpr uint64_t kSweepTimeoutNs = 20000000000ull;
 
 // Bump allocator over the context workspace (256-byte aligned pieces).
 struct Carve {
@@ -1031,7 +1034,7 @@ rt_status rt_edt(rt_ctx *ctx, const uint8_t *fg, int64_t ld_fg, int32_t *d2, int
     Phase ph(ctx, RT_PHASE_EDT, s);
     ctx->launches += 3;
     RT_CUDA_TRY(launch_run_pack(r, s));
-    return cuda_status(launch_edt_bits_batch(b, ctx->num_sms, ctx_limits(ctx).timeout_ns, s));
+    return cuda_status(launch_edt_bits_batch(b, ctx->num_sms, kSweepTimeoutNs, s));
 }
 
 rt_status rt_watershed(rt_ctx *ctx, const int32_t *labels, int64_t ld_lab, const int32_t *d2, int64_t ld_d2, int H,
@@ -1367,7 +1370,7 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
         {
             Phase ph(ctx, RT_PHASE_EDT, s);
             ctx->launches += 2;
-            RT_CUDA_TRY(launch_edt_bits_batch(c.eb, ctx->num_sms, lim.timeout_ns, s));
+            RT_CUDA_TRY(launch_edt_bits_batch(c.eb, ctx->num_sms, kSweepTimeoutNs, s));
         }
         if (aside) {   // enqueued last: its launches delay none of the chain's
             RT_CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork, 0));

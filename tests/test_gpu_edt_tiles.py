@@ -56,3 +56,23 @@ def test_no_background_and_many_tiles(rt):
     m = (rng.random((4200, 4161)) < 0.3).astype(np.uint8)   # 66 x 66 tiles
     m[1000:1400, 700:1900] = 1
     same(rt, m)
+
+
+def test_a_bound_on_propagations_leaves_the_transform_alone(rt):
+    """A stripe of foreground 256 columns wide and 32768 rows high: the far
+    stage's walk over its empty segments takes some of the blocks milliseconds
+    while the others wait at the barrier. rt_set_limits bounds propagations
+    only, so the distances are exact and the status is RT_OK."""
+    H, W, c0, n = 32768, 4096, 1024, 256
+    fg = torch.zeros((H, W), dtype=torch.uint8, device="cuda")
+    fg[:, c0:c0 + n] = 1
+    c = torch.arange(n, device="cuda", dtype=torch.int32)
+    want = torch.minimum(c + 1, n - c) ** 2
+    st = torch.full((1,), 99, dtype=torch.int32, device="cuda")
+    ctx = rt.Context()
+    ctx.set_limits(timeout_ms=1)
+    d = rt.edt(fg, status=st, ctx=ctx)
+    assert int(st.item()) == rt.RT_OK
+    assert bool((d[:, c0:c0 + n] == want).all())
+    assert int(d.sum(dtype=torch.int64).item()) == H * int(want.sum().item())
+    ctx.close()
