@@ -29,6 +29,8 @@ struct rt_ctx {
     int num_sms = 0;
     void *ws = nullptr;       // device workspace
     size_t ws_bytes = 0;
+    bool ws_captured = false;   // a captured call has used ws
+    std::vector<void *> kept;   // earlier workspaces that captured calls have used
     uint32_t *visits_dev = nullptr;  // [visits, iterations] of the last reconstruction (workspace)
     int64_t launches = 0;     // kernels launched
     bool timing = false;
@@ -123,22 +125,58 @@ class DeviceGuard {
     int prev_ = 0, dev_ = 0;
 };
 
-rt_status ensure_ws(rt_ctx *ctx, size_t bytes)
+// Whether work on s is being captured into a graph.
+bool capturing(cudaStream_t s)
 {
-    if (bytes <= ctx->ws_bytes) return RT_OK;
-    if (ctx->ws) {
-        cudaFree(ctx->ws);
-        ctx->ws = nullptr;
-        ctx->ws_bytes = 0;
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &c) != cudaSuccess) cudaGetLastError();
+    return c == cudaStreamCaptureStatusActive;
+}
+
+// A workspace of at least `bytes` for a call on s. A block that a graph may
+// hold (ws_captured) is not freed when the workspace grows but kept for the
+// graph until the context goes; the next block is then twice as large if it
+// can be, so that the kept ones are never more than the current one. Under
+// capture the allocation itself stays outside the graph (relaxed capture
+// mode): operations have come to need more than a context was reserved with
+// for them, and a call that fitted must not end its capture.
+rt_status ensure_ws(rt_ctx *ctx, size_t bytes, cudaStream_t s)
+{
+    const bool cap = capturing(s);
+    if (bytes > ctx->ws_bytes) {
+        size_t want = (size_t)round_up((int64_t)bytes, 1 << 20);
+        const size_t exact = want;
+        const bool keep = ctx->ws && (cap || ctx->ws_captured);
+        if (keep) {
+            try {
+                ctx->kept.reserve(ctx->kept.size() + 1);
+            } catch (const std::bad_alloc &) {
+                return RT_ENOMEM;
+            }
+            if (want < 2 * ctx->ws_bytes) want = 2 * ctx->ws_bytes;
+        } else if (ctx->ws) {
+            cudaFree(ctx->ws);
+            ctx->ws = nullptr;
+            ctx->ws_bytes = 0;
+        }
         ctx->visits_dev = nullptr;
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if (cap) cudaThreadExchangeStreamCaptureMode(&mode);
+        void *ws = nullptr;
+        while (cudaMalloc(&ws, want) != cudaSuccess) {
+            cudaGetLastError();
+            ws = nullptr;
+            if (want == exact) break;
+            want = exact;
+        }
+        if (cap) cudaThreadExchangeStreamCaptureMode(&mode);
+        if (!ws) return RT_ENOMEM;
+        if (keep) ctx->kept.push_back(ctx->ws);
+        ctx->ws = ws;
+        ctx->ws_bytes = want;
+        ctx->ws_captured = false;
     }
-    size_t want = (size_t)round_up((int64_t)bytes, 1 << 20);
-    if (cudaMalloc(&ctx->ws, want) != cudaSuccess) {
-        cudaGetLastError();
-        ctx->ws = nullptr;
-        return RT_ENOMEM;
-    }
-    ctx->ws_bytes = want;
+    ctx->ws_captured |= cap;
     return RT_OK;
 }
 
@@ -729,7 +767,12 @@ rt_status rt_create(rt_ctx **ctx, int device, size_t workspace_bytes)
         delete c;
         return RT_ECUDA;
     }
-    if (workspace_bytes > 0 && ensure_ws(c, workspace_bytes) != RT_OK) {
+    if (workspace_bytes > 0) {
+        const size_t want = (size_t)round_up((int64_t)workspace_bytes, 1 << 20);
+        if (cudaMalloc(&c->ws, want) == cudaSuccess) c->ws_bytes = want;
+    }
+    if (c->ws_bytes < workspace_bytes) {
+        cudaGetLastError();
         free_host_side(c);
         delete c;
         return RT_ENOMEM;
@@ -767,6 +810,7 @@ void rt_destroy(rt_ctx *ctx)
     DeviceGuard g(ctx->device);
     if (ctx->ws) {
         cudaDeviceSynchronize();
+        for (void *p : ctx->kept) cudaFree(p);
         cudaFree(ctx->ws);
     }
     for (const PhaseRec &r : ctx->recs) {
@@ -879,7 +923,7 @@ rt_status rt_reconstruct(rt_ctx *ctx, const uint8_t *marker, int64_t ld_marker, 
             if (pass) cc.base = (char *)ctx->ws;
             cerr = cc.take<int32_t>(1);
             carve_contract(cc, cb);
-            if (!pass && (cst = ensure_ws(ctx, cc.off)) != RT_OK) return cst;
+            if (!pass && (cst = ensure_ws(ctx, cc.off, s)) != RT_OK) return cst;
         }
         if (dev_status) cerr = dev_status;
         RT_CUDA_TRY(cudaMemsetAsync(cerr, 0, sizeof(int32_t), s));
@@ -896,7 +940,7 @@ rt_status rt_reconstruct(rt_ctx *ctx, const uint8_t *marker, int64_t ld_marker, 
     Carve cv;
     ReconWs w;
     carve_recon(cv, b, w, false, fq_cap);
-    rt_status st = ensure_ws(ctx, cv.off);
+    rt_status st = ensure_ws(ctx, cv.off, s);
     if (st != RT_OK) return st;
     cv = Carve();
     cv.base = (char *)ctx->ws;
@@ -936,7 +980,7 @@ rt_status rt_fill_holes(rt_ctx *ctx, const uint8_t *in, int64_t ld_in, uint8_t *
         carve_bits(cv, b);
         carve_runs_late(cv, b, true, false);
         rt_status st = RT_OK;
-        if (!real && (st = ensure_ws(ctx, cv.off)) != RT_OK) return st;
+        if (!real && (st = ensure_ws(ctx, cv.off, s)) != RT_OK) return st;
     }
     if (dev_status) RT_CUDA_TRY(cudaMemsetAsync(dev_status, 0, sizeof(int32_t), s));
     Phase ph(ctx, RT_PHASE_FILL, s);
@@ -955,7 +999,7 @@ rt_status rt_label_area(rt_ctx *ctx, const uint8_t *bin, int64_t ld_bin, int32_t
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
     if ((int64_t)run_tiles(H, W) <= kUfMaxTiles) {
-        rt_status st = ensure_ws(ctx, uf_workspace_bytes(H, W));
+        rt_status st = ensure_ws(ctx, uf_workspace_bytes(H, W), s);
         if (st != RT_OK) return st;
         UfImage u;
         std::memset(&u, 0, sizeof(u));
@@ -991,7 +1035,7 @@ rt_status rt_label_area(rt_ctx *ctx, const uint8_t *bin, int64_t ld_bin, int32_t
         carve_bits(cv, b);
         carve_runs_late(cv, b, false, true);
         rt_status st = RT_OK;
-        if (!real && (st = ensure_ws(ctx, cv.off)) != RT_OK) return st;
+        if (!real && (st = ensure_ws(ctx, cv.off, s)) != RT_OK) return st;
     }
     if (dev_status) RT_CUDA_TRY(cudaMemsetAsync(dev_status, 0, sizeof(int32_t), s));
     Phase ph(ctx, RT_PHASE_LABEL, s);
@@ -1022,7 +1066,7 @@ rt_status rt_edt(rt_ctx *ctx, const uint8_t *fg, int64_t ld_fg, int32_t *d2, int
         carve_bits(cv, r);
         char *ews = cv.take<char>(edt_bits_workspace_bytes(H, W));
         rt_status st = RT_OK;
-        if (!real && (st = ensure_ws(ctx, cv.off)) != RT_OK) return st;
+        if (!real && (st = ensure_ws(ctx, cv.off, s)) != RT_OK) return st;
         if (real) edt_bits_add(b, H, W, d2, ld_d2, ews);
     }
     b.bits = r.bits;
@@ -1048,7 +1092,7 @@ rt_status rt_watershed(rt_ctx *ctx, const int32_t *labels, int64_t ld_lab, const
         return RT_EINVAL;
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
-    rt_status st = ensure_ws(ctx, obj_workspace_bytes(H, W, false, true, 0));
+    rt_status st = ensure_ws(ctx, obj_workspace_bytes(H, W, false, true, 0), s);
     if (st != RT_OK) return st;
     ObjArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -1080,7 +1124,7 @@ rt_status rt_object_features(rt_ctx *ctx, const int32_t *labels, int64_t ld_lab,
     if (cap > 0 && (!obj_labels || !feat)) return RT_EINVAL;
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
-    rt_status st = ensure_ws(ctx, obj_workspace_bytes(H, W, true, false, cap));
+    rt_status st = ensure_ws(ctx, obj_workspace_bytes(H, W, true, false, cap), s);
     if (st != RT_OK) return st;
     ObjArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -1111,7 +1155,7 @@ rt_status rt_synth_tile(rt_ctx *ctx, uint8_t *out, int64_t ld, int H, int W, uin
     if (vlo < 0 || vhi > 255 || vlo > vhi || rmin < 0 || rmax < rmin || amin < 0 || amax < amin) return RT_EINVAL;
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
-    rt_status st = ensure_ws(ctx, synth_workspace_bytes(H, W));
+    rt_status st = ensure_ws(ctx, synth_workspace_bytes(H, W), s);
     if (st != RT_OK) return st;
     SynthArgs a;
     a.H = H;
@@ -1158,7 +1202,7 @@ rt_status rt_tile_features(rt_ctx *ctx, const uint8_t *const *imgs, const int64_
     FeatBatch fb;
     Carve cv;
     layout(cv, fb);
-    rt_status st = ensure_ws(ctx, cv.off);
+    rt_status st = ensure_ws(ctx, cv.off, s);
     if (st != RT_OK) return st;
     cv = Carve();
     cv.base = (char *)ctx->ws;
@@ -1205,7 +1249,7 @@ rt_status rt_mlp_backward(rt_ctx *ctx, const uint16_t *wb, const float *norm, co
 {
     if (!ctx || !wb || !norm || !x || !act || !logits || !label || !grad || B < 1) return RT_EINVAL;
     DeviceGuard g(ctx->device);
-    rt_status st = ensure_ws(ctx, mlp_backward_workspace_bytes(B));
+    rt_status st = ensure_ws(ctx, mlp_backward_workspace_bytes(B), (cudaStream_t)stream);
     if (st != RT_OK) return st;
     ctx->launches += 2;
     return cuda_status(launch_mlp_backward(wb, norm, x, act, logits, label, B, grad, loss, (float *)ctx->ws,
@@ -1218,7 +1262,7 @@ rt_status rt_mlp_backward_tc(rt_ctx *ctx, const uint16_t *wb, const float *norm,
 {
     if (!ctx || !wb || !norm || !x || !act || !logits || !label || !grad || B < 1) return RT_EINVAL;
     DeviceGuard g(ctx->device);
-    rt_status st = ensure_ws(ctx, mlp_backward_tc_workspace_bytes(B));
+    rt_status st = ensure_ws(ctx, mlp_backward_tc_workspace_bytes(B), (cudaStream_t)stream);
     if (st != RT_OK) return st;
     ctx->launches += 2;
     return cuda_status(launch_mlp_backward_tc(wb, norm, x, act, logits, label, B, grad, loss, (float *)ctx->ws,
@@ -1309,7 +1353,7 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
     const bool learned = P.policy == RT_POLICY_LEARNED && ctx->picker_wb && ctx->picker_norm;
     const Limits lim = seg_limits(ctx, P);
     // one allocation for the largest chunk, before anything is enqueued
-    rt_status st = ensure_ws(ctx, segment_ws_bytes(tiles, n, P, learned, ctx));
+    rt_status st = ensure_ws(ctx, segment_ws_bytes(tiles, n, P, learned, ctx), s);
     if (st != RT_OK) return st;
 
     for (int c0 = 0; c0 < n; c0 += kMaxImgs) {
