@@ -535,6 +535,16 @@ bool bad_tile(const rt_tile &t)
     return false;
 }
 
+// Whether an output of the chain lies over its image.
+bool in_place(const rt_tile &t)
+{
+    const size_t n = span(t.H, t.ld_img, 1, t.W);
+    return (t.recon && overlaps(t.img, n, t.recon, span(t.H, t.ld_recon, 1, t.W))) ||
+           (t.filled && overlaps(t.img, n, t.filled, span(t.H, t.ld_filled, 1, t.W))) ||
+           overlaps(t.img, n, t.labels, span(t.H, t.ld_labels, 4, t.W)) ||
+           overlaps(t.img, n, t.d2, span(t.H, t.ld_d2, 4, t.W));
+}
+
 // Starts an EDT batch: takes its control words with the status word before
 // them (`words` in all, to be cleared), for images of `bands` bands of rows.
 int32_t *take_edt_ctl(Carve &cv, EdtBitsBatch &b, size_t bands, int &words)
@@ -1381,7 +1391,9 @@ rt_status rt_segment_batch(rt_ctx *ctx, const rt_tile *tiles, int n, const rt_se
             // call's start and joined at its end (by events, so a capture of
             // the call captures both).
             const bool pick = picks_matter(ctx, P, cn);
+            // Not where the chain writes over the image that the picker reads.
             aside = pick && c.contract;
+            for (int i = 0; i < cn; ++i) aside = aside && !in_place(tiles[c0 + i]);
             if (aside) {
                 RT_CUDA_TRY(cudaEventRecord(ctx->fork, s));
             } else if (pick) {
