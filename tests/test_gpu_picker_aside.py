@@ -60,3 +60,53 @@ def test_output_over_the_image(rt, name, dark):
         for k in want[0]:
             assert torch.equal(want[0][k], outs[0][k]), k
     ctx.close()
+
+
+@pytest.mark.parametrize("want_recon", [False, True])
+def test_captured_call_captures_both_streams(rt, want_recon):
+    """Two inputs through one graph: picks and outputs of the eager calls."""
+    ctx = rt.Context()
+    pk = dark_picker(rt, ctx)
+    p = rt.SegParams(policy=1)
+    imgs = [tile(rt, False), tile(rt, True)]
+    want = [rt.segment_batch([i], p, ctx=ctx, want_recon=want_recon)[0] for i in imgs]
+    img = imgs[0].clone()
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        outs = rt.segment_batch([img], p, ctx=ctx, want_recon=want_recon)
+    s.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        rt.segment_batch([img], p, outputs=outs, ctx=ctx)
+    for k in (1, 0, 1):
+        img.copy_(imgs[k])
+        for o in outs[0].values():
+            o.fill_(77)
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert rt.last_picks(ctx) == [k]
+        for name, t in want[k].items():
+            assert torch.equal(t, outs[0][name]), name
+    ctx.close()
+
+
+@pytest.mark.parametrize("want_recon", [False, True])
+def test_last_tile_of_33_is_a_chunk_of_its_own(rt, want_recon):
+    """32 tiles run the plain schedule; the 33rd forks, in the same
+    workspace. Plain calls of one tile each give the same outputs."""
+    shapes = [(150 + 17 * (i % 7), 130 + 29 * (i % 5)) for i in range(32)] + [(1500, 1300)]
+    for dark in (False, True):
+        imgs = [rt.config2_tile(100 + i, H=H, W=W) for i, (H, W) in enumerate(shapes[:32])] + [tile(rt, dark)]
+        ctx = rt.Context()
+        pk = dark_picker(rt, ctx)
+        for _ in range(2):
+            outs = rt.segment_batch(imgs, rt.SegParams(policy=1), ctx=ctx, want_recon=want_recon)
+            assert rt.last_picks(ctx) == [1 if dark else 0]
+        for i, o in zip(imgs, outs):
+            w = rt.segment_batch([i], want_recon=want_recon)[0]
+            torch.cuda.synchronize()
+            for name, t in w.items():
+                assert torch.equal(t, o[name]), name
+        ctx.close()
