@@ -349,6 +349,7 @@ constexpr int kBwA2 = kBwB1 + kMlpH * kMlpH * 2;    // 128 x 128: [dh2 | dh1]^T
 constexpr int kBwB2 = kBwA2 + kTcM * kTcM * 2;      // 96 x 128: [h1 | xn | 1]^T
 constexpr int kBwSmem = kBwB2 + kBwN2 * kTcM * 2;   // 73728 bytes (dynamic)
 constexpr int kBwPart = kW3;                        // partial sums per CTA: W1 b1 W2 b2
+constexpr int kBwEarly = 4;                         // CTAs up to which the second kernel is placed early
 
 // Column t (even and odd lanes side by side) of a K = 128 operand, rows
 // n .. n + 15: lanes exchange one value of each pair of rows, so every store
@@ -588,7 +589,15 @@ cudaError_t launch_mlp_backward_tc(const uint16_t *wb, const float *norm, const 
     if (e != cudaSuccess) return e;
     launch_early(kernel, nblk, kTcThreads, kBwSmem, s, wb, norm, x, act, logits, label, B, part, dz, lossb, err);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    launch_early(mlp_grad_tc_kernel, (unsigned)ceil_div((int64_t)(kMlpParams + 1) * 32, 256), 256, 0, s, part, nblk, dz, act, lossb, B, grad, loss);
+    // The sums live on their sectors staying in L1 (eight parameters share
+    // one). Blocks placed early sit beside the products' 72 KB of shared
+    // memory, which L1 is cut by, so they are only placed early for a batch
+    // of few CTAs: whole backward with and without, 16.1 and 16.6 us for 512
+    // samples, 19.7 and 18.7 for 1024, 40 and 33 for 4096, 253 and 107 for
+    // 20000.
+    const unsigned grid = (unsigned)ceil_div((int64_t)(kMlpParams + 1) * 32, 256);
+    if (nblk <= kBwEarly) launch_early(mlp_grad_tc_kernel, grid, 256, 0, s, part, nblk, dz, act, lossb, B, grad, loss);
+    else mlp_grad_tc_kernel<<<grid, 256, 0, s>>>(part, nblk, dz, act, lossb, B, grad, loss);
     return cudaGetLastError();
 }
 
