@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
                 const int r = side == 0 ? r0 - 1 : side == 1 ? r0 + kCtSide : r0 + si + k;
                 const int c = side == 2 ? c0 - 1 : side == 3 ? c0 + kCtSide : c0 + si + k;
                 if (r >= 0 && r < d.H && c >= 0 && c < d.W)
-                    halo = max(halo, (uint32_t)__ldg(d.mask + (int64_t)r * d.ld_mask + c) + 1u);
+                    halo = max(halo, (uint32_t)d.mask[(int64_t)r * d.ld_mask + c] + 1u);
             }
         }
     }
@@ -204,11 +204,11 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
             const uint32_t off = (uint32_t)(uintptr_t)p & 3u;
             if (n == 4 && (off == 0 || (c >= 4 && c + 8 <= d.W))) {   // the aligned words around them, in the row
                 const uint32_t *q = reinterpret_cast<const uint32_t *>(p - off);
-                v = __ldg(q);
-                if (off) v = __funnelshift_r(v, __ldg(q + 1), 8u * off);
+                v = q[0];
+                if (off) v = __funnelshift_r(v, q[1], 8u * off);
             } else {
 #pragma unroll 1
-                for (int k = 0; k < n; ++k) v |= (uint32_t)__ldg(p + k) << (8 * k);
+                for (int k = 0; k < n; ++k) v |= (uint32_t)p[k] << (8 * k);
             }
             const uint32_t idx = (uint32_t)(rr * kCtSide + 4 * (t & 15));
             uint32_t o[4];
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : 1) ct_local_kernel(const _
                 const int gr = r0 + r, gc = c0 + c;
                 uint32_t *sk = const_cast<uint32_t *>(nlink + k);
                 if (MARKER) {
-                    const uint32_t J = __ldg(d.marker + (int64_t)gr * d.ld_marker + gc);
+                    const uint32_t J = d.marker[(int64_t)gr * d.ld_marker + gc];
                     bad |= J > I;
                     const uint32_t s = kRootBit | min(J, I);
                     if (nlink[k] < s) atomicMax(sk, s);
@@ -827,7 +827,7 @@ __global__ void __launch_bounds__(kCtUnits * 32) ct_seam_kernel(const __grid_con
         const int t1 = down ? tile + d.nx : tile + 1;           // the tile across
         const int step = down ? 1 : d.nx;                       // to the next tile along the seam
         const int s0 = down ? 1 : 3, s1 = down ? 0 : 2;         // the sides that meet
-        auto rim = [&](int ut, int side, int at) { return (uint32_t)__ldg(b.rim + ((int64_t)ut * 4 + side) * kCtSide + at); };
+        auto rim = [&](int ut, int side, int at) { return (uint32_t)b.rim[((int64_t)ut * 4 + side) * kCtSide + at]; };
         const uint32_t none = kCtNoNode << 8;
         const uint32_t m0 = rim(tile, s0, i), m1 = rim(t1, s1, i);
         // the ends' neighbours along the seam may be the next tiles'

@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(NT) edt_near_kernel(const __grid_constant__ Ed
     const int nr = min(kEdtSide, d.H - r0), nc = min(kEdtSide, d.W - c0);
     const bool wide = nc == kEdtSide && (((uintptr_t)d.d2 | (uintptr_t)d.ld_d2 * 4u) & 15u) == 0;
     // own bits: thread = half a row
-    uint32_t own = t < 2 * kEdtSide ? __ldg(reinterpret_cast<const uint32_t *>(b.bits + (int64_t)tile * kEdtSide) + t) : 0u;
+    uint32_t own = t < 2 * kEdtSide ? reinterpret_cast<const uint32_t *>(b.bits + (int64_t)tile * kEdtSide)[t] : 0u;
     if (!__syncthreads_or(own != 0u)) {
         if (wide) {
             for (int i = t >> 4; i < nr; i += NT / 16)
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(NT) edt_near_kernel(const __grid_constant__ Ed
         uint32_t v = 0;
         if (r >= 0 && r < d.H && c >= 0 && c < d.W) {
             const int64_t nt = (int64_t)d.tile_base + (int64_t)(r / kEdtSide) * d.nx + c / kEdtSide;
-            v = ~__ldg(reinterpret_cast<const uint32_t *>(b.bits + nt * kEdtSide + r % kEdtSide) + (c / 32 & 1));
+            v = ~reinterpret_cast<const uint32_t *>(b.bits + nt * kEdtSide + r % kEdtSide)[c / 32 & 1];
             if (d.W - c < 32) v &= (1u << (d.W - c)) - 1u;
         }
         bg[y][w] = v;
