@@ -12,7 +12,8 @@ constexpr int kUfMaxRoots = kUfBlock * kUfBlock / 2;   // local components of a 
 constexpr int kUfMaxImgs = 32;
 // Images of at most this many 64 x 64 tiles are labeled here: its four short
 // launches beat the five of the union-find over runs, whose stages are bound
-// by their slowest tile (nuclei images, 180 nuclei per megapixel, label_area:
+// by their slowest tile (whole calls of rt_label_area, which pack bytes to
+// bits for the runs; nuclei images, 180 nuclei per megapixel:
 // 24 against 34 us at 700 x 700, 26 against 36 at 1024 x 1024, 35 against 41
 // at 2048 x 2048, equal at 2400 x 2400, 58 against 54 at 3000 x 3000, 94
 // against 63 at 4096 x 4096; with 380 nuclei the lines cross at 2048 x 2048,

@@ -26,7 +26,10 @@
 // value. A pixel that finds nothing nearer than 32 (or lies in a tile
 // that large objects fill) is written as 1024, no other distance of this stage, and flags its row, and edt_far_kernel (which
 // returns at once if no row is flagged) searches for those pixels as above,
-// with g from column masks of 32-row segments and never stored.
+// with g from column masks of 32-row segments and never stored. Such images
+// pay for both stages: discs of radius 300 take 95 -> 185 us at 1024 x 1024
+// and 1.36 -> 1.81 ms at 4096 x 4096 against the kernels above, nuclei 76 -> 36
+// at 4096 x 4096.
 #include "edt.cuh"
 
 namespace rtk {

@@ -21,12 +21,18 @@
 //     pixels summed over the slots of a tree. The output stage reads the
 //     tile's run words back and writes labels, the kept bits and the count.
 //
-// Measured on one GB300, 4096 x 4096 nuclei tiles: filling eight of them takes
-// 0.22 ms (0.28 as bit-plane floods swept to a fixed point), labeling 0.14 ms
-// (0.66 as a union-find over pixels); one tile alone 59 us against 129 and 43
-// against 99, a 1024 x 1024 one 45 against 64 and 26 against 36. The local
-// stages are bound by the latency of the tiles with the most runs, the label
-// stage by its stores (4 bytes a pixel).
+// Measured on one GB300 as stages of the chain, where the bits are there
+// already and the fill's last launch also makes the labels' local components,
+// nuclei tiles: the fill of eight 4096 x 4096 tiles takes 222 us (281 as
+// bit-plane floods swept to a fixed point), their labels 137 (661 as a
+// union-find over pixels); one tile 55 (109) and 40 (101); a 1024 x 1024 tile
+// 43 (79) and 25 (35). (rt_label_area, a call of its own, packs bytes to bits
+// first and makes its local components itself; with these two launches more
+// the pixels win on small images: kUfMaxTiles in ccl.cuh.) The local stages
+// are bound by the latency of the tiles with the most runs, the label stage by
+// its stores (4 bytes a pixel). Speckle, whose runs are about as many as its
+// pixels, is where floods were faster: rt_fill_holes on 4096 x 4096 pixels of
+// which 60 % are set at random 80 -> 284 us.
 #include "runs.cuh"
 
 namespace rtk {

@@ -53,8 +53,8 @@ cudaError_t launch_run_pack(const RunBatch &b, cudaStream_t s);
 // takes with again = true: the part of bits that its fill adds first
 cudaError_t launch_run_reach(const RunBatch &b, cudaStream_t s);
 // Holes filled in bits (and filled written); conn 4 or 8 is the background's
-// connectivity. With label_conn (4, 8; 0: none) the last launch also makes
-// the local components that launch_run_label needs.
+// connectivity. With label_conn 8 (0: none, another: cudaErrorInvalidValue)
+// the last launch also makes the local components that launch_run_label needs.
 cudaError_t launch_run_fill(const RunBatch &b, int conn, int label_conn, cudaStream_t s, bool again = false);
 // local components of bits, where launch_run_fill has not made them
 cudaError_t launch_run_local(const RunBatch &b, int conn, cudaStream_t s);
